@@ -415,91 +415,6 @@ __global__ void __launch_bounds__(256) k_apply_rows(T* logits, int64_t stride, M
     }
 }
 
-__device__ __forceinline__ float bf16_to_float(uint16_t h) { return __uint_as_float((uint32_t)h << 16); }
-
-// Greedy choice among allowed tokens: one block per row, reads only the
-// 16-byte chunks that hold an allowed position.
-template <typename T>
-__global__ void __launch_bounds__(256) k_argmax_masked(const T* logits, int64_t stride, DevTables D,
-                                                       const int32_t* mid, int B, int V, int vec,
-                                                       int32_t* tokens) {
-    int b = blockIdx.x;
-    if (b >= B) return;
-    int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nwarp = blockDim.x >> 5;
-    const uint32_t* rowids = D.mrows + (size_t)mid[b] * D.nch;
-    const T* row = logits + (size_t)b * stride;
-    float best = 0.f;
-    int bi = -1;
-    auto consider = [&](float v, int i) {
-        if (v != v) return;   // NaN never wins
-        if (bi < 0 || v > best || (v == best && i < bi)) {
-            best = v;
-            bi = i;
-        }
-    };
-    constexpr int E = 16 / sizeof(T);
-    int cpr = (V + 1023) >> 10;
-    for (int j = warp; j < cpr; j += nwarp) {
-        int col0 = j << 10;
-        int wi = (col0 >> 5) + lane;
-        uint32_t word = wi < D.W ? __ldg(D.mchunks + (size_t)__ldg(rowids + j) * 32 + lane) : 0u;
-        if (__ballot_sync(FULL, word != 0) == 0) continue;
-        int ncols = V - col0;
-        if (vec && ncols >= 1024) {
-#pragma unroll
-            for (int k = 0; k < 1024 / E / 32; k++) {
-                int c = k * 32 + lane;
-                uint32_t bits = (__shfl_sync(FULL, word, (c * E) >> 5) >> ((c * E) & 31)) & ((1u << E) - 1u);
-                if (!bits) continue;
-                uint4 v = ld_nc_v4(row + col0 + c * E);
-                uint32_t w[4] = {v.x, v.y, v.z, v.w};
-#pragma unroll
-                for (int e = 0; e < E; e++) {
-                    if (!((bits >> e) & 1)) continue;
-                    float f;
-                    if (sizeof(T) == 2) f = bf16_to_float((uint16_t)((w[e >> 1] >> ((e & 1) * 16)) & 0xFFFF));
-                    else f = __uint_as_float(w[e]);
-                    consider(f, col0 + c * E + e);
-                }
-            }
-        } else {
-            for (int e = 0; e < 32; e++) {
-                int col = col0 + 32 * lane + e;
-                if (col >= V) break;
-                if ((word >> e) & 1) {
-                    float f = sizeof(T) == 2 ? bf16_to_float((uint16_t)row[col]) : __uint_as_float((uint32_t)row[col]);
-                    consider(f, col);
-                }
-            }
-        }
-    }
-    // warp then block reduction of (best, bi)
-    for (int off = 16; off; off >>= 1) {
-        float ov = __shfl_down_sync(FULL, best, off);
-        int oi = __shfl_down_sync(FULL, bi, off);
-        if (oi >= 0 && (bi < 0 || ov > best || (ov == best && oi < bi))) {
-            best = ov;
-            bi = oi;
-        }
-    }
-    __shared__ float sv[32];
-    __shared__ int si[32];
-    if (lane == 0) {
-        sv[warp] = best;
-        si[warp] = bi;
-    }
-    __syncthreads();
-    if (threadIdx.x == 0) {
-        for (int w = 1; w < nwarp; w++) {
-            if (si[w] >= 0 && (bi < 0 || sv[w] > best || (sv[w] == best && si[w] < bi))) {
-                best = sv[w];
-                bi = si[w];
-            }
-        }
-        tokens[b] = bi;
-    }
-}
-
 // Feed one lexeme class to the parser on a row's stack: resolve the class to a
 // terminal with the current top, reduce until it is shifted.  Returns a row
 // status; `low` becomes the lowest stack index written.
@@ -781,6 +696,214 @@ __device__ __forceinline__ unsigned long long best_piece_key_bf16(const BestPiec
     for (int e = 7; e >= 0; e--)
         if (((bp.bits >> e) & 1) && bf16_at(w[e >> 1], e & 1) == bp.val) at = e;
     return make_key(f32_order(__float_as_uint(bp.val)), bp.col + at);
+}
+
+// A row of logits seen from the 32-byte boundary at or below its first element: its
+// columns are the elements [a, end) counted from there, cut into 16-byte pieces and
+// 1024-element chunks.  Rows that are not aligned (a contiguous batch of an odd
+// vocabulary) then take the same vector loads and stores as aligned ones: only the
+// elements outside the whole pieces [lo, hi), fewer than one piece at either end, are
+// handled one by one.  A 32-byte sector is a pair of neighbouring pieces.
+template <typename T>
+struct RowView {
+    static constexpr int E = 16 / sizeof(T);         // elements per piece
+    static constexpr int PIECES = 1024 / E / 32;     // pieces of a chunk per lane
+    static constexpr uint32_t FULLBITS = (1u << E) - 1u;
+    T* org;
+    int a, lo, hi, end;
+    __device__ __forceinline__ RowView(T* row, int V) {
+        uintptr_t p = reinterpret_cast<uintptr_t>(row);
+        a = (int)(p & 31u) / (int)sizeof(T);
+        org = reinterpret_cast<T*>(p & ~(uintptr_t)31);
+        end = a + V;
+        lo = (a + E - 1) / E * E;
+        hi = end / E * E;
+        if (hi < lo) lo = hi = end;   // the row lies inside one piece
+    }
+    __device__ __forceinline__ int chunks() const { return (end + 1023) >> 10; }
+    // does chunk j hold elements outside the whole pieces?  (warp-uniform)
+    __device__ __forceinline__ bool edge(int j) const { return (j == 0 && a > 0) || (j + 1) * 1024 > hi; }
+    __device__ __forceinline__ bool whole(int x) const { return x >= lo && x < hi; }   // x: a piece's first element
+    // the element outside the whole pieces that `lane` handles in chunk j (lanes 0-7: before
+    // them, 8-15: after them), or -1
+    __device__ __forceinline__ int edge_element(int j, int lane) const {
+        int x = lane < 8 ? a + lane : hi + lane - 8;
+        bool in = lane < 8 ? x < lo : lane < 16 && x < end;
+        return in && (x >> 10) == j ? x : -1;
+    }
+};
+
+// Mask word of elements [1024 j + 32 lane, +32) of a row view from the mask words of its
+// columns: cur = word 32 j + lane, before = word 32 j - 1 (needed by lane 0).
+__device__ __forceinline__ uint32_t view_word(uint32_t cur, uint32_t before, int a, int lane) {
+    if (a == 0) return cur;   // warp-uniform
+    uint32_t p = __shfl_up_sync(FULL, cur, 1);
+    return __funnelshift_l(lane == 0 ? before : p, cur, a);
+}
+
+// Mask bits of piece k of this lane, from the chunk's view words.
+template <typename T>
+__device__ __forceinline__ uint32_t piece_bits(uint32_t word, int k, int lane) {
+    constexpr int E = RowView<T>::E, PPW = 32 / E;   // pieces per mask word
+    return (__shfl_sync(FULL, word, k * (32 / PPW) + lane / PPW) >> ((lane % PPW) * E)) & RowView<T>::FULLBITS;
+}
+
+template <typename T>
+__device__ __forceinline__ float value_of(T v) {
+    return sizeof(T) == 2 ? __uint_as_float((uint32_t)v << 16) : __uint_as_float((uint32_t)v);
+}
+
+// Folds a piece (bits: its allowed elements; x: its values, -inf where not allowed; col:
+// its first column) into the lane's best; the piece with the larger maximum wins, the
+// earlier one on a tie.  A piece whose allowed values are all -inf or NaN, met before any
+// other allowed value, takes a short scalar path (an allowed -inf is a valid choice).
+template <typename T>
+__device__ __forceinline__ void fold_piece(BestPiece& bp, uint32_t bits, const uint4& x, int col) {
+    float mf;
+    if (sizeof(T) == 2) {
+        uint32_t w[4] = {x.x, x.y, x.z, x.w};
+        __nv_bfloat162* h = reinterpret_cast<__nv_bfloat162*>(w);
+        __nv_bfloat162 m = __hmax2(__hmax2(h[0], h[1]), __hmax2(h[2], h[3]));
+        mf = fmaxf(__low2float(m), __high2float(m));
+    } else {
+        mf = fmaxf(fmaxf(__uint_as_float(x.x), __uint_as_float(x.y)), fmaxf(__uint_as_float(x.z), __uint_as_float(x.w)));
+    }
+    bool upd = mf > bp.val;
+    if (!upd && bits != 0u && bp.col < 0) {
+        uint32_t w[4] = {x.x, x.y, x.z, x.w};
+#pragma unroll
+        for (int e = 0; e < RowView<T>::E; e++) {
+            float f = sizeof(T) == 2 ? bf16_at(w[e >> 1], e & 1) : __uint_as_float(w[e & 3]);
+            if (((bits >> e) & 1) && f == -INFINITY) upd = true;
+        }
+    }
+    bp.val = upd ? mf : bp.val;
+    bp.col = upd ? col : bp.col;
+    bp.bits = upd ? bits : bp.bits;
+    bp.x.x = upd ? x.x : bp.x.x;
+    bp.x.y = upd ? x.y : bp.x.y;
+    bp.x.z = upd ? x.z : bp.x.z;
+    bp.x.w = upd ? x.w : bp.x.w;
+}
+
+// Key of the piece's first allowed value equal to the best.
+template <typename T>
+__device__ __forceinline__ unsigned long long best_piece_key(const BestPiece& bp) {
+    if (bp.col < 0) return 0ull;
+    uint32_t w[4] = {bp.x.x, bp.x.y, bp.x.z, bp.x.w};
+    int at = 0;
+#pragma unroll
+    for (int e = RowView<T>::E - 1; e >= 0; e--) {
+        float f = sizeof(T) == 2 ? bf16_at(w[e >> 1], e & 1) : __uint_as_float(w[e & 3]);
+        if (((bp.bits >> e) & 1) && f == bp.val) at = e;
+    }
+    return make_key(f32_order(__float_as_uint(bp.val)), bp.col + at);
+}
+
+// Allowed-position masks of a 16-byte piece: the shared-memory table of bf16 pieces, or
+// (f32) one comparison per element.
+template <typename T>
+__device__ __forceinline__ uint4 mask_piece(const uint4& v, uint32_t bits, const uint4* lut) {
+    constexpr uint32_t N = NegInf<T>::pair;
+    if (sizeof(T) == 2) {
+        uint4 am = lut[bits];
+        return make_uint4(sel_ninf(v.x, am.x, N), sel_ninf(v.y, am.y, N), sel_ninf(v.z, am.z, N), sel_ninf(v.w, am.w, N));
+    }
+    return make_uint4(bits & 1u ? v.x : N, bits & 2u ? v.y : N, bits & 4u ? v.z : N, bits & 8u ? v.w : N);
+}
+
+// The larger of the warp's 64-bit keys (the high words, then the low words of the lanes holding it).
+__device__ __forceinline__ unsigned long long warp_max_key(unsigned long long key) {
+    uint32_t khi = (uint32_t)(key >> 32), klo = (uint32_t)key;
+    uint32_t mhi = __reduce_max_sync(FULL, khi);
+    uint32_t mlo = __reduce_max_sync(FULL, khi == mhi ? klo : 0u);
+    return ((unsigned long long)mhi << 32) | mlo;
+}
+
+// Greedy choice among allowed tokens without masking (psc_argmax_masked): a cluster of
+// CTAs per row, a warp per 1024-element chunk, reading only the 16-byte pieces that hold
+// an allowed position; the warps' keys meet in the shared memory of the cluster's first
+// CTA (distributed shared memory), so the call needs no scratch.  Bound: reading the
+// allowed pieces; with few rows the number of loads in flight, hence up to CHOOSE_CLUSTER
+// CTAs per row.  64 rows x 262,144 bf16 tokens: two steps of masking, choice and advance
+// called apart take 71 us; with one 256-thread CTA per row the choice alone took 133 us of
+// each step (279 us in all; 12 % of the warps active).
+constexpr int CHOOSE_CLUSTER = 8;
+template <typename T>
+__global__ void __launch_bounds__(256) k_choose(const T* logits, int64_t stride, DevTables D, const int32_t* mid, int V,
+                                                int csize, int32_t* tokens) {
+    __shared__ uint4 s_lut[sizeof(T) == 2 ? 256 : 1];
+    __shared__ unsigned long long s_key[CHOOSE_CLUSTER * 8];
+    if (sizeof(T) == 2) build_allow_lut<T>(s_lut);
+    __syncthreads();
+    const int b = blockIdx.x / csize, rank = blockIdx.x - b * csize;
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const uint32_t* rowids = D.mrows + (size_t)mid[b] * D.nch;
+    const RowView<T> R(const_cast<T*>(logits) + (size_t)b * stride, V);
+    BestPiece bp = best_piece_none();
+    Best best{0.f, -1};
+    const int n = R.chunks(), step = csize * 8;
+    // mask word `lane` of chunk j (and the word before the chunk, for lane 0)
+    auto words = [&](int j, uint32_t& cur, uint32_t& before) {
+        cur = before = 0u;
+        if (j < D.nch && j < n) cur = __ldg(D.mchunks + (size_t)__ldg(rowids + j) * 32 + lane);
+        if (R.a && lane == 0 && j > 0 && j < n) before = __ldg(D.mchunks + (size_t)__ldg(rowids + j - 1) * 32 + 31);
+    };
+    uint32_t cur, before;
+    int j = rank * 8 + warp;
+    words(j, cur, before);
+    for (; j < n; j += step) {
+        uint32_t w = view_word(cur, before, R.a, lane);
+        words(j + step, cur, before);   // in flight while this chunk is read
+        if (__ballot_sync(FULL, w != 0u) == 0u) continue;
+        uint32_t bits[RowView<T>::PIECES];
+#pragma unroll
+        for (int k = 0; k < RowView<T>::PIECES; k++) bits[k] = piece_bits<T>(w, k, lane);
+        const int x0 = (j << 10) + lane * RowView<T>::E;
+        if (R.edge(j)) {
+#pragma unroll
+            for (int k = 0; k < RowView<T>::PIECES; k++)
+                if (!R.whole(x0 + k * 32 * RowView<T>::E)) bits[k] = 0u;
+            int x = R.edge_element(j, lane);
+            uint32_t ew = __shfl_sync(FULL, w, (x >> 5) & 31);
+            if (x >= 0 && ((ew >> (x & 31)) & 1u)) {
+                float f = value_of(R.org[x]);
+                if (!isnan(f)) note_best(best, f, x - R.a);
+            }
+        }
+#pragma unroll
+        for (int h = 0; h < RowView<T>::PIECES; h += 4) {   // four pieces in flight
+            uint4 v[4];
+#pragma unroll
+            for (int k = 0; k < 4; k++)
+                v[k] = bits[h + k] ? ld_nc_v4(R.org + x0 + (h + k) * 32 * RowView<T>::E) : make_uint4(0u, 0u, 0u, 0u);
+#pragma unroll
+            for (int k = 0; k < 4; k++)
+                if (bits[h + k])
+                    fold_piece<T>(bp, bits[h + k], mask_piece<T>(v[k], bits[h + k], s_lut),
+                                  x0 + (h + k) * 32 * RowView<T>::E - R.a);
+        }
+    }
+    unsigned long long key = best_key_of(best), kp = best_piece_key<T>(bp);
+    key = warp_max_key(kp > key ? kp : key);
+    uint32_t dst = static_cast<uint32_t>(__cvta_generic_to_shared(&s_key[rank * 8 + warp]));
+    if (csize > 1) {
+        // every CTA of the cluster has started before its shared memory is written to
+        asm volatile("barrier.cluster.arrive.release.aligned;\nbarrier.cluster.wait.acquire.aligned;" ::: "memory");
+        uint32_t remote;
+        asm volatile("mapa.shared::cluster.u32 %0, %1, 0;" : "=r"(remote) : "r"(dst));
+        if (lane == 0) asm volatile("st.shared::cluster.u64 [%0], %1;" ::"r"(remote), "l"(key) : "memory");
+        asm volatile("barrier.cluster.arrive.release.aligned;\nbarrier.cluster.wait.acquire.aligned;" ::: "memory");
+    } else {
+        if (lane == 0) s_key[warp] = key;
+        __syncthreads();
+    }
+    if (rank == 0 && warp == 0) {
+        unsigned long long k = 0ull;
+        for (int i = lane; i < step; i += 32) k = s_key[i] > k ? s_key[i] : k;
+        k = warp_max_key(k);
+        if (lane == 0) tokens[b] = k ? (int32_t)(~(uint32_t)k) : -1;
+    }
 }
 
 // A lane's four 16-byte pieces of a bf16 chunk in registers: the mask bits of
@@ -2078,6 +2201,27 @@ psc_status launch_pdl(void (*kernel)(KArgs...), dim3 grid, dim3 block, size_t sm
     return cuda_check(cudaLaunchKernelEx(&cfg, kernel, static_cast<KArgs>(args)...), what);
 }
 
+// psc_argmax_masked: a cluster of up to CHOOSE_CLUSTER 256-thread CTAs per row, as many
+// as it takes for the batch to fill the SMs (about four CTAs on each) and no more than
+// one warp per chunk of the row.
+template <typename T>
+psc_status launch_choose(const T* logits, int64_t stride, const psc_handle* h, const int32_t* mid, int B, int V,
+                         int32_t* d_tokens, cudaStream_t cs) {
+    int chunks = (V + 32 + 1023) / 1024;
+    int csize = 1;
+    while (csize < CHOOSE_CLUSTER && (long)B * csize < 4L * sm_count(h->device) && csize * 8 < chunks) csize *= 2;
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3((unsigned)(B * csize));
+    cfg.blockDim = dim3(256);
+    cfg.stream = cs;
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeClusterDimension;
+    attr[0].val.clusterDim = {(unsigned)csize, 1u, 1u};
+    cfg.attrs = attr;
+    cfg.numAttrs = 1;
+    return cuda_check(cudaLaunchKernelEx(&cfg, k_choose<T>, logits, stride, h->d, mid, V, csize, d_tokens), "k_choose");
+}
+
 // Algorithm 2 steps 1-2 for every row (the token given, or the fused pass's greedy
 // choice when d_tokens_out is set), then step 3 for the new configurations: the
 // rows' mask ids are current afterwards.
@@ -2881,15 +3025,9 @@ psc_status psc_argmax_masked(const psc_handle* h, const psc_states* st, int32_t 
         return fail_with(PSC_ERR_ARG, "psc_argmax_masked: bad arguments");
     cudaStream_t cs = (cudaStream_t)stream;
     if ((s = ensure_mid(h, st, cs)) != PSC_OK) return s;
-    size_t esz = dtype == PSC_BF16 ? 2 : 4;
-    int vec = aligned16(d_logits) && ((row_stride * (int64_t)esz) % 16 == 0);
     if (dtype == PSC_BF16)
-        k_argmax_masked<uint16_t><<<B, 256, 0, cs>>>((const uint16_t*)d_logits, row_stride, h->d, st->d.mid, B, V, vec,
-                                                     d_tokens);
-    else
-        k_argmax_masked<uint32_t><<<B, 256, 0, cs>>>((const uint32_t*)d_logits, row_stride, h->d, st->d.mid, B, V, vec,
-                                                     d_tokens);
-    return launch_check("k_argmax_masked");
+        return launch_choose((const uint16_t*)d_logits, row_stride, h, st->d.mid, B, V, d_tokens, cs);
+    return launch_choose((const uint32_t*)d_logits, row_stride, h, st->d.mid, B, V, d_tokens, cs);
 }
 
 psc_status psc_fill_apply_argmax(const psc_handle* h, const psc_states* st, int32_t B, void* d_logits,

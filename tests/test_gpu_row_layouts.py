@@ -1,0 +1,137 @@
+"""GPU: every masking and choosing call on rows of any layout: vocabularies around the
+edges of words, chunks and pieces, rows that start at any element, logit types, values.
+
+The masks come from the oracle; masked logits and greedy tokens are compared bit for
+bit with numpy, and everything outside the rows must keep its bytes.
+"""
+from __future__ import annotations
+
+import numpy as np
+import pytest
+
+from oracle import Oracle, Vocab
+from workloads import grammars
+
+torch = pytest.importorskip("torch")
+pytestmark = pytest.mark.gpu
+
+B = 6
+VOCABS = (2, 7, 33, 512, 1017, 1024, 1025, 2055, 9001)
+SENTINEL = 77.0
+
+
+@pytest.fixture(scope="module")
+def psc():
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    from paper_2608_03065_gb300 import build, psc as mod
+    build.build()
+    mod.load()
+    return mod
+
+
+def _vocabulary(V):
+    """V - 1 token strings (all the punctuation, then random JSON-like text) and the end token."""
+    rng = np.random.default_rng(V)
+    chars = b'[]{},:"0123456789truefalsn -.e\\ab'
+    toks = dict.fromkeys(bytes([c]) for c in b'["1,]{:}truefalsn -.e0ab')
+    while len(toks) < V:
+        toks[bytes(chars[i] for i in rng.integers(0, len(chars), rng.integers(1, 7)))] = None
+    return list(toks)[:V - 1] + [b""]
+
+
+@pytest.fixture(scope="module")
+def batches(psc):
+    """V -> (handle, states, allowed [B][V]): rows at the start, in an array, in a string, with a
+    pending number, done, and rejected."""
+    g = grammars.json_grammar().text()
+    o = Oracle(g)
+    out = {}
+    for V in VOCABS:
+        toks = _vocabulary(V)
+        h = psc.psc_compile(g, toks, V - 1)
+        voc = Vocab.from_list(toks, V - 1)
+        seqs = [[], ["["], ["[", '"'], ["1"], ["1", None], ["]"]]
+        ids = [[V - 1 if t is None else toks.index(t.encode()) if t.encode() in toks else -1 for t in s] for s in seqs]
+        st = psc.psc_state_init(h, B, 16)
+        for j in range(2):
+            col = [r[j] if j < len(r) else -1 for r in ids]
+            psc.psc_advance(h, st, torch.tensor(col, dtype=torch.int32, device="cuda"))
+        ocs = []
+        for r in ids:
+            oc = o.initial()
+            o.advance_tokens(oc, voc, [t for t in r if t >= 0])
+            ocs.append(oc)
+        bits = np.unpackbits(o.masks(ocs, voc).view(np.uint8), axis=-1, bitorder="little")[:, :V].astype(bool)
+        out[V] = (h, st, bits)
+    return out
+
+
+def _raw(t):
+    t = t.cpu()
+    return t.view(torch.int16 if t.dtype == torch.bfloat16 else torch.int32).numpy()
+
+
+def _values(V, seed):
+    """Normal values with ties, both zeros, infinities and NaN payloads among them; a row that is
+    all NaN and one that is all -inf."""
+    rng = np.random.default_rng([V, seed])
+    x = np.round(rng.standard_normal((B, V)) * 4).astype(np.float32) / 4
+    special = np.array([0.0, -0.0, -np.inf, np.inf, np.nan], dtype=np.float32)
+    at = rng.random((B, V)) < 0.2
+    x[at] = rng.choice(special[:3 if seed % 2 else 5], at.sum())
+    if seed % 3 == 1:
+        x[1] = np.nan
+        x[2] = -np.inf
+    return x
+
+
+def _greedy(x, allowed):
+    out = np.full(B, -1, dtype=np.int64)
+    for b in range(B):
+        idx = np.nonzero(allowed[b] & ~np.isnan(x[b]))[0]
+        if len(idx):
+            out[b] = idx[np.argmax(x[b, idx])]
+    return out
+
+
+@pytest.mark.parametrize("dtype", [torch.bfloat16, torch.float32])
+@pytest.mark.parametrize("V", VOCABS)
+def test_rows_of_any_layout(psc, batches, V, dtype):
+    h, st, allowed = batches[V]
+    ninf = np.int16(-128) if dtype == torch.bfloat16 else np.int32(-8388608)
+    # (first element, row stride): contiguous, padded, odd offsets and strides
+    for seed, (off, ld) in enumerate([(0, V), (0, V + 1), (0, -(-V // 64) * 64), (8, V + 8), (1, V + 3), (5, V + 16),
+                                      (3, V)]):
+        x = torch.from_numpy(_values(V, seed)).to(dtype)
+        base = torch.full((off + B * ld + 64,), SENTINEL, dtype=dtype)
+        base.as_strided((B, V), (ld, 1), off).copy_(x)
+        want = base.clone()
+        view = _raw(want)
+        rows = np.lib.stride_tricks.as_strided(view[off:], (B, V), (ld * view.itemsize, view.itemsize))
+        rows[~allowed] = ninf
+        greedy = _greedy(x.float().numpy(), allowed)
+        bm = torch.zeros(B, h.W, dtype=torch.int32, device="cuda")
+        psc.psc_fill_mask(h, st, bm)
+        forked = psc.psc_state_init(h, B, 16)
+        psc.psc_state_copy(forked, st)
+        for call in ("fill_apply", "apply_mask", "fill_apply_argmax", "decode_step"):
+            dev = base.cuda()
+            lg = dev.as_strided((B, V), (ld, 1), off)
+            tok = torch.full((B,), -7, dtype=torch.int32, device="cuda")
+            out = torch.full((B, h.W), -1, dtype=torch.int32, device="cuda")
+            if call == "fill_apply":
+                psc.psc_argmax_masked(h, st, lg, tok)          # before masking: only allowed values count
+                np.testing.assert_array_equal(tok.cpu().numpy(), greedy, err_msg=f"{call} {off} {ld}")
+                psc.psc_fill_apply(h, st, lg, out)
+                psc.psc_argmax_masked(h, st, lg, tok)
+            elif call == "apply_mask":
+                psc.psc_apply_mask(lg, bm, B, V)
+            elif call == "fill_apply_argmax":
+                psc.psc_fill_apply_argmax(h, st, lg, tok, out)
+            else:
+                psc.psc_decode_step(h, forked, lg, tok, out)
+            np.testing.assert_array_equal(_raw(dev), _raw(want), err_msg=f"{call} {off} {ld}")
+            if call != "apply_mask":
+                np.testing.assert_array_equal(tok.cpu().numpy(), greedy, err_msg=f"{call} {off} {ld}")
+                np.testing.assert_array_equal(out.cpu().numpy(), bm.cpu().numpy(), err_msg=f"{call} {off} {ld}")
