@@ -7,7 +7,7 @@
 //              stopping at absorbing states; kept incremental by the bottom-up
 //              classifier (its state per stack prefix, so a step re-reads only
 //              the entries it changed, then one lookup by q)    -> k_advance_warp / k_classify
-//   step 4     the precomputed mask of the reached state         -> k_step_tma / k_fill / k_apply_rows
+//   step 4     the precomputed mask of the reached state         -> k_step_warp / k_fill / k_apply_rows
 // plus applying the mask to the logits and greedy sampling over the allowed
 // tokens (left to the serving engine in the paper).
 //
@@ -33,6 +33,7 @@
 #include <mutex>
 #include <new>
 #include <string>
+#include <type_traits>
 
 #include "../../include/psc.h"
 #include "psc_internal.h"
@@ -111,7 +112,6 @@ struct psc_handle {
     DevTables d{};
     void* blocks[32] = {};
     int n_blocks = 0;
-    int tma_ctas[2] = {1, 1};   // resident k_step_tma CTAs per SM (bf16, f32)
     int tables = 0;             // psc_options.global_tables the handle was made with
     int mid0 = 0;               // mask id of the empty prefix
 };
@@ -122,8 +122,8 @@ struct psc_states {
     int device = -1;
     uint64_t gen = 1;        // bumped by every call that changes the rows
     uint64_t mid_gen = 0;    // generation the mask ids in d.mid were computed for
-    bool after_mask = false; // the last work enqueued on these states is the TMA masking pass with
-                             // the mask ids as they were (the advance may read the rows early)
+    bool after_mask = false; // the last work enqueued on these states is the masking pass with the
+                             // mask ids as they were (the advance may read the rows early)
 };
 
 namespace {
@@ -193,21 +193,6 @@ __device__ __forceinline__ int sparse_step_warp(const int32_t* rows, int s, int 
     return def;
 }
 
-// The same transition by one thread (binary search over the row's exceptions).
-__device__ __forceinline__ int sparse_step_thread(const int32_t* rows, int s, int X) {
-    const int2* r2 = reinterpret_cast<const int2*>(rows + s);
-    int2 h = __ldg(r2);
-    int lo = 0, hi = h.x;
-    while (lo < hi) {
-        int m = (lo + hi) >> 1;
-        int2 p = __ldg(r2 + 2 + m);
-        if (p.x == X) return p.y;
-        if (p.x < X) lo = m + 1;
-        else hi = m;
-    }
-    return h.y;
-}
-
 // Mask id of the classifier state s when the stack ends there (either layout).
 __device__ __forceinline__ int state_mask(const DevTables& T, int s) {
     return T.dfa_sparse ? __ldg(T.dfa_rows + s + 2) : __ldg(T.dfa_mask + s);
@@ -242,29 +227,6 @@ __device__ int warp_classify(const DevTables& T, const DevStates& S, int b, int 
             if (nx < 0) return -nx - 1;
             s = nx;
         }
-    }
-    return state_mask(T, s);
-}
-
-// the same classification by one thread (same guard on stack symbols)
-__device__ int thread_classify(const DevTables& T, const DevStates& S, int b) {
-    int status = S.status[b];
-    if (status == ROW_DONE) return 1;
-    if (status != ROW_OK) return 0;
-    int q = S.q[b];
-    int depth = S.depth[b];
-    if (q < 0 || q >= T.nq || depth < 1 || depth > S.cap) return 0;
-    int m = memo_classify(T, S, b, q, depth);
-    if (m >= 0) return m;
-    int s = __ldg(T.dfa_start + q);
-    if (s < 0) return -s - 1;
-    const uint16_t* st = S.stack + (size_t)b * S.cap;
-    for (int i = depth - 1; i >= 0; i--) {
-        int X = st[i];
-        if (X >= T.n_lr) return 0;
-        int nx = T.dfa_sparse ? sparse_step_thread(T.dfa_rows, s, X) : __ldg(T.dfa + (size_t)s * T.n_lr + X);
-        if (nx < 0) return -nx - 1;
-        s = nx;
     }
     return state_mask(T, s);
 }
@@ -405,6 +367,24 @@ struct MaskSrc {
         uint32_t c = __ldg(rows + (size_t)__ldg(mid + b) * nch + j);
         return __ldg(chunks + (size_t)c * 32 + lane);
     }
+    // word `lane` of chunks j .. j + SPAN - 1 of row b (0 past W) and, when BEFORE, the word
+    // before them (0 at the row's start), all through the device mask table and without
+    // branches, so that the SPAN + 1 chains of dependent loads run side by side
+    template <int SPAN, bool BEFORE>
+    __device__ __forceinline__ void table_words(int b, int j, int lane, uint32_t (&cur)[SPAN], uint32_t& before) const {
+        const uint32_t* r = rows + (size_t)__ldcg(mid + b) * nch;
+        uint32_t id[SPAN], idb = 0u;
+#pragma unroll
+        for (int i = 0; i < SPAN; i++) id[i] = __ldg(r + min(j + i, nch - 1));
+        if (BEFORE) idb = __ldg(r + min(max(j - 1, 0), nch - 1));
+#pragma unroll
+        for (int i = 0; i < SPAN; i++) cur[i] = __ldg(chunks + (size_t)id[i] * 32 + lane);
+        before = BEFORE ? __ldg(chunks + (size_t)idb * 32 + 31) : 0u;
+#pragma unroll
+        for (int i = 0; i < SPAN; i++)
+            if (j + i >= nch) cur[i] = 0u;
+        if (j == 0) before = 0u;
+    }
 };
 
 template <typename T>
@@ -480,8 +460,8 @@ __device__ int memo_extend(const DevTables& T, const uint16_t* st, int32_t* memo
 }
 
 // Algorithm 2 steps 1-2 for one row per thread.
-__global__ void k_advance(DevTables T, DevStates S, const int32_t* tokens, int B, int use_mid,
-                          int32_t* status_out, int from_keys, int32_t* tokens_out) {
+__global__ void k_advance(DevTables T, DevStates S, const int32_t* tokens, int B, int32_t* status_out,
+                          int from_keys, int32_t* tokens_out) {
     int b = blockIdx.x * blockDim.x + threadIdx.x;
     if (b >= B) return;
     int tok;
@@ -501,8 +481,7 @@ __global__ void k_advance(DevTables T, DevStates S, const int32_t* tokens, int B
             if (tok >= T.V) {
                 status = ROW_REJECTED;
             } else {
-                int mid = use_mid ? S.mid[b] : thread_classify(T, S, b);
-                bool allowed = (mask_word(T, mid, tok >> 5) >> (tok & 31)) & 1;
+                bool allowed = (mask_word(T, S.mid[b], tok >> 5) >> (tok & 31)) & 1;
                 if (!allowed) {
                     status = ROW_REJECTED;
                 } else if (tok == T.eos_id) {
@@ -554,15 +533,15 @@ __device__ __forceinline__ unsigned long long make_key(uint32_t ordered, int col
     return ((unsigned long long)ordered << 32) | (uint32_t)(~(uint32_t)col);
 }
 
-// Greedy state of one lane: the largest allowed value seen so far and the
-// lowest column holding it (col < 0: nothing yet).  NaN never becomes best.
+// Greedy state of one lane: the largest allowed value seen so far and the lowest column
+// holding it (col < 0: nothing yet; val is then -inf).  NaN never becomes best.
 struct Best {
-    float val;
-    int col;
+    float val = -INFINITY;
+    int col = -1;
 };
 
 __device__ __forceinline__ void note_best(Best& best, float v, int col) {
-    if (best.col < 0 || v > best.val || (v == best.val && col < best.col)) {
+    if (v > best.val || (v == best.val && (best.col < 0 || col < best.col))) {
         best.val = v;
         best.col = col;
     }
@@ -594,139 +573,25 @@ __device__ __forceinline__ uint32_t sel_ninf(uint32_t w, uint32_t allow, uint32_
     return (w & allow) | (ninf & ~allow);
 }
 
-__device__ __forceinline__ float bf16_at(uint32_t w, int half) {
-    return __uint_as_float(half ? (w & 0xFFFF0000u) : (w << 16));
-}
-
-// One 1024-column chunk of bf16: write -inf where masked (no read when the
-// whole 16-byte piece is masked), read the pieces that hold an allowed
-// position and fold their allowed values into the lane's best with packed
-// bf16x2 maxima; the column is searched only when the piece can win.
-__device__ __forceinline__ void apply_argmax_chunk_bf16(const uint16_t* src, uint16_t* row, int col0, uint32_t word, int lane,
-                                                        Best& best, const uint4* lut) {
-    const uint4 ninf = make_uint4(0xFF80FF80u, 0xFF80FF80u, 0xFF80FF80u, 0xFF80FF80u);
-    uint32_t bits[4];
-    uint4 v[4];
-#pragma unroll
-    for (int k = 0; k < 4; k++) bits[k] = (__shfl_sync(FULL, word, k * 8 + (lane >> 2)) >> ((lane & 3) * 8)) & 0xFFu;
-#pragma unroll
-    for (int k = 0; k < 4; k++)   // issue every needed load before any store
-        if (bits[k]) v[k] = *reinterpret_cast<const uint4*>(src + (k * 32 + lane) * 8);
-#pragma unroll
-    for (int k = 0; k < 4; k++) {
-        uint16_t* p = row + col0 + (k * 32 + lane) * 8;
-        uint32_t bk = bits[k];
-        if (bk == 0) {
-            st_cs_v4(p, ninf);
-            continue;
-        }
-        uint4 am = lut[bk];
-        uint32_t x0 = sel_ninf(v[k].x, am.x, 0xFF80FF80u), x1 = sel_ninf(v[k].y, am.y, 0xFF80FF80u);
-        uint32_t x2 = sel_ninf(v[k].z, am.z, 0xFF80FF80u), x3 = sel_ninf(v[k].w, am.w, 0xFF80FF80u);
-        __nv_bfloat162 m = __hmax2(__hmax2(*reinterpret_cast<__nv_bfloat162*>(&x0), *reinterpret_cast<__nv_bfloat162*>(&x1)),
-                                   __hmax2(*reinterpret_cast<__nv_bfloat162*>(&x2), *reinterpret_cast<__nv_bfloat162*>(&x3)));
-        float mf = fmaxf(__low2float(m), __high2float(m));
-        if (best.col < 0 || mf >= best.val) {   // rare: this piece may hold the lane's best
-            uint32_t w[4] = {v[k].x, v[k].y, v[k].z, v[k].w};
-#pragma unroll
-            for (int e = 0; e < 8; e++) {
-                float f = bf16_at(w[e >> 1], e & 1);
-                if (((bk >> e) & 1) && f == mf) {
-                    note_best(best, f, col0 + (k * 32 + lane) * 8 + e);
-                    break;
-                }
-            }
-        }
-        st_cs_v4(p, make_uint4(x0, x1, x2, x3));   // whole pieces: no partly written sectors
-    }
-}
-
-// One 1024-column chunk of f32 (4 elements per 16-byte piece), in two halves of
-// four pieces per lane (eight pieces and their bits at once exceed the register
-// budget of three resident CTAs).
-__device__ __forceinline__ void apply_argmax_chunk_f32(const uint32_t* src, uint32_t* row, int col0, uint32_t word, int lane,
-                                                       Best& best, const uint4* lut) {
-    const uint4 ninf = make_uint4(0xFF800000u, 0xFF800000u, 0xFF800000u, 0xFF800000u);
-#pragma unroll 1
-    for (int h = 0; h < 8; h += 4) {
-        uint32_t bits[4];
-        uint4 v[4];
-#pragma unroll
-        for (int k = 0; k < 4; k++)
-            bits[k] = (__shfl_sync(FULL, word, (h + k) * 4 + (lane >> 3)) >> ((lane & 7) * 4)) & 0xFu;
-#pragma unroll
-        for (int k = 0; k < 4; k++)
-            if (bits[k]) v[k] = *reinterpret_cast<const uint4*>(src + ((h + k) * 32 + lane) * 4);
-#pragma unroll
-        for (int k = 0; k < 4; k++) {
-            uint32_t* p = row + col0 + ((h + k) * 32 + lane) * 4;
-            uint32_t bk = bits[k];
-            if (bk == 0) {
-                st_cs_v4(p, ninf);
-                continue;
-            }
-            uint4 am = lut[bk];
-            uint32_t x0 = sel_ninf(v[k].x, am.x, 0xFF800000u), x1 = sel_ninf(v[k].y, am.y, 0xFF800000u);
-            uint32_t x2 = sel_ninf(v[k].z, am.z, 0xFF800000u), x3 = sel_ninf(v[k].w, am.w, 0xFF800000u);
-            float mf = fmaxf(fmaxf(__uint_as_float(x0), __uint_as_float(x1)), fmaxf(__uint_as_float(x2), __uint_as_float(x3)));
-            if (best.col < 0 || mf >= best.val) {
-                uint32_t w[4] = {v[k].x, v[k].y, v[k].z, v[k].w};
-#pragma unroll
-                for (int e = 0; e < 4; e++) {
-                    float f = __uint_as_float(w[e]);
-                    if (((bk >> e) & 1) && f == mf) {
-                        note_best(best, f, col0 + ((h + k) * 32 + lane) * 4 + e);
-                        break;
-                    }
-                }
-            }
-            st_cs_v4(p, make_uint4(x0, x1, x2, x3));
-        }
-    }
-}
-
-// Greedy state of a lane that streams bf16 chunks: the largest allowed value
-// seen so far and the 16-byte piece holding its first occurrence (the piece's
-// values and mask bits), resolved to a column once per work item.  The per-piece
-// update is a handful of selects, so no lane diverges while it streams.
-struct BestPiece {
-    float val;       // -inf until an allowed value is seen
-    int col;         // first column of the piece (-1: nothing yet)
-    uint32_t bits;   // the piece's mask bits
-    uint4 x;         // the piece's values
-};
-
-__device__ __forceinline__ BestPiece best_piece_none() {
-    return BestPiece{-INFINITY, -1, 0u, make_uint4(0u, 0u, 0u, 0u)};
-}
-
-// Column and key of the piece's first allowed value equal to the best.
-__device__ __forceinline__ unsigned long long best_piece_key_bf16(const BestPiece& bp) {
-    if (bp.col < 0) return 0ull;
-    uint32_t w[4] = {bp.x.x, bp.x.y, bp.x.z, bp.x.w};
-    int at = 0;
-#pragma unroll
-    for (int e = 7; e >= 0; e--)
-        if (((bp.bits >> e) & 1) && bf16_at(w[e >> 1], e & 1) == bp.val) at = e;
-    return make_key(f32_order(__float_as_uint(bp.val)), bp.col + at);
-}
-
 // A row of logits seen from the 32-byte boundary at or below its first element: its
 // columns are the elements [a, end) counted from there, cut into 16-byte pieces and
 // 1024-element chunks.  Rows that are not aligned (a contiguous batch of an odd
 // vocabulary) then take the same vector loads and stores as aligned ones: only the
 // elements outside the whole pieces [lo, hi), fewer than one piece at either end, are
 // handled one by one.  A 32-byte sector is a pair of neighbouring pieces.
-template <typename T>
+// ANY = false: every row starts on a 32-byte boundary and holds whole chunks (the tests
+// for the ends of a row then fold away).
+template <typename T, bool ANY = true>
 struct RowView {
-    static constexpr int E = 16 / sizeof(T);         // elements per piece
-    static constexpr int PIECES = 1024 / E / 32;     // pieces of a chunk per lane
-    static constexpr uint32_t FULLBITS = (1u << E) - 1u;
+    [[maybe_unused]] static constexpr int E = 16 / sizeof(T);         // elements per piece
+    [[maybe_unused]] static constexpr int PIECES = 1024 / E / 32;     // pieces of a chunk per lane
+    [[maybe_unused]] static constexpr uint32_t FULLBITS = (1u << E) - 1u;
     T* org;
     int a, lo, hi, end;
+    __device__ __forceinline__ RowView() {}
     __device__ __forceinline__ RowView(T* row, int V) {
         uintptr_t p = reinterpret_cast<uintptr_t>(row);
-        a = (int)(p & 31u) / (int)sizeof(T);
+        a = ANY ? (int)(p & 31u) / (int)sizeof(T) : 0;
         org = reinterpret_cast<T*>(p & ~(uintptr_t)31);
         end = a + V;
         lo = (a + E - 1) / E * E;
@@ -735,7 +600,7 @@ struct RowView {
     }
     __device__ __forceinline__ int chunks() const { return (end + 1023) >> 10; }
     // does chunk j hold elements outside the whole pieces?  (warp-uniform)
-    __device__ __forceinline__ bool edge(int j) const { return (j == 0 && a > 0) || (j + 1) * 1024 > hi; }
+    __device__ __forceinline__ bool edge(int j) const { return ANY && ((j == 0 && a > 0) || (j + 1) * 1024 > hi); }
     __device__ __forceinline__ bool whole(int x) const { return x >= lo && x < hi; }   // x: a piece's first element
     // the element outside the whole pieces that `lane` handles in chunk j (lanes 0-7: before
     // them, 8-15: after them), or -1
@@ -766,51 +631,67 @@ __device__ __forceinline__ float value_of(T v) {
     return sizeof(T) == 2 ? __uint_as_float((uint32_t)v << 16) : __uint_as_float((uint32_t)v);
 }
 
-// Folds a piece (bits: its allowed elements; x: its values, -inf where not allowed; col:
-// its first column) into the lane's best; the piece with the larger maximum wins, the
-// earlier one on a tie.  A piece whose allowed values are all -inf or NaN, met before any
-// other allowed value, takes a short scalar path (an allowed -inf is a valid choice).
+// Largest value of a piece (NaN only when all its values are).
 template <typename T>
-__device__ __forceinline__ void fold_piece(BestPiece& bp, uint32_t bits, const uint4& x, int col) {
-    float mf;
+__device__ __forceinline__ float piece_max(const uint4& x) {
     if (sizeof(T) == 2) {
         uint32_t w[4] = {x.x, x.y, x.z, x.w};
         __nv_bfloat162* h = reinterpret_cast<__nv_bfloat162*>(w);
         __nv_bfloat162 m = __hmax2(__hmax2(h[0], h[1]), __hmax2(h[2], h[3]));
-        mf = fmaxf(__low2float(m), __high2float(m));
-    } else {
-        mf = fmaxf(fmaxf(__uint_as_float(x.x), __uint_as_float(x.y)), fmaxf(__uint_as_float(x.z), __uint_as_float(x.w)));
+        return fmaxf(__low2float(m), __high2float(m));
     }
-    bool upd = mf > bp.val;
-    if (!upd && bits != 0u && bp.col < 0) {
-        uint32_t w[4] = {x.x, x.y, x.z, x.w};
-#pragma unroll
-        for (int e = 0; e < RowView<T>::E; e++) {
-            float f = sizeof(T) == 2 ? bf16_at(w[e >> 1], e & 1) : __uint_as_float(w[e & 3]);
-            if (((bits >> e) & 1) && f == -INFINITY) upd = true;
-        }
-    }
-    bp.val = upd ? mf : bp.val;
-    bp.col = upd ? col : bp.col;
-    bp.bits = upd ? bits : bp.bits;
-    bp.x.x = upd ? x.x : bp.x.x;
-    bp.x.y = upd ? x.y : bp.x.y;
-    bp.x.z = upd ? x.z : bp.x.z;
-    bp.x.w = upd ? x.w : bp.x.w;
+    return fmaxf(fmaxf(__uint_as_float(x.x), __uint_as_float(x.y)), fmaxf(__uint_as_float(x.z), __uint_as_float(x.w)));
 }
 
-// Key of the piece's first allowed value equal to the best.
+// The allowed elements of a piece (bits) that equal v, as bits.
 template <typename T>
-__device__ __forceinline__ unsigned long long best_piece_key(const BestPiece& bp) {
-    if (bp.col < 0) return 0ull;
-    uint32_t w[4] = {bp.x.x, bp.x.y, bp.x.z, bp.x.w};
-    int at = 0;
+__device__ __forceinline__ uint32_t piece_equal(const uint4& x, uint32_t bits, float v) {
+    uint32_t eq = 0u;
+    if (sizeof(T) == 2) {
+        const __nv_bfloat162 vv = __float2bfloat162_rn(v);   // v is one of the piece's values, or -inf
+        const uint32_t w[4] = {x.x, x.y, x.z, x.w};
 #pragma unroll
-    for (int e = RowView<T>::E - 1; e >= 0; e--) {
-        float f = sizeof(T) == 2 ? bf16_at(w[e >> 1], e & 1) : __uint_as_float(w[e & 3]);
-        if (((bp.bits >> e) & 1) && f == bp.val) at = e;
+        for (int k = 0; k < 4; k++)
+            eq |= __heq2_mask(*reinterpret_cast<const __nv_bfloat162*>(&w[k]), vv) & (0x00020001u << (2 * k));
+        eq |= eq >> 16;
+    } else {
+        eq = (__uint_as_float(x.x) == v ? 1u : 0u) | (__uint_as_float(x.y) == v ? 2u : 0u) |
+             (__uint_as_float(x.z) == v ? 4u : 0u) | (__uint_as_float(x.w) == v ? 8u : 0u);
     }
-    return make_key(f32_order(__float_as_uint(bp.val)), bp.col + at);
+    return eq & bits;
+}
+
+// Folds a lane's four pieces of a chunk (bits: their allowed elements; x: their values,
+// -inf where not allowed; col: the first piece's first column, the others 32 pieces apart)
+// into its best: a larger value wins, on a tie the earlier column does.
+template <typename T>
+__device__ __forceinline__ void fold_quad(Best& best, const uint32_t (&bits)[4], const uint4 (&x)[4], int col) {
+    constexpr int E = 16 / sizeof(T);
+    float m[4];
+#pragma unroll
+    for (int k = 0; k < 4; k++) m[k] = piece_max<T>(x[k]);
+    const float qm = fmaxf(fmaxf(m[0], m[1]), fmaxf(m[2], m[3]));
+    if (qm > best.val) {   // so an allowed value: the masked ones are -inf
+        uint4 p = x[3];
+        uint32_t pb = bits[3];
+        int k0 = 3;
+#pragma unroll
+        for (int k = 2; k >= 0; k--)
+            if (m[k] == qm) {
+                p = x[k];
+                pb = bits[k];
+                k0 = k;
+            }
+        best.val = qm;
+        best.col = col + k0 * 32 * E + __ffs(piece_equal<T>(p, pb, qm)) - 1;
+    } else if (best.col < 0 && (bits[0] | bits[1] | bits[2] | bits[3]) != 0u) {
+        // nothing yet and all the allowed values are -inf or NaN: the first -inf is a valid choice
+#pragma unroll
+        for (int k = 3; k >= 0; k--) {
+            uint32_t eq = piece_equal<T>(x[k], bits[k], -INFINITY);
+            if (eq) best.col = col + k * 32 * E + __ffs(eq) - 1;
+        }
+    }
 }
 
 // Allowed-position masks of a 16-byte piece: the shared-memory table of bf16 pieces, or
@@ -853,8 +734,7 @@ __global__ void __launch_bounds__(256) k_choose(const T* logits, int64_t stride,
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const uint32_t* rowids = D.mrows + (size_t)mid[b] * D.nch;
     const RowView<T> R(const_cast<T*>(logits) + (size_t)b * stride, V);
-    BestPiece bp = best_piece_none();
-    Best best{0.f, -1};
+    Best best;
     const int n = R.chunks(), step = csize * 8;
     // mask word `lane` of chunk j (and the word before the chunk, for lane 0)
     auto words = [&](int j, uint32_t& cur, uint32_t& before) {
@@ -873,32 +753,32 @@ __global__ void __launch_bounds__(256) k_choose(const T* logits, int64_t stride,
 #pragma unroll
         for (int k = 0; k < RowView<T>::PIECES; k++) bits[k] = piece_bits<T>(w, k, lane);
         const int x0 = (j << 10) + lane * RowView<T>::E;
-        if (R.edge(j)) {
+        const bool edged = R.edge(j);
+        if (edged) {
 #pragma unroll
             for (int k = 0; k < RowView<T>::PIECES; k++)
                 if (!R.whole(x0 + k * 32 * RowView<T>::E)) bits[k] = 0u;
-            int x = R.edge_element(j, lane);
-            uint32_t ew = __shfl_sync(FULL, w, (x >> 5) & 31);
-            if (x >= 0 && ((ew >> (x & 31)) & 1u)) {
-                float f = value_of(R.org[x]);
-                if (!isnan(f)) note_best(best, f, x - R.a);
-            }
         }
 #pragma unroll
         for (int h = 0; h < RowView<T>::PIECES; h += 4) {   // four pieces in flight
+            uint32_t qb[4];
             uint4 v[4];
 #pragma unroll
-            for (int k = 0; k < 4; k++)
-                v[k] = bits[h + k] ? ld_nc_v4(R.org + x0 + (h + k) * 32 * RowView<T>::E) : make_uint4(0u, 0u, 0u, 0u);
+            for (int k = 0; k < 4; k++) {
+                qb[k] = bits[h + k];
+                v[k] = qb[k] ? ld_nc_v4(R.org + x0 + (h + k) * 32 * RowView<T>::E) : make_uint4(0u, 0u, 0u, 0u);
+            }
 #pragma unroll
-            for (int k = 0; k < 4; k++)
-                if (bits[h + k])
-                    fold_piece<T>(bp, bits[h + k], mask_piece<T>(v[k], bits[h + k], s_lut),
-                                  x0 + (h + k) * 32 * RowView<T>::E - R.a);
+            for (int k = 0; k < 4; k++) v[k] = mask_piece<T>(v[k], qb[k], s_lut);
+            fold_quad<T>(best, qb, v, x0 + h * 32 * RowView<T>::E - R.a);
+        }
+        if (edged) {
+            int x = R.edge_element(j, lane);
+            uint32_t ew = __shfl_sync(FULL, w, (x >> 5) & 31);
+            if (x >= 0 && ((ew >> (x & 31)) & 1u)) note_best(best, value_of(R.org[x]), x - R.a);
         }
     }
-    unsigned long long key = best_key_of(best), kp = best_piece_key<T>(bp);
-    key = warp_max_key(kp > key ? kp : key);
+    const unsigned long long key = warp_max_key(best_key_of(best));
     uint32_t dst = static_cast<uint32_t>(__cvta_generic_to_shared(&s_key[rank * 8 + warp]));
     if (csize > 1) {
         // every CTA of the cluster has started before its shared memory is written to
@@ -919,196 +799,74 @@ __global__ void __launch_bounds__(256) k_choose(const T* logits, int64_t stride,
     }
 }
 
-// A lane's four 16-byte pieces of a bf16 chunk in registers: the mask bits of
-// each piece and its values with -inf where masked.
-struct ChunkRegs {
-    uint32_t bits[4];
-    uint4 x[4];
+// What a lane reads of one chunk before the chunk's mask word is known: its whole pieces
+// and its element outside them.
+template <typename T>
+struct ChunkAhead {
+    uint4 v[RowView<T>::PIECES];
+    T edge;
+    __device__ __forceinline__ ChunkAhead() {}
+    template <bool ANY>
+    __device__ __forceinline__ ChunkAhead(const RowView<T, ANY>& R, int j, int lane) {
+        const int x0 = (j << 10) + lane * RowView<T>::E;
+        const bool edged = R.edge(j);
+#pragma unroll
+        for (int k = 0; k < RowView<T>::PIECES; k++) {
+            int x = x0 + k * 32 * RowView<T>::E;
+            v[k] = !edged || R.whole(x) ? *reinterpret_cast<const uint4*>(R.org + x) : make_uint4(0u, 0u, 0u, 0u);
+        }
+        int x = edged ? R.edge_element(j, lane) : -1;
+        edge = x >= 0 ? R.org[x] : (T)0;
+    }
 };
 
-// Reads the lane's pieces of one 1024-column bf16 chunk from shared memory
-// (pieces with nothing allowed are not read) and masks them.  The stage may be
-// handed back as soon as this returns.
-__device__ __forceinline__ void load_mask_chunk_bf16(const uint16_t* src, uint32_t word, int lane, const uint4* lut,
-                                                     ChunkRegs& r) {
-    uint4 v[4];
+// One chunk of a row: -inf where w (the chunk's view word of this lane) masks, every
+// sector that holds a masked token written whole and no other (a partly written sector
+// costs a read-modify-write when the L2 evicts it); allowed values folded into the lane's
+// best when GREEDY.  The values come from `ahead` when it is given, else only the pieces
+// that must be read are (GREEDY: those that hold an allowed token, else those of sectors
+// to be written that do), four at a time.
+template <typename T, bool GREEDY, bool ANY>
+__device__ __forceinline__ void mask_chunk(const RowView<T, ANY>& R, int j, uint32_t w, int lane, const uint4* lut,
+                                           const ChunkAhead<T>* ahead, Best& best) {
+    constexpr int E = RowView<T>::E, P = RowView<T>::PIECES;
+    constexpr uint32_t F = RowView<T>::FULLBITS, N = NegInf<T>::pair;
+    const bool edged = R.edge(j);
+    const int x0 = (j << 10) + lane * E;
 #pragma unroll
-    for (int k = 0; k < 4; k++) r.bits[k] = (__shfl_sync(FULL, word, k * 8 + (lane >> 2)) >> ((lane & 3) * 8)) & 0xFFu;
+    for (int h = 0; h < P; h += 4) {
+        uint32_t bits[4];
+        uint4 v[4];
+        bool store[4];
 #pragma unroll
-    for (int k = 0; k < 4; k++)
-        v[k] = r.bits[k] ? *reinterpret_cast<const uint4*>(src + (k * 32 + lane) * 8) : make_uint4(0u, 0u, 0u, 0u);
+        for (int k = 0; k < 4; k++) {
+            bits[k] = piece_bits<T>(w, h + k, lane);
+            const bool in = !edged || R.whole(x0 + (h + k) * 32 * E);
+            if (!in) bits[k] = F;   // not this row's, or handled below: left as it is
+            store[k] = (bits[k] & __shfl_xor_sync(FULL, bits[k], 1)) != F && in;
+            if (!in) bits[k] = 0u;
+        }
 #pragma unroll
-    for (int k = 0; k < 4; k++) {
-        uint4 am = lut[r.bits[k]];
-        r.x[k] = make_uint4(sel_ninf(v[k].x, am.x, 0xFF80FF80u), sel_ninf(v[k].y, am.y, 0xFF80FF80u),
-                            sel_ninf(v[k].z, am.z, 0xFF80FF80u), sel_ninf(v[k].w, am.w, 0xFF80FF80u));
+        for (int k = 0; k < 4; k++) {
+            const bool need = bits[k] != 0u && (GREEDY || store[k]);
+            if (ahead) v[k] = ahead->v[h + k];
+            else v[k] = need ? *reinterpret_cast<const uint4*>(R.org + x0 + (h + k) * 32 * E) : make_uint4(N, N, N, N);
+        }
+#pragma unroll
+        for (int k = 0; k < 4; k++) {
+            v[k] = mask_piece<T>(v[k], bits[k], lut);
+            if (store[k]) st_cs_v4(R.org + x0 + (h + k) * 32 * E, v[k]);
+        }
+        if (GREEDY) fold_quad<T>(best, bits, v, x0 + h * 32 * E - R.a);
     }
-}
-
-// Folds a masked chunk into the lane's best piece with packed bf16x2 maxima (NaN
-// never wins: the maximum returns the other operand) and writes it to the row
-// (32-byte sectors with every token allowed are left as they are).
-// Every lane runs the same instructions for every piece; only a piece whose
-// allowed values are all -inf or NaN, met before any other allowed value, takes
-// a short scalar path.
-__device__ __forceinline__ void fold_store_chunk_bf16(uint16_t* row, int col0, int lane, const ChunkRegs& r,
-                                                      BestPiece& bp) {
-#pragma unroll
-    for (int k = 0; k < 4; k++) {
-        uint32_t bk = r.bits[k];
-        uint32_t x0 = r.x[k].x, x1 = r.x[k].y, x2 = r.x[k].z, x3 = r.x[k].w;
-        __nv_bfloat162 m = __hmax2(__hmax2(*reinterpret_cast<__nv_bfloat162*>(&x0), *reinterpret_cast<__nv_bfloat162*>(&x1)),
-                                   __hmax2(*reinterpret_cast<__nv_bfloat162*>(&x2), *reinterpret_cast<__nv_bfloat162*>(&x3)));
-        float mf = fmaxf(__low2float(m), __high2float(m));
-        int pc = col0 + (k * 32 + lane) * 8;
-        bool upd = mf > bp.val;
-        if (!upd && bk != 0u && bp.col < 0) {
-            // nothing allowed seen yet and this piece's allowed values are -inf or NaN:
-            // an allowed -inf is still a valid choice
-#pragma unroll
-            for (int e = 0; e < 8; e++) {
-                uint32_t wv = e < 2 ? x0 : e < 4 ? x1 : e < 6 ? x2 : x3;
-                if (((bk >> e) & 1) && bf16_at(wv, e & 1) == -INFINITY) upd = true;
-            }
+    if (edged) {   // after the pieces: a tie goes to the lower column either way
+        int x = R.edge_element(j, lane);
+        uint32_t ew = __shfl_sync(FULL, w, (x >> 5) & 31);
+        if (x >= 0) {
+            bool ok = (ew >> (x & 31)) & 1u;
+            if (GREEDY && ok) note_best(best, value_of(ahead ? ahead->edge : R.org[x]), x - R.a);
+            if (!ok) R.org[x] = (T)NegInf<T>::one;
         }
-        bp.val = upd ? mf : bp.val;
-        bp.col = upd ? pc : bp.col;
-        bp.bits = upd ? bk : bp.bits;
-        bp.x.x = upd ? x0 : bp.x.x;
-        bp.x.y = upd ? x1 : bp.x.y;
-        bp.x.z = upd ? x2 : bp.x.z;
-        bp.x.w = upd ? x3 : bp.x.w;
-        // a 32-byte sector (this lane's piece and its neighbour's) is written whole or not
-        // at all: a partly written sector costs a read-modify-write when the L2 evicts it.
-        // Only sectors whose 16 tokens are all allowed stay as they are.
-        uint32_t pair = bk & __shfl_xor_sync(FULL, bk, 1);
-        if (pair != 0xFFu) st_cs_v4(row + pc, r.x[k]);
-    }
-}
-
-template <typename T>
-__device__ __forceinline__ void apply_argmax_chunk_scalar(T* row, int col0, int ncols, uint32_t word, int lane,
-                                                          Best& best) {
-    int c0 = 32 * lane;
-    for (int e = 0; e < 32; e++) {
-        if (c0 + e >= ncols) break;
-        int col = col0 + c0 + e;
-        if (!((word >> e) & 1)) {
-            row[col] = (T)NegInf<T>::one;
-        } else {
-            float f = sizeof(T) == 2 ? __uint_as_float((uint32_t)row[col] << 16) : __uint_as_float((uint32_t)row[col]);
-            if (!isnan(f)) note_best(best, f, col);
-        }
-    }
-}
-
-template <typename T>
-__device__ __forceinline__ void apply_argmax_any(T* row, int col0, int V, uint32_t word, int lane, int vec, Best& best,
-                                                 const uint4* lut) {
-    int ncols = V - col0;
-    if (vec && ncols >= 1024) {
-        if (sizeof(T) == 2)
-            apply_argmax_chunk_bf16(reinterpret_cast<uint16_t*>(row) + col0, reinterpret_cast<uint16_t*>(row), col0,
-                                    word, lane, best, lut);
-        else
-            apply_argmax_chunk_f32(reinterpret_cast<uint32_t*>(row) + col0, reinterpret_cast<uint32_t*>(row), col0,
-                                   word, lane, best, lut);
-    } else {
-        apply_argmax_chunk_scalar<T>(row, col0, ncols < 1024 ? ncols : 1024, word, lane, best);
-    }
-}
-
-// Fused masking + greedy choice.  Work item = (row, segment of seg_chunks
-// 1024-column chunks); the 8 warps of a CTA split a segment, reduce their keys
-// in shared memory, and one 64-bit atomic max per item merges the row's best.
-// WALK: the CTA classifies its rows itself (Algorithm 2 step 3): warp 0 walks
-// the classifier for the next item's row while the CTA streams the current
-// item, chunks being handed out through a shared counter so that warp 0 joins
-// once its walk is done; the segment-0 CTA of a row records the row's mask id.
-// Per-row keys must be zero on entry (state init, finalize and advance clear them).
-template <typename T, bool WALK>
-__global__ void __launch_bounds__(256, 4) k_apply_argmax(T* logits, int64_t stride, MaskSrc M, int B, int V, int vec,
-                                                         int seg_chunks, unsigned long long* __restrict__ best_key,
-                                                         DevTables D, DevStates S) {
-    __shared__ unsigned long long red[8];
-    __shared__ int s_mid[2];
-    __shared__ int s_ctr;
-    __shared__ uint4 s_lut[256];
-    int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    int cpr = (V + 1023) >> 10;
-    int nseg = (cpr + seg_chunks - 1) / seg_chunks;
-    long items = (long)B * nseg;
-    int cur = 0;
-    build_allow_lut<T>(s_lut);
-    __syncthreads();
-    if (WALK) {
-        if (warp == 0 && (long)blockIdx.x < items) {
-            int m = warp_classify(D, S, (int)(blockIdx.x / nseg), lane);
-            if (lane == 0) s_mid[0] = m;
-        }
-        if (threadIdx.x == 0) s_ctr = 0;
-        __syncthreads();
-    }
-    for (long it = blockIdx.x; it < items; it += gridDim.x) {
-        int b = (int)(it / nseg);
-        int sg = (int)(it - (long)b * nseg);
-        int c0 = sg * seg_chunks;
-        int c1 = min(c0 + seg_chunks, cpr);
-        int wmid = 0;
-        if (WALK) {
-            wmid = s_mid[cur];
-            if (sg == 0 && threadIdx.x == 0) S.mid[b] = wmid;
-        }
-        // word `lane` of chunk j of this row's mask
-        auto word_at = [&](int j) -> uint32_t {
-            if (!WALK) return M.word(b, j, lane);
-            int wi = j * 32 + lane;
-            return wi < D.W ? __ldg(D.mchunks + (size_t)__ldg(D.mrows + (size_t)wmid * D.nch + j) * 32 + lane) : 0u;
-        };
-        T* row = logits + (size_t)b * stride;
-        Best best{0.f, -1};
-        if (WALK) {
-            long nx = it + gridDim.x;
-            if (warp == 0 && nx < items) {
-                int m = warp_classify(D, S, (int)(nx / nseg), lane);
-                if (lane == 0) s_mid[cur ^ 1] = m;
-            }
-            for (;;) {
-                int j = 0;
-                if (lane == 0) j = atomicAdd(&s_ctr, 1);
-                j = __shfl_sync(FULL, j, 0) + c0;
-                if (j >= c1) break;
-                int col0 = j << 10;
-                int wi = (col0 >> 5) + lane;
-                uint32_t word = word_at(j);
-                if (M.copy_out && wi < M.W) M.copy_out[(size_t)b * M.W + wi] = word;
-                apply_argmax_any<T>(row, col0, V, word, lane, vec, best, s_lut);
-            }
-        } else {
-            for (int j = c0 + warp; j < c1; j += 8) {
-                int col0 = j << 10;
-                int wi = (col0 >> 5) + lane;
-                uint32_t word = word_at(j);
-                if (M.copy_out && wi < M.W) M.copy_out[(size_t)b * M.W + wi] = word;
-                apply_argmax_any<T>(row, col0, V, word, lane, vec, best, s_lut);
-            }
-        }
-        unsigned long long key = best_key_of(best);
-#pragma unroll
-        for (int off = 16; off; off >>= 1) {
-            unsigned long long o = __shfl_xor_sync(FULL, key, off);
-            key = o > key ? o : key;
-        }
-        if (lane == 0) red[warp] = key;
-        __syncthreads();
-        if (threadIdx.x == 0) {
-            unsigned long long k = red[0];
-            for (int w = 1; w < 8; w++) k = red[w] > k ? red[w] : k;
-            if (k) atomicMax(best_key + b, k);
-            if (WALK) s_ctr = 0;
-        }
-        cur ^= 1;
-        __syncthreads();
     }
 }
 
@@ -1198,11 +956,6 @@ __device__ __forceinline__ int lds_u16(uint32_t a) {
 __device__ __forceinline__ int lds_u8(uint32_t a) {
     unsigned short v;
     asm volatile("ld.shared.u8 %0, [%1];" : "=h"(v) : "r"(a));
-    return v;
-}
-__device__ __forceinline__ int lds_s32(uint32_t a) {
-    int v;
-    asm volatile("ld.shared.s32 %0, [%1];" : "=r"(v) : "r"(a));
     return v;
 }
 __device__ __forceinline__ uint32_t lds_u32(uint32_t a) {
@@ -1478,8 +1231,9 @@ __device__ __forceinline__ int warp_memo_extend(const DevTables& T, const StackV
 // rows; the host sets `early` only when the masking pass is the last work on
 // these states and took the mask ids as they were.
 template <bool PACKED, bool COMB>
-__global__ void __launch_bounds__(ADV_WARPS * 32) k_advance_warp(DevTables T, DevStates S, const int32_t* tokens,
-                                                                 int B, int use_mid, int32_t* status_out,
+__global__ void __launch_bounds__(ADV_WARPS * 32, 1)   // the staged tables leave room for one CTA per SM: no spills
+    k_advance_warp(DevTables T, DevStates S, const int32_t* tokens,
+                                                                 int B, int32_t* status_out,
                                                                  int from_keys, int32_t* tokens_out, int early) {
     extern __shared__ uint4 smem4[];
     __shared__ __align__(8) uint64_t bar;
@@ -1521,7 +1275,7 @@ __global__ void __launch_bounds__(ADV_WARPS * 32) k_advance_warp(DevTables T, De
         depth = __ldcg(S.depth + b);
         depth0 = depth;
         status = __ldcg(S.status + b);
-        cur_mid = use_mid ? __ldcg(S.mid + b) : 0;
+        cur_mid = __ldcg(S.mid + b);
         live = status == ROW_OK && depth >= 1 && depth <= S.cap;
         if (live) {
             sv.base = depth > ADV_KEEP ? depth - ADV_KEEP : 0;
@@ -1552,13 +1306,6 @@ __global__ void __launch_bounds__(ADV_WARPS * 32) k_advance_warp(DevTables T, De
                 if (tok >= T.V) {
                     status = ROW_REJECTED;
                 } else {
-                    if (!use_mid) {   // the kept bottom-up block, else a walk of the stack in global memory
-                        int e = __shfl_sync(FULL, memo_top, 0);
-                        cur_mid = memo && live && q >= 0 && q < T.nq ? memo_mask(T, e, q) : -1;
-                        StackView g{sv.win, sv.st, 0x40000000, 0x7FFFFFFF, sv.wa};
-                        if (cur_mid < 0)
-                            cur_mid = depth >= 1 && depth <= S.cap ? warp_walk(T, g, q, depth, lane) : 0;
-                    }
                     // the token's mask bit (in flight while the token is parsed); the row is
                     // only committed (q, depth) when it is set
                     mword = mask_word(T, cur_mid, tok >> 5);
@@ -1738,364 +1485,59 @@ __global__ void __launch_bounds__(ADV_WARPS * 32) k_advance_warp(DevTables T, De
     if (lane == 0) S.mid[b] = mid;
 }
 
-// ------------------------------------------ TMA-pipelined decode masking pass
-__device__ __forceinline__ void mbar_init(uint32_t bar, uint32_t count) {
-    asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(bar), "r"(count) : "memory");
-}
-__device__ __forceinline__ void mbar_arrive(uint32_t bar) {
-    asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(bar) : "memory");
-}
-__device__ __forceinline__ void mbar_arrive_tx(uint32_t bar, uint32_t bytes) {
-    asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(bar), "r"(bytes) : "memory");
-}
-// Bounded wait for the phase with the given parity to complete (about a few
-// seconds at most; a pipeline wait that gives up is counted and the kernel ends).
-__device__ __forceinline__ bool mbar_wait(uint32_t bar, uint32_t parity) {
-    for (int it = 0; it < (1 << 22); it++) {
-        uint32_t ok;
-        asm volatile(
-            "{\n .reg .pred p;\n mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n selp.u32 %0, 1, 0, p;\n}"
-            : "=r"(ok)
-            : "r"(bar), "r"(parity)
-            : "memory");
-        if (ok) return true;
-    }
-    return false;
-}
-// 1-D bulk copy global -> shared, completing on the mbarrier (16-byte aligned, size a multiple of 16).
-__device__ __forceinline__ void tma_load_1d(uint32_t dst, const void* src, uint32_t bytes, uint32_t bar) {
-    asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];"
-                 ::"r"(dst), "l"(gmem_addr(src)), "r"(bytes), "r"(bar)
-                 : "memory");
-}
-// The same with an L2 cache policy (the streamed logits go first when L2 evicts,
-// so the classifier table and mask rows the walks and the mask copies read stay).
-__device__ __forceinline__ void tma_load_1d_hint(uint32_t dst, const void* src, uint32_t bytes, uint32_t bar,
-                                                 uint64_t policy) {
-    asm volatile(
-        "cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes.L2::cache_hint [%0], [%1], %2, [%3], %4;"
-        ::"r"(dst), "l"(gmem_addr(src)), "r"(bytes), "r"(bar), "l"(policy)
-        : "memory");
-}
-__device__ __forceinline__ uint64_t l2_evict_first_policy() {
-    uint64_t p;
-    asm volatile("createpolicy.fractional.L2::evict_first.b64 %0, 1.0;" : "=l"(p));
-    return p;
-}
-
-
-constexpr long WARP_STEP_CHUNKS = 4096;   // batches of at most this many 1024-column chunks: k_step_warp
-constexpr int TMA_SEG = 32;     // most 1024-column chunks per work item (one per lane of a warp)
-constexpr int TMA_NCONS = 8;    // consumer warps; a ring stage holds one chunk for each of them
-constexpr int TMA_WARPS = TMA_NCONS + 2;   // + producer + walker
-constexpr int TMA_MIDS = 4;     // classified rows the walker may run ahead (it walks them together)
-constexpr int TMA_MSLOTS = 3;   // mask-word buffers: the next item's words load while this item streams
-
-// Shared-memory plan of the pipelined pass: NS ring stages of TMA_NCONS chunks,
-// TMA_MSLOTS mask-word buffers (TMA_SEG x 32 words each), then the mbarriers.
-template <typename T>
-struct TmaShape {
-    static constexpr int CHUNK = 1024 * (int)sizeof(T);   // bytes of one 1024-column chunk
-    static constexpr int STAGE = TMA_NCONS * CHUNK;
-    static constexpr int NS = sizeof(T) == 2 ? 3 : 2;
-    static constexpr int NBARS = 2 * NS + 2 * TMA_MSLOTS + 2 * TMA_MIDS;
-    static constexpr int SMEM = NS * STAGE + TMA_MSLOTS * TMA_SEG * 32 * 4 + NBARS * 8;
-};
-
-// The decode masking pass for small batches of bf16 rows whose mask ids are
-// current, a warp per 1024-column chunk, eight chunks per CTA.  A lane loads its
-// four 16-byte pieces of the chunk at once, whatever the mask (at these sizes the
-// bytes are cheap and the latency is not), while the chunk's mask word comes
-// through the row's mask id and chunk id; then the same masking, greedy fold,
-// sector rule and keys as k_step_tma.  Requires 16-byte aligned rows.
-__global__ void __launch_bounds__(256) k_step_warp(uint16_t* logits, int64_t stride, int B, int V, uint32_t* copy_out,
-                                                   unsigned long long* __restrict__ best_key, DevTables D,
-                                                   DevStates S) {
-    __shared__ uint4 s_lut[256];
-    build_allow_lut<uint16_t>(s_lut);
+// ------------------------------------------------------------ decode masking pass
+// The masking pass: a warp takes SPAN neighbouring 1024-element chunks of a row view, eight
+// warps per CTA.  The chunks' mask words come through the row's mask id and the chunk ids
+// (three dependent loads, side by side for the chunks); then every piece that holds an
+// allowed token is read, masked, folded into the greedy choice and written back (sectors
+// with nothing masked are not written, pieces with nothing allowed are not read).  cpv:
+// chunks of the longest row view.
+//
+// Large batches are bound by DRAM: what counts is bytes in flight, so few registers (a lane
+// keeps a value and a column, not the piece) and several chunks' words per chain of
+// dependent loads.  1024 rows x 262,144 bf16 tokens, whole decode step replayed from a
+// CUDA graph: 148 us with SPAN 4, 150 with 2, 162 with 1, 172 with the TMA-pipelined pass
+// that this one replaced; x 128,256 tokens: 71 / 75 / 79 / 101 us; 512 x 151,665 (rows not
+// aligned): 65 / 69 / 76 / 385 us (element by element).  f32, 512 rows x 262,144: 150 us
+// with SPAN 2 (152 with 4, 198 with the TMA pass).
+//
+// Small batches are bound by that chain of loads: AHEAD reads all the pieces while the mask
+// word arrives (one row of 151,936 f32 tokens: 8.9 us per step instead of 10.3; one of
+// 262,144 bf16 tokens 7.3 instead of 7.7).
+template <typename T, bool ANY, int SPAN, bool AHEAD>
+__global__ void __launch_bounds__(256) k_step_warp(T* logits, int64_t stride, MaskSrc M, int B, int V, int cpv,
+                                                   unsigned long long* __restrict__ best_key) {
+    __shared__ uint4 s_lut[sizeof(T) == 2 ? 256 : 1];
+    if (sizeof(T) == 2) build_allow_lut<T>(s_lut);
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const int cpr = (V + 1023) >> 10, cpb = (cpr + 7) >> 3;   // chunks per row, CTAs per row
-    const int b = blockIdx.x / cpb, j = (blockIdx.x - b * cpb) * 8 + warp;
+    const unsigned c = blockIdx.x * 8u + warp;   // fewer than 2^32: a chunk takes 2 KiB of logits or a whole row
+    const unsigned spr = (unsigned)(cpv + SPAN - 1) / SPAN;
+    const int b = (int)(c / spr), j0 = (int)(c - (unsigned)b * spr) * SPAN;
     grid_dep_wait();   // logits, mask ids and greedy keys come from earlier kernels
     grid_dep_launch();
     __syncthreads();   // the allow-mask table
-    if (b >= B || j >= cpr) return;
-    uint16_t* row = logits + (size_t)b * stride;
-    const int col0 = j << 10;
-    const bool whole = col0 + 1024 <= V;
-    uint4 v[4];
-    if (whole) {
+    if (b >= B) return;
+    const RowView<T, ANY> R(logits + (size_t)b * stride, V);
+    const int n = R.chunks();
+    if (j0 >= n) return;
+    ChunkAhead<T> ahead[SPAN];
+    uint32_t cur[SPAN], before;
 #pragma unroll
-        for (int k = 0; k < 4; k++) v[k] = *reinterpret_cast<const uint4*>(row + col0 + (k * 32 + lane) * 8);
-    }
-    const int mid = S.mid[b];
-    const uint32_t cid = __ldg(D.mrows + (size_t)mid * D.nch + j);
-    const uint32_t w = __ldg(D.mchunks + (size_t)cid * 32 + lane);
-    if (copy_out) {
-        int wi = j * 32 + lane;
-        if (wi < D.W) copy_out[(size_t)b * D.W + wi] = w;
-    }
-    Best best{0.f, -1};
-    BestPiece bp = best_piece_none();
-    if (!whole) {
-        apply_argmax_chunk_scalar<uint16_t>(row, col0, V - col0, w, lane, best);
-    } else {
-        ChunkRegs r;
+    for (int i = 0; i < SPAN; i++)
+        if (AHEAD && (SPAN == 1 || j0 + i < n)) ahead[i] = ChunkAhead<T>(R, j0 + i, lane);
+    M.template table_words<SPAN, ANY>(b, j0, lane, cur, before);
+    Best best;
 #pragma unroll
-        for (int k = 0; k < 4; k++) r.bits[k] = (__shfl_sync(FULL, w, k * 8 + (lane >> 2)) >> ((lane & 3) * 8)) & 0xFFu;
-#pragma unroll
-        for (int k = 0; k < 4; k++) {
-            uint4 am = s_lut[r.bits[k]];
-            r.x[k] = make_uint4(sel_ninf(v[k].x, am.x, 0xFF80FF80u), sel_ninf(v[k].y, am.y, 0xFF80FF80u),
-                                sel_ninf(v[k].z, am.z, 0xFF80FF80u), sel_ninf(v[k].w, am.w, 0xFF80FF80u));
-        }
-        fold_store_chunk_bf16(row, col0, lane, r, bp);
+    for (int i = 0; i < SPAN; i++) {
+        const int j = j0 + i;
+        if (SPAN > 1 && j >= n) break;
+        if (M.copy_out && j * 32 + lane < M.W) M.copy_out[(size_t)b * M.W + j * 32 + lane] = cur[i];
+        if (i > 0) before = __shfl_sync(FULL, cur[i - 1], 31);
+        mask_chunk<T, true>(R, j, view_word(cur[i], before, R.a, lane), lane, s_lut,
+                            AHEAD ? &ahead[i] : (const ChunkAhead<T>*)nullptr, best);
     }
-    unsigned long long key = best_key_of(best), kp = best_piece_key_bf16(bp);
-    key = kp > key ? kp : key;
-    uint32_t khi = (uint32_t)(key >> 32), klo = (uint32_t)key;
-    uint32_t mhi = __reduce_max_sync(FULL, khi);
-    uint32_t mlo = __reduce_max_sync(FULL, khi == mhi ? klo : 0u);
-    key = ((unsigned long long)mhi << 32) | mlo;
+    const unsigned long long key = warp_max_key(best_key_of(best));
     if (lane == 0 && key) atomicMax(best_key + b, key);
-}
-
-// One decode masking pass (classification, mask, apply, greedy key) with the
-// logits streamed through shared memory by TMA bulk copies.  Work item = (row,
-// segment of `seg` <= TMA_SEG chunks).  Warp 0 (producer) fetches each item's mask words
-// one item ahead, then for every ring stage copies the stage's chunks that hold
-// an allowed position (runs of neighbouring chunks in one copy; chunks with
-// nothing allowed are not read); warp 1 reads (or, when they are not current,
-// computes) the mask ids of the CTA's upcoming rows; consumer warp c takes chunk c of every stage, writes -inf where
-// masked and folds allowed values into the row's greedy key.
-// Requires 16-byte aligned rows; rows' mask rows padded to whole chunks.
-template <typename T>
-__global__ void __launch_bounds__(TMA_WARPS * 32, 3) k_step_tma(T* logits, int64_t stride, int B, int V,
-                                                                uint32_t* copy_out,
-                                                                unsigned long long* __restrict__ best_key,
-                                                                DevTables D, DevStates S, int have_mid, int seg) {
-    using Sh = TmaShape<T>;
-    constexpr int NS = Sh::NS, CHUNK = Sh::CHUNK, STAGE = Sh::STAGE;
-    static_assert(TMA_SEG == 32, "one lane per chunk of an item");
-    static_assert(TMA_NCONS <= 32 && TMA_SEG % TMA_NCONS == 0, "whole stages per item");
-    extern __shared__ __align__(128) uint8_t smem[];
-    uint8_t* tiles = smem;
-    uint32_t* mbuf = reinterpret_cast<uint32_t*>(smem + NS * STAGE);
-    uint64_t* bars = reinterpret_cast<uint64_t*>(mbuf + TMA_MSLOTS * TMA_SEG * 32);
-    __shared__ int s_mid[TMA_MIDS];
-    __shared__ uint4 s_lut[256];
-    int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    int cpr = (V + 1023) >> 10;
-    int nseg = (cpr + seg - 1) / seg;
-    build_allow_lut<T>(s_lut);
-    long items = (long)B * nseg;
-    const uint32_t full0 = smem_addr(bars), empty0 = full0 + 8 * NS, mfull0 = empty0 + 8 * NS;
-    const uint32_t mempty0 = mfull0 + 8 * TMA_MSLOTS, midf0 = mempty0 + 8 * TMA_MSLOTS, mide0 = midf0 + 8 * TMA_MIDS;
-    if (threadIdx.x == 0) {
-        for (int k = 0; k < NS; k++) {
-            mbar_init(full0 + 8 * k, 1);
-            mbar_init(empty0 + 8 * k, TMA_NCONS);
-        }
-        for (int k = 0; k < TMA_MSLOTS; k++) {
-            mbar_init(mfull0 + 8 * k, 1);
-            mbar_init(mempty0 + 8 * k, TMA_NCONS);
-        }
-        for (int k = 0; k < TMA_MIDS; k++) {
-            mbar_init(midf0 + 8 * k, 1);
-            mbar_init(mide0 + 8 * k, 1);
-        }
-        asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
-        asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
-    }
-    __syncthreads();
-    grid_dep_wait();   // mask ids, greedy keys and rows come from the previous kernel
-    // the next kernel (the advance) may start now: the rows' writer before this pass
-    // has completed, so the advance can read the rows before its own wait
-    grid_dep_launch();
-    bool failed = false;
-    if (warp == 0) {
-        // ---------------------------------------------------------- producer
-        long s = 0;            // ring stages issued
-        int issued = -1;       // last item whose mask words were requested
-        const uint64_t stream_policy = l2_evict_first_policy();
-        // request item ii's mask words (its row classified by the walker) into slot ii % TMA_MSLOTS
-        auto fetch_mask = [&](int ii, long itm) -> bool {
-            int b = (int)(itm / nseg), sg = (int)(itm - (long)b * nseg);
-            int c0 = sg * seg, nch = min(seg, cpr - c0);
-            int ms = ii % TMA_MIDS;
-            if (!__shfl_sync(FULL, (int)mbar_wait(midf0 + 8 * ms, (uint32_t)((ii / TMA_MIDS) & 1)), 0)) return false;
-            int mid = s_mid[ms];
-            __syncwarp();
-            int slot = ii % TMA_MSLOTS, use = ii / TMA_MSLOTS;
-            if (lane == 0) {
-                mbar_arrive(mide0 + 8 * ms);
-                if (sg == 0 && !have_mid) S.mid[b] = mid;
-            }
-            if (use >= 1 && !__shfl_sync(FULL, (int)mbar_wait(mempty0 + 8 * slot, (uint32_t)((use - 1) & 1)), 0))
-                return false;
-            // the item's chunk ids, then one 128-byte bulk copy per chunk (lane k: chunk k)
-            uint32_t cid = lane < nch ? __ldg(D.mrows + (size_t)mid * D.nch + c0 + lane) : 0u;
-            if (lane == 0) mbar_arrive_tx(mfull0 + 8 * slot, nch * 128);
-            __syncwarp();
-            if (lane < nch)
-                tma_load_1d(smem_addr(mbuf + slot * TMA_SEG * 32 + lane * 32), D.mchunks + (size_t)cid * 32, 128,
-                            mfull0 + 8 * slot);
-            issued = ii;
-            return true;
-        };
-        int i = 0;
-        if ((long)blockIdx.x < items && !fetch_mask(0, blockIdx.x)) failed = true;
-        for (long it = blockIdx.x; it < items && !failed; it += gridDim.x, i++) {
-            int b = (int)(it / nseg), sg = (int)(it - (long)b * nseg);
-            int c0 = sg * seg, nch = min(seg, cpr - c0);
-            if (it + gridDim.x < items && !fetch_mask(i + 1, it + gridDim.x)) { failed = true; break; }
-            int slot = i % TMA_MSLOTS;
-            if (!__shfl_sync(FULL, (int)mbar_wait(mfull0 + 8 * slot, (uint32_t)((i / TMA_MSLOTS) & 1)), 0)) {
-                failed = true;
-                break;
-            }
-            // lane k: does chunk k of the item hold an allowed position?  (rotated reads: no bank conflicts)
-            const uint32_t* mb = mbuf + slot * TMA_SEG * 32;
-            uint32_t acc = 0;
-#pragma unroll 8
-            for (int k = 0; k < 32; k++) acc |= mb[lane * 32 + ((k + lane) & 31)];
-            uint32_t load = __ballot_sync(FULL, acc != 0u && lane < nch);
-            if (c0 + nch == cpr && (V & 1023)) load &= ~(1u << (nch - 1));   // the ragged chunk is read directly
-            const T* row = logits + (size_t)b * stride;
-            for (int g = 0; g * TMA_NCONS < nch; g++, s++) {
-                int stg = (int)(s % NS);
-                if (s >= NS && !__shfl_sync(FULL, (int)mbar_wait(empty0 + 8 * stg, (uint32_t)(((s / NS) - 1) & 1)), 0)) {
-                    failed = true;
-                    break;
-                }
-                if (lane == 0) {
-                    uint32_t f = (load >> (g * TMA_NCONS)) & ((1u << TMA_NCONS) - 1u);
-                    if (f) {
-                        mbar_arrive_tx(full0 + 8 * stg, (uint32_t)(__popc(f) * CHUNK));
-                        while (f) {
-                            int a = __ffs(f) - 1;
-                            int len = __ffs(~(f >> a)) - 1;
-                            tma_load_1d_hint(smem_addr(tiles + stg * STAGE + a * CHUNK),
-                                             row + (size_t)(c0 + g * TMA_NCONS + a) * 1024, (uint32_t)(len * CHUNK),
-                                             full0 + 8 * stg, stream_policy);
-                            f &= ~(((1u << len) - 1u) << a);
-                        }
-                    } else {
-                        mbar_arrive(full0 + 8 * stg);
-                    }
-                }
-            }
-        }
-        if (failed && lane == 0) {
-            // let this CTA's copies in flight land before it exits (bounded)
-            for (long tt = s > NS ? s - NS : 0; tt < s; tt++) mbar_wait(full0 + 8 * (int)(tt % NS), (uint32_t)((tt / NS) & 1));
-            for (int ii = issued > 0 ? issued - 1 : 0; ii <= issued; ii++)
-                mbar_wait(mfull0 + 8 * (ii % TMA_MSLOTS), (uint32_t)((ii / TMA_MSLOTS) & 1));
-        }
-    } else if (warp == 1) {
-        // ------------------------------------------------------------ walker
-        // lanes 0..TMA_MIDS-1 each classify one of the next TMA_MIDS items' rows, so
-        // the dependent table loads of those classifications overlap
-        int i = 0;
-        for (long it = blockIdx.x; it < items && !failed; it += (long)gridDim.x * TMA_MIDS, i += TMA_MIDS) {
-            if (i >= TMA_MIDS && !__shfl_sync(FULL, (int)mbar_wait(mide0 + 8 * (TMA_MIDS - 1),
-                                                                    ((i / TMA_MIDS) - 1) & 1), 0)) {
-                failed = true;
-                break;
-            }
-            long my = it + (long)lane * gridDim.x;
-            int mid = 0;
-            if (lane < TMA_MIDS && my < items) {
-                int rb = (int)(my / nseg);
-                mid = have_mid ? S.mid[rb] : thread_classify(D, S, rb);
-            }
-            if (lane < TMA_MIDS && my < items) {
-                s_mid[lane] = mid;
-                mbar_arrive(midf0 + 8 * lane);
-            }
-            __syncwarp();
-        }
-    } else {
-        // --------------------------------------------------------- consumers
-        int c = warp - 2;
-        long s = 0;
-        int i = 0;
-        for (long it = blockIdx.x; it < items && !failed; it += gridDim.x, i++) {
-            int b = (int)(it / nseg), sg = (int)(it - (long)b * nseg);
-            int c0 = sg * seg, nch = min(seg, cpr - c0);
-            int slot = i % TMA_MSLOTS;
-            if (!__shfl_sync(FULL, (int)mbar_wait(mfull0 + 8 * slot, (uint32_t)((i / TMA_MSLOTS) & 1)), 0)) {
-                failed = true;
-                break;
-            }
-            const uint32_t* mb = mbuf + slot * TMA_SEG * 32;
-            T* row = logits + (size_t)b * stride;
-            Best best{0.f, -1};
-            BestPiece bp = best_piece_none();
-            for (int g = 0; g * TMA_NCONS < nch; g++, s++) {
-                int stg = (int)(s % NS);
-                if (!__shfl_sync(FULL, (int)mbar_wait(full0 + 8 * stg, (uint32_t)((s / NS) & 1)), 0)) {
-                    failed = true;
-                    break;
-                }
-                int k = g * TMA_NCONS + c;
-                bool released = false;
-                if (k < nch) {
-                    int j = c0 + k;
-                    uint32_t w = mb[k * 32 + lane];
-                    if (copy_out) {
-                        int wi = j * 32 + lane;
-                        if (wi < D.W) copy_out[(size_t)b * D.W + wi] = w;
-                    }
-                    int col0 = j << 10;
-                    const uint8_t* tile = tiles + stg * STAGE + c * CHUNK;
-                    if ((j == cpr - 1) && (V & 1023)) {
-                        apply_argmax_chunk_scalar<T>(row, col0, V - col0, w, lane, best);
-                    } else if (__ballot_sync(FULL, w != 0u) == 0u) {
-                        constexpr int PIECES = CHUNK / 16 / 32;
-                        uint4 ninf = make_uint4(NegInf<T>::pair, NegInf<T>::pair, NegInf<T>::pair, NegInf<T>::pair);
-#pragma unroll
-                        for (int q = 0; q < PIECES; q++)
-                            st_cs_v4(reinterpret_cast<uint8_t*>(row + col0) + (q * 32 + lane) * 16, ninf);
-                    } else if constexpr (sizeof(T) == 2) {
-                        // the chunk goes to registers and the stage back to the producer
-                        // before the chunk is folded and written out
-                        ChunkRegs r;
-                        load_mask_chunk_bf16(reinterpret_cast<const uint16_t*>(tile), w, lane, s_lut, r);
-                        __syncwarp();
-                        if (lane == 0) mbar_arrive(empty0 + 8 * stg);
-                        released = true;
-                        fold_store_chunk_bf16(reinterpret_cast<uint16_t*>(row), col0, lane, r, bp);
-                    } else {
-                        apply_argmax_chunk_f32(reinterpret_cast<const uint32_t*>(tile), reinterpret_cast<uint32_t*>(row),
-                                               col0, w, lane, best, s_lut);
-                    }
-                }
-                if (!released) {
-                    __syncwarp();
-                    if (lane == 0) mbar_arrive(empty0 + 8 * stg);
-                }
-            }
-            unsigned long long key = best_key_of(best);
-            if constexpr (sizeof(T) == 2) {
-                unsigned long long kp = best_piece_key_bf16(bp);
-                key = kp > key ? kp : key;
-            }
-            // warp maximum of the 64-bit keys: the high words, then the low words of the lanes holding it
-            uint32_t khi = (uint32_t)(key >> 32), klo = (uint32_t)key;
-            uint32_t mhi = __reduce_max_sync(FULL, khi);
-            uint32_t mlo = __reduce_max_sync(FULL, khi == mhi ? klo : 0u);
-            key = ((unsigned long long)mhi << 32) | mlo;
-            if (lane == 0) {
-                if (key) atomicMax(best_key + b, key);
-                mbar_arrive(mempty0 + 8 * slot);
-            }
-        }
-    }
-    if (failed && lane == 0) {
-        atomicAdd(&g_pipeline_timeouts, 1);
-        if (S.fault) atomicAdd(S.fault, 1);
-    }
 }
 
 // A bounded wait on an mbarrier phase that nothing completes: gives up after
@@ -2105,7 +1547,7 @@ __global__ void k_wait_gives_up(DevStates S, int limit) {
     __shared__ __align__(8) uint64_t bar;
     uint32_t a = smem_addr(&bar);
     if (threadIdx.x == 0) {
-        mbar_init(a, 1);
+        asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(a) : "memory");
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
     __syncthreads();
@@ -2158,6 +1600,8 @@ psc_status check_device(const psc_handle* h, const char* what) {
     return PSC_OK;
 }
 
+// Classifies the rows when their mask ids are not current (an earlier launch failed; every
+// call that changes rows computes the ids with them).
 psc_status ensure_mid(const psc_handle* h, const psc_states* st, cudaStream_t s) {
     const_cast<psc_states*>(st)->after_mask = false;
     if (st->mid_gen == st->gen) return PSC_OK;
@@ -2188,8 +1632,16 @@ psc_status launch_apply(void* logits, psc_dtype dtype, int64_t row_stride, const
     return launch_check("k_apply_rows");
 }
 
-// Masking + greedy choice with in-kernel classification; leaves each row's
-// key in st->d.best and its mask id in st->d.mid.
+// The most elements between a row's first element and the 32-byte boundary at or below
+// it, over the batch's rows (RowView's a): 0 when every row starts on one.
+int row_lead(const void* logits, psc_dtype dtype, int64_t row_stride, int B) {
+    const int esz = dtype == PSC_BF16 ? 2 : 4;
+    int most = 0;
+    for (int b = 0; b < std::min(B, 32 / esz); b++)   // the leads repeat with at most this period
+        most = std::max(most, (int)(((uintptr_t)logits + (uintptr_t)b * (uintptr_t)row_stride * esz) & 31u) / esz);
+    return most;
+}
+
 // Launches a kernel that may start while the previous kernel of the stream finishes
 // (programmatic dependent launch): it waits for that kernel's results itself.
 template <typename... KArgs, typename... Args>
@@ -2232,14 +1684,14 @@ psc_status launch_choose(const T* logits, int64_t stride, const psc_handle* h, c
 // Algorithm 2 steps 1-2 for every row (the token given, or the fused pass's greedy
 // choice when d_tokens_out is set), then step 3 for the new configurations: the
 // rows' mask ids are current afterwards.
-using AdvanceKernel = void (*)(DevTables, DevStates, const int32_t*, int, int, int32_t*, int, int32_t*, int);
+using AdvanceKernel = void (*)(DevTables, DevStates, const int32_t*, int, int32_t*, int, int32_t*, int);
 AdvanceKernel advance_kernel(const DevTables& d) {
     if (d.adv_comb) return d.adv_packed ? k_advance_warp<true, true> : k_advance_warp<false, true>;
     return d.adv_packed ? k_advance_warp<true, false> : k_advance_warp<false, false>;
 }
 
-psc_status launch_advance(const psc_handle* h, psc_states* st, const int32_t* d_tokens, int use_mid,
-                          int32_t* d_row_status, int32_t* d_tokens_out, cudaStream_t cs) {
+psc_status launch_advance(const psc_handle* h, psc_states* st, const int32_t* d_tokens, int32_t* d_row_status,
+                          int32_t* d_tokens_out, cudaStream_t cs) {
     int B = st->d.B;
     int from_keys = d_tokens_out ? 1 : 0;
     int early = from_keys && st->after_mask ? 1 : 0;
@@ -2248,10 +1700,10 @@ psc_status launch_advance(const psc_handle* h, psc_states* st, const int32_t* d_
     if (h->d.adv_bytes > 0) {
         s = launch_pdl(advance_kernel(h->d),
                        dim3((B + ADV_WARPS - 1) / ADV_WARPS), dim3(ADV_WARPS * 32), adv_smem(h->d), cs,
-                       "k_advance_warp", h->d, st->d, d_tokens, B, use_mid, d_row_status, from_keys, d_tokens_out,
+                       "k_advance_warp", h->d, st->d, d_tokens, B, d_row_status, from_keys, d_tokens_out,
                        early);
     } else {
-        k_advance<<<(B + 127) / 128, 128, 0, cs>>>(h->d, st->d, d_tokens, B, use_mid, d_row_status, from_keys,
+        k_advance<<<(B + 127) / 128, 128, 0, cs>>>(h->d, st->d, d_tokens, B, d_row_status, from_keys,
                                                     d_tokens_out);
         s = launch_check("k_advance");
         if (s == PSC_OK) {
@@ -2265,62 +1717,48 @@ psc_status launch_advance(const psc_handle* h, psc_states* st, const int32_t* d_
     return s;
 }
 
+// k_step_warp's variant by the batch's chunks (bf16, us per step: 32 rows x 128,256, 4,032
+// chunks, 10.9 with AHEAD, 11.8 with SPAN 2; 32 rows x 262,144 16.3 / 14.5; 256 rows, 65,536 chunks, 47.1 with
+// SPAN 2, 48.5 with 4; 512 rows 84.3 / 84.5, unaligned rows 69.0 / 64.5 at 76,000 chunks.
+// f32 x 151,936: 32 rows, 4,768 chunks, 16.7 with AHEAD, 17.1 with SPAN 2; 128 rows 34.8 /
+// 33.2).
+constexpr long AHEAD_CHUNKS_BF16 = 4096, AHEAD_CHUNKS_F32 = 8192, SPAN4_CHUNKS = 65536;
+template <int SPAN, bool AHEAD, typename T>
+psc_status launch_step_warp(T* logits, int64_t stride, const MaskSrc& M, int B, int V, int cpv, bool any,
+                            unsigned long long* best, cudaStream_t cs) {
+    dim3 grid((unsigned)(((long)B * ((cpv + SPAN - 1) / SPAN) + 7) / 8));
+    return launch_pdl(any ? k_step_warp<T, true, SPAN, AHEAD> : k_step_warp<T, false, SPAN, AHEAD>, grid, dim3(256), 0, cs,
+                      "k_step_warp", logits, stride, M, B, V, cpv, best);
+}
+
+// Masking + greedy choice; leaves each row's key in st->d.best.
 psc_status launch_fused(const psc_handle* h, const psc_states* st, void* d_logits, psc_dtype dtype, int64_t row_stride,
                         int V, uint32_t* d_bitmask_out, cudaStream_t cs) {
     int B = st->d.B;
+    psc_status s = ensure_mid(h, st, cs);
+    if (s != PSC_OK) return s;
     MaskSrc M{nullptr, h->d.mchunks, h->d.mrows, st->d.mid, h->d.W, h->d.nch, d_bitmask_out};
-    size_t esz = dtype == PSC_BF16 ? 2 : 4;
-    int vec = aligned16(d_logits) && ((row_stride * (int64_t)esz) % 16 == 0);
-    int cpr = (V + 1023) / 1024;
-    int have_mid = st->mid_gen == st->gen ? 1 : 0;   // mask ids current: no classifier walks
-    psc_status s;
-    if (vec) {
-        // the pipelined pass (rows 16-byte aligned): as many CTAs as are resident at once;
-        // items of 32 chunks; smaller (multiples of a stage) when the batch has too few
-        // chunks to give every resident CTA work (one chunk per item instead of a stage
-        // was measured no faster at batch 1: 8.3 us per graph-replayed step either way)
-        long resident = (long)sm_count(h->device) * h->tma_ctas[dtype == PSC_BF16 ? 0 : 1];
-        // small bf16 batches with current mask ids: a warp per chunk (measured on config 5's
-        // tables, decode steps replayed from CUDA graphs: 7.5 instead of 9.2 us at batch 1,
-        // 11.7 instead of 14.1 at 16).  Larger batches: the TMA pipeline below keeps more
-        // bytes in flight (at batch 1024 the warp-per-chunk pass took 169.7 us per launch
-        // against 157.6)
-        if (dtype == PSC_BF16 && have_mid && (long)B * cpr <= WARP_STEP_CHUNKS) {
-            s = launch_pdl(k_step_warp, dim3(B * ((cpr + 7) / 8)), dim3(256), 0, cs, "k_step_warp",
-                           (uint16_t*)d_logits, row_stride, B, V, d_bitmask_out, st->d.best, h->d, st->d);
-            if (s == PSC_OK) const_cast<psc_states*>(st)->mid_gen = st->gen;
-            const_cast<psc_states*>(st)->after_mask = s == PSC_OK;
-            return s;
-        }
-        long want = ((long)B * cpr + resident - 1) / resident;
-        int seg = (int)std::min<long>(TMA_SEG, std::max<long>(TMA_NCONS, (want + TMA_NCONS - 1) / TMA_NCONS * TMA_NCONS));
-        long titems = (long)B * ((cpr + seg - 1) / seg);
-        int tgrid = (int)std::max(1L, std::min<long>(titems, resident));
-        if (dtype == PSC_BF16)
-            s = launch_pdl(k_step_tma<uint16_t>, dim3(tgrid), dim3(TMA_WARPS * 32), TmaShape<uint16_t>::SMEM, cs,
-                           "k_step_tma", (uint16_t*)d_logits, row_stride, B, V, d_bitmask_out, st->d.best, h->d,
-                           st->d, have_mid, seg);
-        else
-            s = launch_pdl(k_step_tma<uint32_t>, dim3(tgrid), dim3(TMA_WARPS * 32), TmaShape<uint32_t>::SMEM, cs,
-                           "k_step_tma", (uint32_t*)d_logits, row_stride, B, V, d_bitmask_out, st->d.best, h->d,
-                           st->d, have_mid, seg);
+    const int lead = row_lead(d_logits, dtype, row_stride, B);
+    const int cpv = (lead + V + 1023) / 1024;
+    const bool any = lead != 0 || V % 1024 != 0;
+    const long chunks = (long)B * cpv;
+    auto launch = [&](auto kernel_span, auto ahead, auto* logits) {
+        return launch_step_warp<decltype(kernel_span)::value, decltype(ahead)::value>(logits, row_stride, M, B, V, cpv, any,
+                                                                                     st->d.best, cs);
+    };
+    using One = std::integral_constant<int, 1>;
+    using Two = std::integral_constant<int, 2>;
+    using Four = std::integral_constant<int, 4>;
+    if (dtype == PSC_F32) {
+        auto* x = (uint32_t*)d_logits;
+        s = chunks <= AHEAD_CHUNKS_F32 ? launch(One{}, std::true_type{}, x) : launch(Two{}, std::false_type{}, x);
     } else {
-        // rows not 16-byte aligned: warp-per-chunk pass, 4 resident CTAs of 256 threads per SM
-        int slots = sm_count(h->device) * 4;
-        long seg = ((long)cpr * B) / (2L * slots);
-        int seg_chunks = (int)std::max(1L, std::min(32L, seg));
-        long items = (long)B * ((cpr + seg_chunks - 1) / seg_chunks);
-        int grid = (int)std::max(1L, std::min<long>(items, slots));
-        if (dtype == PSC_BF16)
-            k_apply_argmax<uint16_t, true><<<grid, 256, 0, cs>>>((uint16_t*)d_logits, row_stride, M, B, V, vec,
-                                                                  seg_chunks, st->d.best, h->d, st->d);
-        else
-            k_apply_argmax<uint32_t, true><<<grid, 256, 0, cs>>>((uint32_t*)d_logits, row_stride, M, B, V, vec,
-                                                                  seg_chunks, st->d.best, h->d, st->d);
-        s = launch_check("k_apply_argmax");
+        auto* x = (uint16_t*)d_logits;
+        s = chunks <= AHEAD_CHUNKS_BF16 ? launch(One{}, std::true_type{}, x)
+            : chunks <= SPAN4_CHUNKS    ? launch(Two{}, std::false_type{}, x)
+                                        : launch(Four{}, std::false_type{}, x);
     }
-    if (s == PSC_OK) const_cast<psc_states*>(st)->mid_gen = st->gen;
-    const_cast<psc_states*>(st)->after_mask = s == PSC_OK && vec && have_mid;
+    const_cast<psc_states*>(st)->after_mask = s == PSC_OK;
     return s;
 }
 
@@ -2745,23 +2183,6 @@ psc_status upload_tables(std::unique_ptr<psc_handle>& h, int tables) {
             return s;
         }
     }
-    // the TMA masking pass uses more than the default 48 KiB of shared memory
-    if ((s = cuda_check(cudaFuncSetAttribute(k_step_tma<uint16_t>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                             TmaShape<uint16_t>::SMEM),
-                        "cudaFuncSetAttribute(k_step_tma)")) != PSC_OK ||
-        (s = cuda_check(cudaFuncSetAttribute(k_step_tma<uint32_t>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                             TmaShape<uint32_t>::SMEM),
-                        "cudaFuncSetAttribute(k_step_tma)")) != PSC_OK ||
-        (s = cuda_check(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&h->tma_ctas[0], k_step_tma<uint16_t>,
-                                                                      TMA_WARPS * 32, TmaShape<uint16_t>::SMEM),
-                        "cudaOccupancyMaxActiveBlocksPerMultiprocessor(k_step_tma)")) != PSC_OK ||
-        (s = cuda_check(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&h->tma_ctas[1], k_step_tma<uint32_t>,
-                                                                      TMA_WARPS * 32, TmaShape<uint32_t>::SMEM),
-                        "cudaOccupancyMaxActiveBlocksPerMultiprocessor(k_step_tma)")) != PSC_OK) {
-        for (int i = 0; i < h->n_blocks; i++) cudaFree(h->blocks[i]);
-        return s;
-    }
-    for (int k = 0; k < 2; k++) h->tma_ctas[k] = std::max(1, h->tma_ctas[k]);
     d.q0 = t.q0;
     d.nq = t.nq;
     d.n_lr = t.n_lr;
@@ -2989,8 +2410,8 @@ psc_status psc_advance(const psc_handle* h, psc_states* st, const int32_t* d_tok
     psc_status s = check_device(h, "psc_advance");
     if (s != PSC_OK) return s;
     if (!st || st->h != h || B != st->d.B || !d_tokens) return fail_with(PSC_ERR_ARG, "psc_advance: bad arguments");
-    int use_mid = st->mid_gen == st->gen ? 1 : 0;
-    return launch_advance(h, st, d_tokens, use_mid, d_row_status, nullptr, (cudaStream_t)stream);
+    if ((s = ensure_mid(h, st, (cudaStream_t)stream)) != PSC_OK) return s;   // the tokens are checked against the masks
+    return launch_advance(h, st, d_tokens, d_row_status, nullptr, (cudaStream_t)stream);
 }
 
 psc_status psc_fill_mask(const psc_handle* h, const psc_states* st, int32_t B, uint32_t* d_bitmask, void* stream) {
@@ -3070,7 +2491,7 @@ psc_status psc_decode_step(const psc_handle* h, psc_states* st, int32_t B, void*
         return fail_with(PSC_ERR_ARG, "psc_decode_step: bad arguments");
     cudaStream_t cs = (cudaStream_t)stream;
     if ((s = launch_fused(h, st, d_logits, dtype, row_stride, V, d_bitmask_out, cs)) != PSC_OK) return s;
-    return launch_advance(h, st, nullptr, 1, d_row_status, d_tokens, cs);
+    return launch_advance(h, st, nullptr, d_row_status, d_tokens, cs);
 }
 
 psc_status psc_decode_step_mask(const psc_handle* h, psc_states* st, int32_t B, void* d_logits, psc_dtype dtype,
@@ -3091,7 +2512,7 @@ psc_status psc_decode_step_advance(const psc_handle* h, psc_states* st, int32_t 
         return fail_with(PSC_ERR_ARG, "psc_decode_step_advance: bad arguments");
     // the greedy keys were made for the mask ids the masking pass used (current
     // unless rows changed since): the advance checks tokens against those
-    return launch_advance(h, st, nullptr, 1, d_row_status, d_tokens, (cudaStream_t)stream);
+    return launch_advance(h, st, nullptr, d_row_status, d_tokens, (cudaStream_t)stream);
 }
 
 psc_status psc_states_download(const psc_states* st, int32_t* h_q, int32_t* h_depth, uint16_t* h_stack,
