@@ -7,7 +7,7 @@
 //              stopping at absorbing states; kept incremental by the bottom-up
 //              classifier (its state per stack prefix, so a step re-reads only
 //              the entries it changed, then one lookup by q)    -> k_advance_warp / k_classify
-//   step 4     the precomputed mask of the reached state         -> k_step_warp / k_fill / k_apply_rows
+//   step 4     the precomputed mask of the reached state         -> k_mask_rows / k_fill
 // plus applying the mask to the logits and greedy sampling over the allowed
 // tokens (left to the serving engine in the paper).
 //
@@ -33,7 +33,6 @@
 #include <mutex>
 #include <new>
 #include <string>
-#include <type_traits>
 
 #include "../../include/psc.h"
 #include "psc_internal.h"
@@ -263,29 +262,6 @@ __global__ void k_classify(DevTables T, DevStates S, int B) {
     }
 }
 
-// out[b][:] = masks[mid[b]][:]   (16-byte vector copies when W % 4 == 0)
-__global__ void k_fill(DevTables D, const int32_t* __restrict__ mid, int B, uint32_t* __restrict__ out, int vec) {
-    size_t tid = blockIdx.x * (size_t)blockDim.x + threadIdx.x;
-    size_t stride = (size_t)gridDim.x * blockDim.x;
-    int W = D.W;
-    if (vec) {
-        int W4 = W >> 2;
-        size_t total = (size_t)B * W4;
-        for (size_t i = tid; i < total; i += stride) {
-            int b = (int)(i / W4), w = (int)(i % W4);
-            uint32_t c = __ldg(D.mrows + (size_t)__ldg(mid + b) * D.nch + ((4 * w) >> 5));
-            uint4 v = ld_nc_v4(D.mchunks + (size_t)c * 32 + ((4 * w) & 31));
-            st_cs_v4(out + (size_t)b * W + 4 * w, v);
-        }
-    } else {
-        size_t total = (size_t)B * W;
-        for (size_t i = tid; i < total; i += stride) {
-            int b = (int)(i / W), w = (int)(i % W);
-            out[i] = mask_word(D, __ldg(mid + b), w);
-        }
-    }
-}
-
 template <typename T>
 struct NegInf;
 template <>
@@ -299,59 +275,8 @@ struct NegInf<uint32_t> {
     static constexpr uint32_t one = 0xFF800000u;
 };
 
-// Apply one 1024-column chunk of row b: `word` is this lane's mask word for
-// columns [col0 + 32*lane, col0 + 32*lane + 32).  E = elements per 16 bytes.
-template <typename T>
-__device__ __forceinline__ void apply_chunk(T* row, int col0, uint32_t word, int lane) {
-    constexpr int E = 16 / sizeof(T);
-    constexpr int PASSES = 1024 / E / 32;
-    constexpr uint32_t FULLBITS = (1u << E) - 1u;
-    uint4 ninf = make_uint4(NegInf<T>::pair, NegInf<T>::pair, NegInf<T>::pair, NegInf<T>::pair);
-#pragma unroll
-    for (int k = 0; k < PASSES; k++) {
-        int c = k * 32 + lane;                      // 16-byte chunk index within the 1024 columns
-        int wsrc = (c * E) >> 5;
-        int sh = (c * E) & 31;
-        uint32_t bits = (__shfl_sync(FULL, word, wsrc) >> sh) & FULLBITS;
-        // a 32-byte sector (this lane's 16 bytes and its neighbour's) is written whole or not
-        // at all, so the L2 never holds a partly written sector (read-modify-write on eviction)
-        bool keep = (bits & __shfl_xor_sync(FULL, bits, 1)) == FULLBITS;
-        T* p = row + col0 + c * E;
-        if (bits == 0) {
-            st_cs_v4(p, ninf);
-        } else if (!keep) {
-            uint4 v = *reinterpret_cast<const uint4*>(p);
-            uint32_t w[4] = {v.x, v.y, v.z, v.w};
-            if (sizeof(T) == 2) {
-#pragma unroll
-                for (int e = 0; e < 8; e++)
-                    if (!((bits >> e) & 1)) {
-                        uint32_t& x = w[e >> 1];
-                        x = (e & 1) ? ((x & 0x0000FFFFu) | 0xFF800000u) : ((x & 0xFFFF0000u) | 0x0000FF80u);
-                    }
-            } else {
-#pragma unroll
-                for (int e = 0; e < 4; e++)
-                    if (!((bits >> e) & 1)) w[e] = 0xFF800000u;
-            }
-            *reinterpret_cast<uint4*>(p) = make_uint4(w[0], w[1], w[2], w[3]);
-        }
-    }
-}
-
-// element-by-element path for ragged chunks or unaligned rows: each lane
-// handles the 32 columns of its own mask word
-template <typename T>
-__device__ __forceinline__ void apply_chunk_scalar(T* row, int col0, int ncols, uint32_t word, int lane) {
-    int c0 = 32 * lane;
-    for (int e = 0; e < 32; e++) {
-        if (c0 + e >= ncols) break;
-        if (!((word >> e) & 1)) row[col0 + c0 + e] = (T)NegInf<T>::one;
-    }
-}
-
-// Mask source for the apply kernels: a caller bitmask [B][W], or the device
-// mask table row picked by the classifier (mid[b]).
+// Mask source of the masking passes: a caller bitmask [B][W], or the device mask table
+// row picked by the classifier (mid[b]).
 struct MaskSrc {
     const uint32_t* bitmask;   // nullable
     const uint32_t* chunks;    // the device mask table (chunk ids + chunks)
@@ -359,54 +284,30 @@ struct MaskSrc {
     const int32_t* mid;
     int W, nch;
     uint32_t* copy_out;        // nullable: also write the words here ([B][W])
-    // word `lane` of 1024-column chunk j of row b (0 past W)
-    __device__ __forceinline__ uint32_t word(int b, int j, int lane) const {
-        int wi = j * 32 + lane;
-        if (wi >= W) return 0u;
-        if (bitmask) return __ldg(bitmask + (size_t)b * W + wi);
-        uint32_t c = __ldg(rows + (size_t)__ldg(mid + b) * nch + j);
-        return __ldg(chunks + (size_t)c * 32 + lane);
+    // lane l: what locates chunk j + l of row b (its id in the device mask table)
+    template <bool TABLE>
+    __device__ __forceinline__ uint32_t locate(int b, int j, int lane) const {
+        return TABLE ? __ldg(rows + (size_t)__ldcg(mid + b) * nch + min(j + lane, nch - 1)) : 0u;
     }
-    // word `lane` of chunks j .. j + SPAN - 1 of row b (0 past W) and, when BEFORE, the word
-    // before them (0 at the row's start), all through the device mask table and without
-    // branches, so that the SPAN + 1 chains of dependent loads run side by side
-    template <int SPAN, bool BEFORE>
-    __device__ __forceinline__ void table_words(int b, int j, int lane, uint32_t (&cur)[SPAN], uint32_t& before) const {
-        const uint32_t* r = rows + (size_t)__ldcg(mid + b) * nch;
-        uint32_t id[SPAN], idb = 0u;
-#pragma unroll
-        for (int i = 0; i < SPAN; i++) id[i] = __ldg(r + min(j + i, nch - 1));
-        if (BEFORE) idb = __ldg(r + min(max(j - 1, 0), nch - 1));
-#pragma unroll
-        for (int i = 0; i < SPAN; i++) cur[i] = __ldg(chunks + (size_t)id[i] * 32 + lane);
-        before = BEFORE ? __ldg(chunks + (size_t)idb * 32 + 31) : 0u;
-#pragma unroll
-        for (int i = 0; i < SPAN; i++)
-            if (j + i >= nch) cur[i] = 0u;
-        if (j == 0) before = 0u;
+    // word `lane` of chunk j of row b, id: what locates that chunk (0 past W)
+    template <bool TABLE>
+    __device__ __forceinline__ uint32_t word(int b, int j, int lane, uint32_t id) const {
+        if (TABLE) {
+            uint32_t w = __ldg(chunks + (size_t)id * 32 + lane);
+            return j < nch ? w : 0u;
+        }
+        const int wi = j * 32 + lane;
+        uint32_t w = __ldcg(bitmask + (size_t)b * W + min(wi, W - 1));
+        return wi < W ? w : 0u;
+    }
+    // the word before chunk j of row b (0 at the row's start)
+    template <bool TABLE>
+    __device__ __forceinline__ uint32_t word_before(int b, int j) const {
+        const int jb = max(j - 1, 0);
+        uint32_t w = word<TABLE>(b, jb, 31, locate<TABLE>(b, jb, 0));
+        return j == 0 ? 0u : w;
     }
 };
-
-template <typename T>
-__global__ void __launch_bounds__(256) k_apply_rows(T* logits, int64_t stride, MaskSrc M, int B, int V, int vec) {
-    int lane = threadIdx.x & 31;
-    int gw = (int)((blockIdx.x * (size_t)blockDim.x + threadIdx.x) >> 5);
-    int nw = (int)((gridDim.x * (size_t)blockDim.x) >> 5);
-    int cpr = (V + 1023) >> 10;
-    long total = (long)B * cpr;
-    for (long c = gw; c < total; c += nw) {
-        int b = (int)(c / cpr);
-        int j = (int)(c - (long)b * cpr);
-        int col0 = j << 10;
-        int wi = (col0 >> 5) + lane;
-        uint32_t word = M.word(b, j, lane);
-        if (M.copy_out && wi < M.W) M.copy_out[(size_t)b * M.W + wi] = word;
-        T* row = logits + (size_t)b * stride;
-        int ncols = V - col0;
-        if (vec && ncols >= 1024) apply_chunk<T>(row, col0, word, lane);
-        else apply_chunk_scalar<T>(row, col0, ncols < 1024 ? ncols : 1024, word, lane);
-    }
-}
 
 // Feed one lexeme class to the parser on a row's stack: resolve the class to a
 // terminal with the current top, reduce until it is shifted.  Returns a row
@@ -583,9 +484,9 @@ __device__ __forceinline__ uint32_t sel_ninf(uint32_t w, uint32_t allow, uint32_
 // for the ends of a row then fold away).
 template <typename T, bool ANY = true>
 struct RowView {
-    [[maybe_unused]] static constexpr int E = 16 / sizeof(T);         // elements per piece
-    [[maybe_unused]] static constexpr int PIECES = 1024 / E / 32;     // pieces of a chunk per lane
-    [[maybe_unused]] static constexpr uint32_t FULLBITS = (1u << E) - 1u;
+    static constexpr int E = 16 / sizeof(T);         // elements per piece
+    static constexpr int PIECES = 1024 / E / 32;     // pieces of a chunk per lane
+    static constexpr uint32_t FULLBITS = (1u << E) - 1u;
     T* org;
     int a, lo, hi, end;
     __device__ __forceinline__ RowView() {}
@@ -805,7 +706,6 @@ template <typename T>
 struct ChunkAhead {
     uint4 v[RowView<T>::PIECES];
     T edge;
-    __device__ __forceinline__ ChunkAhead() {}
     template <bool ANY>
     __device__ __forceinline__ ChunkAhead(const RowView<T, ANY>& R, int j, int lane) {
         const int x0 = (j << 10) + lane * RowView<T>::E;
@@ -820,44 +720,60 @@ struct ChunkAhead {
     }
 };
 
-// One chunk of a row: -inf where w (the chunk's view word of this lane) masks, every
-// sector that holds a masked token written whole and no other (a partly written sector
-// costs a read-modify-write when the L2 evicts it); allowed values folded into the lane's
-// best when GREEDY.  The values come from `ahead` when it is given, else only the pieces
-// that must be read are (GREEDY: those that hold an allowed token, else those of sectors
-// to be written that do), four at a time.
+// N pieces (from piece h) of a chunk of a row: -inf where w (the chunk's view word of this
+// lane) masks, every sector that holds a masked token written whole and no other (a partly
+// written sector costs a read-modify-write when the L2 evicts it); allowed values folded
+// into the lane's best when GREEDY.  EDGED: the chunk may hold elements outside the whole
+// pieces.  The values come from `ahead` when it is given, else only the pieces that must
+// be read are (GREEDY: those that hold an allowed token, else those of sectors to be
+// written that do).
+template <typename T, bool GREEDY, bool EDGED, bool ANY>
+__device__ __forceinline__ void mask_quad(const RowView<T, ANY>& R, int j, int h, uint32_t w, int lane, const uint4* lut,
+                                          const ChunkAhead<T>* ahead, Best& best) {
+    constexpr int E = RowView<T, ANY>::E;
+    constexpr uint32_t F = RowView<T, ANY>::FULLBITS, N = NegInf<T>::pair;
+    const int x0 = (j << 10) + (h * 32 + lane) * E;
+    uint32_t bits[4];
+    uint4 v[4];
+    bool store[4];
+#pragma unroll
+    for (int k = 0; k < 4; k++) {
+        bits[k] = piece_bits<T>(w, h + k, lane);
+        const bool in = !EDGED || R.whole(x0 + k * 32 * E);
+        if (!in) bits[k] = F;   // not this row's, or handled element by element: left as it is
+        store[k] = (bits[k] & __shfl_xor_sync(FULL, bits[k], 1)) != F && in;
+        if (!in) bits[k] = 0u;
+    }
+#pragma unroll
+    for (int k = 0; k < 4; k++) {
+        const bool need = bits[k] != 0u && (GREEDY || store[k]);
+        if (ahead) v[k] = ahead->v[h + k];
+        else v[k] = need ? *reinterpret_cast<const uint4*>(R.org + x0 + k * 32 * E) : make_uint4(N, N, N, N);
+    }
+#pragma unroll
+    for (int k = 0; k < 4; k++) {
+        v[k] = mask_piece<T>(v[k], bits[k], lut);
+        if (store[k]) st_cs_v4(R.org + x0 + k * 32 * E, v[k]);
+    }
+    if (GREEDY) fold_quad<T>(best, bits, v, x0 - R.a);
+}
+
+// One chunk of a row (see mask_quad).
 template <typename T, bool GREEDY, bool ANY>
 __device__ __forceinline__ void mask_chunk(const RowView<T, ANY>& R, int j, uint32_t w, int lane, const uint4* lut,
                                            const ChunkAhead<T>* ahead, Best& best) {
-    constexpr int E = RowView<T>::E, P = RowView<T>::PIECES;
-    constexpr uint32_t F = RowView<T>::FULLBITS, N = NegInf<T>::pair;
+    constexpr int P = RowView<T, ANY>::PIECES;
     const bool edged = R.edge(j);
-    const int x0 = (j << 10) + lane * E;
+    if (ahead || !edged) {
 #pragma unroll
-    for (int h = 0; h < P; h += 4) {
-        uint32_t bits[4];
-        uint4 v[4];
-        bool store[4];
-#pragma unroll
-        for (int k = 0; k < 4; k++) {
-            bits[k] = piece_bits<T>(w, h + k, lane);
-            const bool in = !edged || R.whole(x0 + (h + k) * 32 * E);
-            if (!in) bits[k] = F;   // not this row's, or handled below: left as it is
-            store[k] = (bits[k] & __shfl_xor_sync(FULL, bits[k], 1)) != F && in;
-            if (!in) bits[k] = 0u;
+        for (int h = 0; h < P; h += 4) {
+            if (ahead) mask_quad<T, GREEDY, ANY>(R, j, h, w, lane, lut, ahead, best);
+            else mask_quad<T, GREEDY, false>(R, j, h, w, lane, lut, (const ChunkAhead<T>*)nullptr, best);
         }
-#pragma unroll
-        for (int k = 0; k < 4; k++) {
-            const bool need = bits[k] != 0u && (GREEDY || store[k]);
-            if (ahead) v[k] = ahead->v[h + k];
-            else v[k] = need ? *reinterpret_cast<const uint4*>(R.org + x0 + (h + k) * 32 * E) : make_uint4(N, N, N, N);
-        }
-#pragma unroll
-        for (int k = 0; k < 4; k++) {
-            v[k] = mask_piece<T>(v[k], bits[k], lut);
-            if (store[k]) st_cs_v4(R.org + x0 + (h + k) * 32 * E, v[k]);
-        }
-        if (GREEDY) fold_quad<T>(best, bits, v, x0 + h * 32 * E - R.a);
+    } else {
+#pragma unroll 1
+        for (int h = 0; h < P; h += 4)
+            mask_quad<T, GREEDY, true>(R, j, h, w, lane, lut, (const ChunkAhead<T>*)nullptr, best);
     }
     if (edged) {   // after the pieces: a tie goes to the lower column either way
         int x = R.edge_element(j, lane);
@@ -1486,58 +1402,123 @@ __global__ void __launch_bounds__(ADV_WARPS * 32, 1)   // the staged tables leav
 }
 
 // ------------------------------------------------------------ decode masking pass
-// The masking pass: a warp takes SPAN neighbouring 1024-element chunks of a row view, eight
-// warps per CTA.  The chunks' mask words come through the row's mask id and the chunk ids
-// (three dependent loads, side by side for the chunks); then every piece that holds an
-// allowed token is read, masked, folded into the greedy choice and written back (sectors
-// with nothing masked are not written, pieces with nothing allowed are not read).  cpv:
-// chunks of the longest row view.
-//
-// Large batches are bound by DRAM: what counts is bytes in flight, so few registers (a lane
-// keeps a value and a column, not the piece) and several chunks' words per chain of
-// dependent loads.  1024 rows x 262,144 bf16 tokens, whole decode step replayed from a
-// CUDA graph: 148 us with SPAN 4, 150 with 2, 162 with 1, 172 with the TMA-pipelined pass
-// that this one replaced; x 128,256 tokens: 71 / 75 / 79 / 101 us; 512 x 151,665 (rows not
-// aligned): 65 / 69 / 76 / 385 us (element by element).  f32, 512 rows x 262,144: 150 us
-// with SPAN 2 (152 with 4, 198 with the TMA pass).
-//
-// Small batches are bound by that chain of loads: AHEAD reads all the pieces while the mask
-// word arrives (one row of 151,936 f32 tokens: 8.9 us per step instead of 10.3; one of
-// 262,144 bf16 tokens 7.3 instead of 7.7).
-template <typename T, bool ANY, int SPAN, bool AHEAD>
-__global__ void __launch_bounds__(256) k_step_warp(T* logits, int64_t stride, MaskSrc M, int B, int V, int cpv,
-                                                   unsigned long long* __restrict__ best_key) {
+// The masking pass: a warp takes `span` (at most 32) neighbouring 1024-element chunks of a
+// row view, eight warps per CTA: every piece that holds an allowed token is read, masked,
+// folded into the greedy choice and written back (sectors with nothing masked are not
+// written, pieces with nothing allowed are not read).  The next chunk's mask word is in
+// flight while this one's pieces are.  cpv: chunks of the longest row view.
+// Bound by DRAM at large batches: what counts is bytes in flight, so few registers (a lane
+// keeps a value and a column, the chunks are a rolled loop; five CTAs per SM, four with
+// the code for the ends of rows, which spills at five: 209 us instead of 168 on 1024 rows
+// x 262,145) and one chain of dependent loads (mask id, chunk ids) for all the warp's
+// chunks.  Whole decode steps replayed from a CUDA graph, before -> now (us; before: a
+// pass pipelined with bulk copies, element by element where rows are not aligned): 1024
+// rows x 262,144 bf16 172 -> 147, x 128,256 101 -> 70, x 262,145 1155 -> 158; 512 x
+// 262,144 f32 198 -> 149.  Masking alone from a caller's bitmask (before: a persistent
+// grid, mask word then logits in turn): 1024 x 262,144 bf16 147 -> 125, 256 x 262,145
+// 251 -> 43, 512 x 262,144 f32 139 -> 121.
+template <typename T, bool GREEDY, bool TABLE, bool ANY>
+__global__ void __launch_bounds__(256, ANY ? 4 : 5) k_mask_rows(T* logits, int64_t stride, MaskSrc M, int B, int V, int cpv,
+                                                   int span, unsigned long long* __restrict__ best_key) {
     __shared__ uint4 s_lut[sizeof(T) == 2 ? 256 : 1];
     if (sizeof(T) == 2) build_allow_lut<T>(s_lut);
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const unsigned c = blockIdx.x * 8u + warp;   // fewer than 2^32: a chunk takes 2 KiB of logits or a whole row
-    const unsigned spr = (unsigned)(cpv + SPAN - 1) / SPAN;
-    const int b = (int)(c / spr), j0 = (int)(c - (unsigned)b * spr) * SPAN;
+    const unsigned spr = (unsigned)(cpv + span - 1) / (unsigned)span;
+    const int b = (int)(c / spr), j0 = (int)(c - (unsigned)b * spr) * span;
     grid_dep_wait();   // logits, mask ids and greedy keys come from earlier kernels
     grid_dep_launch();
     __syncthreads();   // the allow-mask table
     if (b >= B) return;
     const RowView<T, ANY> R(logits + (size_t)b * stride, V);
-    const int n = R.chunks();
-    if (j0 >= n) return;
-    ChunkAhead<T> ahead[SPAN];
-    uint32_t cur[SPAN], before;
-#pragma unroll
-    for (int i = 0; i < SPAN; i++)
-        if (AHEAD && (SPAN == 1 || j0 + i < n)) ahead[i] = ChunkAhead<T>(R, j0 + i, lane);
-    M.template table_words<SPAN, ANY>(b, j0, lane, cur, before);
+    const int j1 = min(j0 + span, R.chunks());
+    if (j0 >= j1) return;
+    const uint32_t id = M.template locate<TABLE>(b, j0, lane);
+    uint32_t cur = M.template word<TABLE>(b, j0, lane, __shfl_sync(FULL, id, 0));
+    uint32_t before = ANY ? M.template word_before<TABLE>(b, j0) : 0u;
     Best best;
-#pragma unroll
-    for (int i = 0; i < SPAN; i++) {
-        const int j = j0 + i;
-        if (SPAN > 1 && j >= n) break;
-        if (M.copy_out && j * 32 + lane < M.W) M.copy_out[(size_t)b * M.W + j * 32 + lane] = cur[i];
-        if (i > 0) before = __shfl_sync(FULL, cur[i - 1], 31);
-        mask_chunk<T, true>(R, j, view_word(cur[i], before, R.a, lane), lane, s_lut,
-                            AHEAD ? &ahead[i] : (const ChunkAhead<T>*)nullptr, best);
+#pragma unroll 1
+    for (int j = j0; j < j1; j++) {
+        uint32_t next = 0u;
+        if (j + 1 < j1) next = M.template word<TABLE>(b, j + 1, lane, __shfl_sync(FULL, id, j + 1 - j0));
+        if (M.copy_out && j * 32 + lane < M.W) M.copy_out[(size_t)b * M.W + j * 32 + lane] = cur;
+        mask_chunk<T, GREEDY>(R, j, view_word(cur, before, R.a, lane), lane, s_lut, (const ChunkAhead<T>*)nullptr, best);
+        if (ANY) before = __shfl_sync(FULL, cur, 31);
+        cur = next;
     }
-    const unsigned long long key = warp_max_key(best_key_of(best));
-    if (lane == 0 && key) atomicMax(best_key + b, key);
+    if (GREEDY) {
+        const unsigned long long key = warp_max_key(best_key_of(best));
+        if (lane == 0 && key) atomicMax(best_key + b, key);
+    }
+}
+
+// The same for small batches, a warp per chunk: there the chain of loads (mask id, chunk
+// id, mask word, logits) is what takes the time, so all the chunk's pieces are read while
+// the mask word arrives, whatever the mask (one row of 151,936 f32 tokens: 8.9 us per
+// decode step instead of 10.3; one of 262,144 bf16 tokens 7.3 instead of 7.7).
+template <typename T, bool GREEDY, bool TABLE, bool ANY>
+__global__ void __launch_bounds__(256) k_mask_rows_ahead(T* logits, int64_t stride, MaskSrc M, int B, int V, int cpv,
+                                                         unsigned long long* __restrict__ best_key) {
+    __shared__ uint4 s_lut[sizeof(T) == 2 ? 256 : 1];
+    if (sizeof(T) == 2) build_allow_lut<T>(s_lut);
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const unsigned c = blockIdx.x * 8u + warp;
+    const int b = (int)(c / (unsigned)cpv), j = (int)(c - (unsigned)b * (unsigned)cpv);
+    grid_dep_wait();
+    grid_dep_launch();
+    __syncthreads();   // the allow-mask table
+    if (b >= B) return;
+    const RowView<T, ANY> R(logits + (size_t)b * stride, V);
+    if (j >= R.chunks()) return;
+    const ChunkAhead<T> ahead(R, j, lane);
+    const uint32_t cur = M.template word<TABLE>(b, j, lane, M.template locate<TABLE>(b, j, 0));
+    const uint32_t before = ANY ? M.template word_before<TABLE>(b, j) : 0u;
+    if (M.copy_out && j * 32 + lane < M.W) M.copy_out[(size_t)b * M.W + j * 32 + lane] = cur;
+    Best best;
+    mask_chunk<T, GREEDY>(R, j, view_word(cur, before, R.a, lane), lane, s_lut, &ahead, best);
+    if (GREEDY) {
+        const unsigned long long key = warp_max_key(best_key_of(best));
+        if (lane == 0 && key) atomicMax(best_key + b, key);
+    }
+}
+
+// out[b][:] = masks[mid[b]][:]: a warp takes FILL_SPAN neighbouring 32-word chunks of a
+// row; lane l loads chunk l's id, then the words go out 16 bytes per lane (VEC: rows of a
+// multiple of four words, 16-byte aligned) or one word per lane.  Bound by the chain mask
+// id, chunk id, words, store (1024 rows x 262,144: 9.2 us for 33.5 MB, 10.3 with a chain per
+// 16 bytes; one row 2.2 us).
+constexpr int FILL_SPAN = 16;
+template <bool VEC>
+__global__ void __launch_bounds__(256) k_fill(MaskSrc M, int B, uint32_t* __restrict__ out) {
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const unsigned c = blockIdx.x * 8u + warp, spr = (unsigned)(M.nch + FILL_SPAN - 1) / FILL_SPAN;
+    const int b = (int)(c / spr), j0 = (int)(c - (unsigned)b * spr) * FILL_SPAN;
+    grid_dep_wait();   // the mask ids come from earlier kernels
+    grid_dep_launch();
+    if (b >= B) return;
+    const int n = min(FILL_SPAN, M.nch - j0);
+    const uint32_t id = __ldg(M.rows + (size_t)__ldcg(M.mid + b) * M.nch + j0 + min(lane, n - 1));
+    uint32_t* row = out + (size_t)b * M.W;
+    if (VEC) {
+        uint4 v[FILL_SPAN / 4];
+#pragma unroll
+        for (int i = 0; i < FILL_SPAN / 4; i++) {
+            const uint32_t ci = __shfl_sync(FULL, id, i * 4 + (lane >> 3));
+            v[i] = ld_nc_v4(M.chunks + (size_t)ci * 32 + (lane & 7) * 4);
+        }
+#pragma unroll
+        for (int i = 0; i < FILL_SPAN / 4; i++) {
+            const int wi = (j0 + i * 4) * 32 + lane * 4;
+            if (wi < M.W) st_cs_v4(row + wi, v[i]);
+        }
+    } else {
+#pragma unroll 4
+        for (int i = 0; i < n; i++) {
+            const uint32_t ci = __shfl_sync(FULL, id, i);
+            const int wi = (j0 + i) * 32 + lane;
+            if (wi < M.W) row[wi] = __ldg(M.chunks + (size_t)ci * 32 + lane);
+        }
+    }
 }
 
 // A bounded wait on an mbarrier phase that nothing completes: gives up after
@@ -1612,24 +1593,6 @@ psc_status ensure_mid(const psc_handle* h, const psc_states* st, cudaStream_t s)
     psc_status r = launch_check("k_classify");
     if (r == PSC_OK) const_cast<psc_states*>(st)->mid_gen = st->gen;
     return r;
-}
-
-bool aligned16(const void* p) { return ((uintptr_t)p & 15u) == 0; }
-
-psc_status launch_apply(void* logits, psc_dtype dtype, int64_t row_stride, const MaskSrc& M, int B, int V,
-                        cudaStream_t s, int device) {
-    size_t esz = dtype == PSC_BF16 ? 2 : 4;
-    int vec = aligned16(logits) && ((row_stride * (int64_t)esz) % 16 == 0);
-    long chunks = (long)B * ((V + 1023) / 1024);
-    int threads = 256;
-    long want = (chunks + 7) / 8;
-    int blocks = (int)std::min<long>(want, (long)sm_count(device) * 8);
-    if (blocks < 1) blocks = 1;
-    if (dtype == PSC_BF16)
-        k_apply_rows<uint16_t><<<blocks, threads, 0, s>>>((uint16_t*)logits, row_stride, M, B, V, vec);
-    else
-        k_apply_rows<uint32_t><<<blocks, threads, 0, s>>>((uint32_t*)logits, row_stride, M, B, V, vec);
-    return launch_check("k_apply_rows");
 }
 
 // The most elements between a row's first element and the 32-byte boundary at or below
@@ -1717,18 +1680,37 @@ psc_status launch_advance(const psc_handle* h, psc_states* st, const int32_t* d_
     return s;
 }
 
-// k_step_warp's variant by the batch's chunks (bf16, us per step: 32 rows x 128,256, 4,032
-// chunks, 10.9 with AHEAD, 11.8 with SPAN 2; 32 rows x 262,144 16.3 / 14.5; 256 rows, 65,536 chunks, 47.1 with
-// SPAN 2, 48.5 with 4; 512 rows 84.3 / 84.5, unaligned rows 69.0 / 64.5 at 76,000 chunks.
-// f32 x 151,936: 32 rows, 4,768 chunks, 16.7 with AHEAD, 17.1 with SPAN 2; 128 rows 34.8 /
-// 33.2).
+// Up to how many chunks a batch goes to k_mask_rows_ahead (bf16, us per decode step: 32 rows
+// x 128,256, 4,032 chunks, 10.9 ahead, 11.8 not; 32 x 262,144, 8,192 chunks, 16.3 / 14.5.
+// f32 x 151,936: 32 rows, 4,768 chunks, 16.7 / 17.1; 128 rows 34.8 / 33.2), and from how
+// many on a warp takes four chunks of bf16 rows instead of two (rows with ends: 1024 x
+// 128,256 70.1 us instead of 73.6, 1024 x 262,145 158 / 169, but 64 x 128,256 masked from
+// a bitmask 6.1 / 5.7 and 256 x 128,256 20.6 / 18.7; rows of whole chunks: 1024 x 262,144
+// 148.0 / 147.5).
 constexpr long AHEAD_CHUNKS_BF16 = 4096, AHEAD_CHUNKS_F32 = 8192, SPAN4_CHUNKS = 65536;
-template <int SPAN, bool AHEAD, typename T>
-psc_status launch_step_warp(T* logits, int64_t stride, const MaskSrc& M, int B, int V, int cpv, bool any,
-                            unsigned long long* best, cudaStream_t cs) {
-    dim3 grid((unsigned)(((long)B * ((cpv + SPAN - 1) / SPAN) + 7) / 8));
-    return launch_pdl(any ? k_step_warp<T, true, SPAN, AHEAD> : k_step_warp<T, false, SPAN, AHEAD>, grid, dim3(256), 0, cs,
-                      "k_step_warp", logits, stride, M, B, V, cpv, best);
+
+template <bool GREEDY, bool TABLE, typename T>
+psc_status launch_rows(T* logits, int64_t stride, const MaskSrc& M, int B, int V, int lead, unsigned long long* best,
+                       cudaStream_t cs) {
+    const int cpv = (lead + V + 1023) / 1024;
+    const long chunks = (long)B * cpv;
+    const bool any = lead != 0 || V % 1024 != 0;
+    if (chunks <= (sizeof(T) == 2 ? AHEAD_CHUNKS_BF16 : AHEAD_CHUNKS_F32))
+        return launch_pdl(any ? k_mask_rows_ahead<T, GREEDY, TABLE, true> : k_mask_rows_ahead<T, GREEDY, TABLE, false>,
+                          dim3((unsigned)((chunks + 7) / 8)), dim3(256), 0, cs, "k_mask_rows_ahead", logits, stride, M, B,
+                          V, cpv, best);
+    const int span = std::min(sizeof(T) == 2 && any && chunks > SPAN4_CHUNKS ? 4 : 2, cpv);
+    dim3 grid((unsigned)(((long)B * ((cpv + span - 1) / span) + 7) / 8));
+    return launch_pdl(any ? k_mask_rows<T, GREEDY, TABLE, true> : k_mask_rows<T, GREEDY, TABLE, false>, grid, dim3(256), 0,
+                      cs, "k_mask_rows", logits, stride, M, B, V, cpv, span, best);
+}
+
+template <bool GREEDY, bool TABLE>
+psc_status launch_mask(void* d_logits, psc_dtype dtype, int64_t stride, const MaskSrc& M, int B, int V,
+                       unsigned long long* best, cudaStream_t cs) {
+    const int lead = row_lead(d_logits, dtype, stride, B);
+    if (dtype == PSC_F32) return launch_rows<GREEDY, TABLE>((uint32_t*)d_logits, stride, M, B, V, lead, best, cs);
+    return launch_rows<GREEDY, TABLE>((uint16_t*)d_logits, stride, M, B, V, lead, best, cs);
 }
 
 // Masking + greedy choice; leaves each row's key in st->d.best.
@@ -1738,26 +1720,7 @@ psc_status launch_fused(const psc_handle* h, const psc_states* st, void* d_logit
     psc_status s = ensure_mid(h, st, cs);
     if (s != PSC_OK) return s;
     MaskSrc M{nullptr, h->d.mchunks, h->d.mrows, st->d.mid, h->d.W, h->d.nch, d_bitmask_out};
-    const int lead = row_lead(d_logits, dtype, row_stride, B);
-    const int cpv = (lead + V + 1023) / 1024;
-    const bool any = lead != 0 || V % 1024 != 0;
-    const long chunks = (long)B * cpv;
-    auto launch = [&](auto kernel_span, auto ahead, auto* logits) {
-        return launch_step_warp<decltype(kernel_span)::value, decltype(ahead)::value>(logits, row_stride, M, B, V, cpv, any,
-                                                                                     st->d.best, cs);
-    };
-    using One = std::integral_constant<int, 1>;
-    using Two = std::integral_constant<int, 2>;
-    using Four = std::integral_constant<int, 4>;
-    if (dtype == PSC_F32) {
-        auto* x = (uint32_t*)d_logits;
-        s = chunks <= AHEAD_CHUNKS_F32 ? launch(One{}, std::true_type{}, x) : launch(Two{}, std::false_type{}, x);
-    } else {
-        auto* x = (uint16_t*)d_logits;
-        s = chunks <= AHEAD_CHUNKS_BF16 ? launch(One{}, std::true_type{}, x)
-            : chunks <= SPAN4_CHUNKS    ? launch(Two{}, std::false_type{}, x)
-                                        : launch(Four{}, std::false_type{}, x);
-    }
+    s = launch_mask<true, true>(d_logits, dtype, row_stride, M, B, V, st->d.best, cs);
     const_cast<psc_states*>(st)->after_mask = s == PSC_OK;
     return s;
 }
@@ -2420,12 +2383,10 @@ psc_status psc_fill_mask(const psc_handle* h, const psc_states* st, int32_t B, u
     if (!st || st->h != h || B != st->d.B || !d_bitmask) return fail_with(PSC_ERR_ARG, "psc_fill_mask: bad arguments");
     cudaStream_t cs = (cudaStream_t)stream;
     if ((s = ensure_mid(h, st, cs)) != PSC_OK) return s;
-    int vec = (h->d.W % 4 == 0) && aligned16(d_bitmask);
-    size_t units = vec ? (size_t)B * (h->d.W / 4) : (size_t)B * h->d.W;
-    int blocks = (int)std::min<size_t>((units + 255) / 256, (size_t)sm_count(h->device) * 8);
-    if (blocks < 1) blocks = 1;
-    k_fill<<<blocks, 256, 0, cs>>>(h->d, st->d.mid, B, d_bitmask, vec);
-    return launch_check("k_fill");
+    MaskSrc M{nullptr, h->d.mchunks, h->d.mrows, st->d.mid, h->d.W, h->d.nch, nullptr};
+    dim3 grid((unsigned)(((long)B * ((h->d.nch + FILL_SPAN - 1) / FILL_SPAN) + 7) / 8));
+    const bool vec = h->d.W % 4 == 0 && ((uintptr_t)d_bitmask & 15u) == 0;
+    return launch_pdl(vec ? k_fill<true> : k_fill<false>, grid, dim3(256), 0, cs, "k_fill", M, B, d_bitmask);
 }
 
 psc_status psc_apply_mask(void* d_logits, psc_dtype dtype, int64_t row_stride, const uint32_t* d_bitmask, int32_t B,
@@ -2433,10 +2394,8 @@ psc_status psc_apply_mask(void* d_logits, psc_dtype dtype, int64_t row_stride, c
     if (!d_logits || !d_bitmask || B < 0 || V <= 0 || row_stride < V || (dtype != PSC_F32 && dtype != PSC_BF16))
         return fail_with(PSC_ERR_ARG, "psc_apply_mask: bad arguments");
     if (B == 0) return PSC_OK;
-    int dev = 0;
-    cudaGetDevice(&dev);
     MaskSrc M{d_bitmask, nullptr, nullptr, nullptr, (V + 31) / 32, 0, nullptr};
-    return launch_apply(d_logits, dtype, row_stride, M, B, V, (cudaStream_t)stream, dev);
+    return launch_mask<false, false>(d_logits, dtype, row_stride, M, B, V, nullptr, (cudaStream_t)stream);
 }
 
 psc_status psc_fill_apply(const psc_handle* h, const psc_states* st, int32_t B, void* d_logits, psc_dtype dtype,
@@ -2449,7 +2408,7 @@ psc_status psc_fill_apply(const psc_handle* h, const psc_states* st, int32_t B, 
     cudaStream_t cs = (cudaStream_t)stream;
     if ((s = ensure_mid(h, st, cs)) != PSC_OK) return s;
     MaskSrc M{nullptr, h->d.mchunks, h->d.mrows, st->d.mid, h->d.W, h->d.nch, d_bitmask_out};
-    return launch_apply(d_logits, dtype, row_stride, M, B, V, cs, h->device);
+    return launch_mask<false, true>(d_logits, dtype, row_stride, M, B, V, nullptr, cs);
 }
 
 psc_status psc_argmax_masked(const psc_handle* h, const psc_states* st, int32_t B, const void* d_logits,
@@ -2657,7 +2616,7 @@ psc_status psc_fill_apply_noalloc(const psc_handle* h, const int32_t* d_q, const
     k_classify<<<blocks, threads, 0, cs>>>(h->d, S, B);
     if ((s = launch_check("k_classify")) != PSC_OK) return s;
     MaskSrc M{nullptr, h->d.mchunks, h->d.mrows, mid, h->d.W, h->d.nch, d_bitmask_out};
-    return launch_apply(d_logits, dtype, row_stride, M, B, V, cs, h->device);
+    return launch_mask<false, true>(d_logits, dtype, row_stride, M, B, V, nullptr, cs);
 }
 
 psc_status psc_save(const psc_handle* h, const char* path) {

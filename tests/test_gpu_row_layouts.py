@@ -135,3 +135,52 @@ def test_rows_of_any_layout(psc, batches, V, dtype):
             if call != "apply_mask":
                 np.testing.assert_array_equal(tok.cpu().numpy(), greedy, err_msg=f"{call} {off} {ld}")
                 np.testing.assert_array_equal(out.cpu().numpy(), bm.cpu().numpy(), err_msg=f"{call} {off} {ld}")
+
+
+@pytest.mark.parametrize("V,rows,dtype", [(2055, 36000, torch.bfloat16), (9001, 8000, torch.bfloat16),
+                                          (9001, 600, torch.bfloat16), (9001, 1000, torch.float32)])
+def test_large_batches_of_odd_rows(psc, batches, V, rows, dtype):
+    """The variants that take several chunks per warp (chosen by the batch's chunks): the six rows
+    above over and over, contiguous and at an odd offset."""
+    h, st6, allowed6 = batches[V]
+    st = psc.psc_state_init(h, rows, 16)
+    back = psc.psc_states_download(st6)
+    toks = _vocabulary(V)
+    first = torch.tensor([-1] + [toks.index(t) for t in (b"[", b"[", b"1", b"1", b"]")], dtype=torch.int32)
+    then = torch.tensor([-1, -1, toks.index(b'"'), -1, V - 1, -1], dtype=torch.int32)
+    for t in (first, then):
+        psc.psc_advance(h, st, t.repeat(rows // B + 1)[:rows].cuda())
+    got = psc.psc_states_download(st)
+    for k in ("q", "depth", "status"):
+        np.testing.assert_array_equal(got[k][:B], back[k])
+    allowed = torch.from_numpy(allowed6).cuda().repeat(rows // B + 1, 1)[:rows]
+    bits = torch.int16 if dtype == torch.bfloat16 else torch.int32
+    for off in (0, 5):
+        gen = torch.Generator(device="cuda").manual_seed(V + off)
+        x = torch.randn(rows, V, generator=gen, device="cuda", dtype=dtype)
+        want = torch.where(allowed, x, torch.tensor(float("-inf"), dtype=dtype, device="cuda"))
+        greedy = torch.where(allowed.any(1), want.float().argmax(1), -1)
+        top = want.float().amax(1, keepdim=True)
+        first_top = (want.float() == top).int().argmax(1)      # torch's argmax may return any of a tie
+        greedy = torch.where(greedy >= 0, first_top, greedy).int()
+        bm = torch.zeros(rows, h.W, dtype=torch.int32, device="cuda")
+        psc.psc_fill_mask(h, st, bm)
+        word = bm[:, torch.arange(V, device="cuda") // 32] >> (torch.arange(V, device="cuda") % 32)
+        assert torch.equal((word & 1).bool(), allowed)
+        for call in ("fill_apply", "apply_mask", "fill_apply_argmax"):
+            base = torch.full((off + rows * V + 64,), SENTINEL, dtype=dtype, device="cuda")
+            lg = base[off:off + rows * V].view(rows, V)
+            lg.copy_(x)
+            tok = torch.full((rows,), -7, dtype=torch.int32, device="cuda")
+            out = torch.full((rows, h.W), -1, dtype=torch.int32, device="cuda")
+            if call == "fill_apply":
+                psc.psc_fill_apply(h, st, lg, out)
+                psc.psc_argmax_masked(h, st, lg, tok)
+            elif call == "apply_mask":
+                psc.psc_apply_mask(lg, bm, rows, V)
+            else:
+                psc.psc_fill_apply_argmax(h, st, lg, tok, out)
+            assert torch.equal(lg.view(bits), want.view(bits)), (call, off)
+            assert (base[:off] == SENTINEL).all() and (base[off + rows * V:] == SENTINEL).all(), (call, off)
+            if call != "apply_mask":
+                assert torch.equal(tok, greedy) and torch.equal(out, bm), (call, off)
