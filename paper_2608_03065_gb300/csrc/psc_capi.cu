@@ -15,7 +15,8 @@
 //   dfa      int32 [S][n_lr]      next classifier state, or -(mask+1) when absorbing
 //   mrows    uint32 [n_masks][nch] mask rows as ids of 1024-token chunks (nch = ceil(W / 32))
 //   mchunks  uint32 [n_chunks][32] the distinct chunks (words past W zero)
-//   bu       int32 [...]          bottom-up classifier blocks [final row, next block per edge slot]
+//   bu       int2 [...]           bottom-up classifier blocks [(final row, -), then per edge slot (next
+//                                 block, its final row)]
 //   bu_slot  int16 [n_lr][n_lr]   slot of the LR edge t -> u among t's successors, -1 none
 //   bu_F     int32 [n_frow][nq]   mask id per final row and lexer state
 //   stacks   uint16 [B][cap]      parser stacks, bottom first; depth[b] entries used
@@ -70,12 +71,13 @@ struct DevTables {
     const uint32_t* mrows;     // mask rows as chunk ids [n_masks][nch]
     const uint8_t* vocab;
     const int64_t* vocab_off;
-    const uint8_t* tok32;      // [V][32] the first 32 bytes of every token (zero-padded)
+    const uint8_t* tok32;      // [V][32] tokens of up to 31 bytes: the bytes, zeros, the length in the last one;
+                               // longer ones: their first 31 bytes, then 255
     int q0, nq, n_lr, n_terms, n_nts, end_term;
     int V, W, nch, eos_id, n_masks;
     // compact lexer/parser tables for k_advance_warp (adv_bytes = 0: not built)
     const uint8_t* adv;
-    int adv_bytes, o_bc, o_trans, o_accept, o_ign, o_resolve, o_action, o_go, o_rlen, o_rlhs, nbc;
+    int adv_bytes, o_bc, o_trans, o_accept, o_resolve, o_action, o_go, o_rlen, o_rlhs, nbc;
     int adv_packed;   // reduce entries of the compact ACTION hold (rule length << 10 | lhs) instead of the rule
     // packed (row-displaced) parser tables, for grammars whose dense compact tables do not
     // fit in shared memory: ACTION and GOTO each as a table of uint32 entries (row id << 16
@@ -84,7 +86,7 @@ struct DevTables {
     // classes resolved through candidate terminal lists
     int adv_comb, o_cand, o_abase, o_gbase, o_acmb, o_gcmb, kc;
     // bottom-up classifier (bu = nullptr: not built; the root block, for the stack [0], is at 0)
-    const int32_t* bu;        // blocks [final row, next block per successor slot]
+    const int2* bu;           // blocks [(final row, -), per successor slot (next block, its final row)]
     const int16_t* bu_slot;   // [n_lr][n_lr] slot of the LR edge t -> u, -1 none
     const int32_t* bu_F;      // [n_frow][nq] mask ids
     int bu_len, n_frow;
@@ -119,6 +121,8 @@ struct psc_states {
     const psc_handle* h = nullptr;
     DevStates d{};
     int device = -1;
+    uint8_t* base = nullptr; // the allocation of all the arrays of d
+    size_t copy_bytes = 0;   // what psc_state_copy copies of it (all but the fault word)
     uint64_t gen = 1;        // bumped by every call that changes the rows
     uint64_t mid_gen = 0;    // generation the mask ids in d.mid were computed for
     bool after_mask = false; // the last work enqueued on these states is the masking pass with the
@@ -157,11 +161,11 @@ __device__ __forceinline__ uint32_t mask_word(const DevTables& T, int mid, int w
 }
 
 // Mask id of a configuration from the bottom-up classifier's block e for its
-// whole stack (final table row, then the lexer state's column); -1 when e is
-// not a usable block (the caller walks the stack instead).
-__device__ __forceinline__ int memo_mask(const DevTables& T, int e, int q) {
+// whole stack (its final table row fr, when the caller has it, else -1; then the lexer
+// state's column); -1 when e is not a usable block (the caller walks the stack instead).
+__device__ __forceinline__ int memo_mask(const DevTables& T, int e, int fr, int q) {
     if (e < 0 || e >= T.bu_len) return -1;
-    int fr = __ldg(T.bu + e);
+    if (fr < 0) fr = __ldg(T.bu + e).x;
     if (fr < 0 || fr >= T.n_frow) return -1;
     return __ldg(T.bu_F + (size_t)fr * T.nq + q);
 }
@@ -169,7 +173,7 @@ __device__ __forceinline__ int memo_mask(const DevTables& T, int e, int q) {
 // The row's mask id from its kept bottom-up state, or -1 (not kept / not built).
 __device__ __forceinline__ int memo_classify(const DevTables& T, const DevStates& S, int b, int q, int depth) {
     if (!S.rmemo || !T.bu) return -1;
-    return memo_mask(T, S.rmemo[(size_t)b * S.cap + depth - 1], q);
+    return memo_mask(T, S.rmemo[(size_t)b * S.cap + depth - 1], -1, q);
 }
 
 // One classifier transition in the sparse layout by a full warp (every lane with
@@ -354,7 +358,7 @@ __device__ int memo_extend(const DevTables& T, const uint16_t* st, int32_t* memo
     for (int i = from; i < depth; i++) {
         int t = st[i - 1], u = st[i];
         int k = t < T.n_lr && u < T.n_lr ? T.bu_slot[(size_t)t * T.n_lr + u] : -1;
-        e = e >= 0 && k >= 0 && e + 1 + k < T.bu_len ? __ldg(T.bu + e + 1 + k) : -1;
+        e = e >= 0 && k >= 0 && e + 1 + k < T.bu_len ? __ldg(T.bu + e + 1 + k).x : -1;
         memo[i] = e;
     }
     return e;
@@ -819,27 +823,13 @@ __device__ __forceinline__ uint64_t gmem_addr(const void* p) {
     return static_cast<uint64_t>(__cvta_generic_to_global(p));
 }
 
-// psc_state_copy: every array of one batch's states into another's in one launch,
-// once the previous kernel on the stream has completed (16-byte copies; a
-// segment's bytes past its last whole 16 one by one; every segment starts on an
-// allocation of its own, so 16-byte aligned).
-struct CopySegs {
-    const uint8_t* src[8];
-    uint8_t* dst[8];
-    unsigned long long bytes[8];
-    int n;
-};
-__global__ void k_state_copy(CopySegs c) {
+// psc_state_copy: one batch's arrays into another's (they lie in one allocation, n16
+// pieces of 16 bytes), once the previous kernel on the stream has completed.
+__global__ void k_state_copy(const uint4* __restrict__ src, uint4* __restrict__ dst, size_t n16) {
     grid_dep_wait();
     grid_dep_launch();
     const size_t tid = blockIdx.x * (size_t)blockDim.x + threadIdx.x, nt = (size_t)gridDim.x * blockDim.x;
-    for (int k = 0; k < c.n; k++) {
-        const size_t n16 = c.bytes[k] / 16;
-        const uint4* src = reinterpret_cast<const uint4*>(c.src[k]);
-        uint4* dst = reinterpret_cast<uint4*>(c.dst[k]);
-        for (size_t i = tid; i < n16; i += nt) dst[i] = src[i];
-        for (size_t i = n16 * 16 + tid; i < c.bytes[k]; i += nt) c.dst[k][i] = c.src[k][i];
-    }
+    for (size_t i = tid; i < n16; i += nt) dst[i] = src[i];
 }
 
 // Bounded wait on phase 0 of an mbarrier; returns false if it did not complete.
@@ -904,12 +894,12 @@ struct StackView {
 // Shared-window addresses of the compact lexer/parser tables staged by
 // k_advance_warp, and their row strides in bytes.
 struct AdvTabs {
-    uint32_t bc, trans, acc, ign, res, act, go, rlen, rlhs;
+    uint32_t bc, trans, acc, res, act, go, rlen, rlhs;
     uint32_t trans_row, res_row, act_row, go_row;   // bytes per row: nbc, n_lr, n_terms, n_nts int16 entries
     uint32_t cand, abase, gbase, acmb, gcmb;       // packed layout
     int q0, kc;
     __device__ __forceinline__ AdvTabs(uint32_t sb, const DevTables& T)
-        : bc(sb + T.o_bc), trans(sb + T.o_trans), acc(sb + T.o_accept), ign(sb + T.o_ign), res(sb + T.o_resolve),
+        : bc(sb + T.o_bc), trans(sb + T.o_trans), acc(sb + T.o_accept), res(sb + T.o_resolve),
           act(sb + T.o_action), go(sb + T.o_go), rlen(sb + T.o_rlen), rlhs(sb + T.o_rlhs),
           trans_row(2u * T.nbc), res_row(2u * T.n_lr), act_row(2u * T.n_terms), go_row(2u * T.n_nts),
           cand(sb + T.o_cand), abase(sb + T.o_abase), gbase(sb + T.o_gbase), acmb(sb + T.o_acmb),
@@ -1081,6 +1071,11 @@ __device__ __forceinline__ int ld_keep(const int32_t* p, uint64_t pol) {
     asm volatile("ld.global.nc.L2::cache_hint.b32 %0, [%1], %2;" : "=r"(v) : "l"(p), "l"(pol));
     return v;
 }
+__device__ __forceinline__ int2 ld_keep2(const int2* p, uint64_t pol) {
+    int2 v;
+    asm volatile("ld.global.nc.L2::cache_hint.v2.b32 {%0, %1}, [%2], %3;" : "=r"(v.x), "=r"(v.y) : "l"(p), "l"(pol));
+    return v;
+}
 __device__ __forceinline__ int warp_walk(const DevTables& T, const StackView& sv, int q, int depth, int lane) {
     if (q < 0 || q >= T.nq || depth < 1) return 0;
     uint64_t pol;
@@ -1102,32 +1097,41 @@ __device__ __forceinline__ int warp_walk(const DevTables& T, const StackView& sv
     return state_mask(T, s);
 }
 
+// Edge slot of stack entry i (from the one below it); -1: not an entry with one below, or
+// not an LR edge.
+__device__ __forceinline__ int edge_slot(const DevTables& T, const StackView& sv, int i, int depth) {
+    if (i < 1 || i >= depth) return -1;
+    int t = sv.get(i - 1), u = sv.get(i);
+    return t < T.n_lr && u < T.n_lr ? __ldg(T.bu_slot + (size_t)t * T.n_lr + u) : -1;
+}
+
 // memo_extend by a full warp: lanes fetch the edge slots of 32 entries at a
 // time, the chain of block loads follows them (broadcast by shuffles), and each
 // lane stores the block of its own entry.  e_below = block of stack [0, from-1]
-// (ignored when from == 0).  Every lane returns the block of the whole stack.
+// (ignored when from == 0); k = this lane's edge slot of the first 32 entries,
+// from max(from, 1) on.  Every lane returns the block of the whole stack; fr becomes its
+// final row when an entry was read (it comes with the block).
 __device__ __forceinline__ int warp_memo_extend(const DevTables& T, const StackView& sv, int32_t* memo, int from,
-                                                int depth, int e_below, int lane) {
+                                                int depth, int e_below, int k, int lane, int& fr) {
     uint64_t pol;
     asm volatile("createpolicy.fractional.L2::evict_last.b64 %0, 1.0;" : "=l"(pol));
     int e = e_below;
     if (from <= 0) {
         e = sv.get(0) == 0 ? 0 : -1;
+        fr = -1;
         if (lane == 0) memo[0] = e;
         from = 1;
     }
     for (int i0 = from; i0 < depth; i0 += 32) {
         int i = i0 + lane;
-        int k = -1;
-        if (i < depth) {
-            int t = sv.get(i - 1), u = sv.get(i);
-            k = t < T.n_lr && u < T.n_lr ? __ldg(T.bu_slot + (size_t)t * T.n_lr + u) : -1;
-        }
+        if (i0 > from) k = edge_slot(T, sv, i, depth);
         int n = depth - i0 < 32 ? depth - i0 : 32;
         int mine = -1;
         for (int j = 0; j < n; j++) {
             int kj = __shfl_sync(FULL, k, j);
-            e = e >= 0 && kj >= 0 && e + 1 + kj < T.bu_len ? ld_keep(T.bu + e + 1 + kj, pol) : -1;
+            int2 nx = e >= 0 && kj >= 0 && e + 1 + kj < T.bu_len ? ld_keep2(T.bu + e + 1 + kj, pol) : make_int2(-1, -1);
+            e = nx.x;
+            fr = nx.y;
             mine = lane == j ? e : mine;
         }
         if (i < depth) memo[i] = mine;
@@ -1136,10 +1140,18 @@ __device__ __forceinline__ int warp_memo_extend(const DevTables& T, const StackV
 }
 
 // Algorithm 2 steps 1-3 for one row per warp: consume the row's token (the
-// given one, or the greedy choice of the fused masking pass when from_keys),
-// then classify the new configuration into S.mid.  Everything that needs only
-// global memory (the row's state, its mask word, the token's bytes, the stack
-// window) is loaded while the tables are still being staged.
+// given one, or the greedy choice of the masking pass when from_keys),
+// then classify the new configuration into S.mid.
+// Bound by the slowest row's chain of dependent steps (clock reads in a copy of the
+// kernel, cycles after the wait for the previous kernel, 64 rows of the Java-sized
+// grammar, tokens given: 14,300 before, 11,700 now; one row of the C-like grammar after a
+// masking pass 8,500 / 7,500): the row's state and token in one round trip, the token's
+// record (bytes and length), mask chunk and stack window in the next (2,100-3,900 before,
+// when the window took a trip per 32 entries and the mask word was waited for; 1,600-2,600
+// now), lexing (two dependent shared reads and a divergent branch per byte before, one read
+// now), parsing (up to 5,000), edge slots and blocks of the entries written (loads in
+// flight during the write-back), the mask id (two loads before, one now: a block's final
+// row comes with the block).
 // early: the row's state (lexer state, depth, status, mask id, stack window, kept
 // bottom-up blocks) is read before waiting for the previous kernel.  Only the greedy
 // keys come from that kernel (the masking pass), and the masking pass lets this
@@ -1153,7 +1165,6 @@ __global__ void __launch_bounds__(ADV_WARPS * 32, 1)   // the staged tables leav
                                                                  int from_keys, int32_t* tokens_out, int early) {
     extern __shared__ uint4 smem4[];
     __shared__ __align__(8) uint64_t bar;
-    __shared__ uint8_t tokc[ADV_WARPS][32];     // the lexer byte classes of each row's token (first 32 bytes)
     __shared__ uint16_t lexcls[ADV_WARPS][32];  // the lexeme classes the token emits (tokens up to 32 bytes)
     uint8_t* sm = reinterpret_cast<uint8_t*>(smem4);
     // one TMA bulk copy stages the compact tables (16-byte aligned, multiple of 16 bytes)
@@ -1167,6 +1178,7 @@ __global__ void __launch_bounds__(ADV_WARPS * 32, 1)   // the staged tables leav
                      : "memory");
     }
     grid_dep_launch();
+    __syncthreads();   // the mbarrier; before the wait, so that no row waits for another row's loads
     int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     int b = blockIdx.x * ADV_WARPS + warp;
     bool active = b < B;   // warp-uniform
@@ -1177,71 +1189,83 @@ __global__ void __launch_bounds__(ADV_WARPS * 32, 1)   // the staged tables leav
     bool parse = false;
     int32_t* memo = active && S.rmemo && T.bu ? S.rmemo + (size_t)b * S.cap : nullptr;
     int memo_top = -1, depth0 = 0;
-    uint32_t mword = 0;
-    int tbyte = 0;   // lane i: byte i of the token (first 32 bytes)
-    int len = 0;
-    int64_t vlo = 0;
+    uint32_t mchunk = 0;   // the mask chunk that holds the token's bit
+    bool eos = false;
+    int tbyte = 0;   // lane i: byte i of the token (lane 31: its length)
     int cur_mid = 0;   // the mask the row's token is checked against
     bool live = false;
-    // the row's state and the window of its stack top (for the parse and for the
-    // classifier walk after it); read from L2 (an SM's L1 may still hold these lines
-    // from an earlier kernel)
+    // the row's state, then the window of its stack top (for the parse and for the
+    // classifier walk after it) and the kept bottom-up blocks of the top 32 prefixes; read
+    // from L2 (an SM's L1 may still hold these lines from an earlier kernel)
     auto load_row = [&]() {
         q = __ldcg(S.q + b);
         depth = __ldcg(S.depth + b);
-        depth0 = depth;
         status = __ldcg(S.status + b);
         cur_mid = __ldcg(S.mid + b);
+    };
+    const bool vec = S.cap % 8 == 0;   // rows of whole 16-byte pieces (their allocation is aligned)
+    uint4 wv = make_uint4(0u, 0u, 0u, 0u);
+    auto load_window = [&]() {   // issues the loads; place_window waits for them
+        depth0 = depth;
         live = status == ROW_OK && depth >= 1 && depth <= S.cap;
-        if (live) {
-            sv.base = depth > ADV_KEEP ? depth - ADV_KEEP : 0;
+        if (!live) return;
+        sv.base = depth > ADV_KEEP ? (depth - ADV_KEEP + 7) & ~7 : 0;
+        if (vec && lane * 8 < depth - sv.base) wv = __ldcg(reinterpret_cast<const uint4*>(sv.st + sv.base) + lane);
+        if (memo && depth - 1 - lane >= 0) memo_top = __ldcg(memo + depth - 1 - lane);   // lane l: stack [0, depth-1-l]
+    };
+    auto place_window = [&]() {
+        if (!live) return;
+        if (vec) {
+            if (lane * 8 < depth - sv.base) *(reinterpret_cast<uint4*>(sv.win) + lane) = wv;
+        } else {
             for (int i = lane; i < depth - sv.base; i += 32) sv.win[i] = __ldcg(sv.st + sv.base + i);
-            // the kept bottom-up blocks of the top 32 prefixes (lane l: stack [0, depth-1-l])
-            if (memo && depth - 1 - lane >= 0) memo_top = __ldcg(memo + depth - 1 - lane);
         }
     };
-    if (active && early) load_row();
+    if (active && early) {
+        load_row();
+        load_window();
+        place_window();
+    }
     grid_dep_wait();   // the greedy keys (and, unless early, the rows) come from the previous kernel
     if (active) {
+        // one round trip for the token and the row's state, the next for the token's bytes,
+        // the mask's chunk id and the window
+        unsigned long long key = 0ull;
+        if (from_keys) key = __ldcg(S.best + b);   // the greedy choice of the masking pass
+        else tok = tokens[b];
         if (!early) load_row();
-        if (from_keys) {   // the greedy choice of the fused masking pass
-            unsigned long long k = S.best[b];
-            tok = k ? (int32_t)(~(uint32_t)(k & 0xFFFFFFFFu)) : -1;
-            __syncwarp();
-            if (lane == 0) {
-                S.best[b] = 0ull;
-                tokens_out[b] = tok;
-            }
-        } else {
-            tok = tokens[b];
+        if (from_keys) tok = key ? (int32_t)(~(uint32_t)(key & 0xFFFFFFFFu)) : -1;
+        const bool known = tok >= 0 && tok < T.V;
+        if (known) tbyte = T.tok32[(size_t)tok * 32 + lane];   // lane i holds byte i, lane 31 the length
+        if (!early) load_window();
+        if (known && status == ROW_OK) mchunk = __ldg(T.mrows + (size_t)cur_mid * T.nch + (tok >> 10));
+        if (!early) place_window();
+        __syncwarp();   // every lane has read the key
+        if (from_keys && lane == 0) {
+            S.best[b] = 0ull;
+            tokens_out[b] = tok;
         }
         if (tok >= 0) {
             if (status == ROW_DONE) {
                 status = tok == T.eos_id ? ROW_DONE : ROW_REJECTED;
             } else if (status == ROW_OK) {
-                if (tok >= T.V) {
-                    status = ROW_REJECTED;
-                } else {
-                    // the token's mask bit (in flight while the token is parsed); the row is
-                    // only committed (q, depth) when it is set
-                    mword = mask_word(T, cur_mid, tok >> 5);
-                    if (tok == T.eos_id) status = ((mword >> (tok & 31)) & 1) ? ROW_DONE : ROW_REJECTED;
-                    else if (!live) status = ROW_REJECTED;
-                    else parse = true;
-                }
+                if (!known) status = ROW_REJECTED;
+                else if (tok == T.eos_id) eos = true;
+                else if (!live) status = ROW_REJECTED;
+                else parse = true;
             }
         }
-        if (parse) {   // the token's bytes: lane i holds byte i (loaded with the length, in parallel)
-            tbyte = T.tok32[(size_t)tok * 32 + lane];
-            vlo = T.vocab_off[tok];
-            len = (int)(T.vocab_off[tok + 1] - vlo);
-        }
     }
-    __syncthreads();
+    // the token's mask word (in flight while the token is parsed); the row is only
+    // committed (q, depth) when the token's bit is set
+    // (chunk 0 when there is no such token: loads without a condition, so that nothing waits
+    // for them here)
+    const uint32_t mword = __ldg(T.mchunks + (size_t)mchunk * 32 + ((tok >> 5) & 31));
+    // the final row of the stack as it is (used when the token writes no stack entry)
+    const int e_top = __shfl_sync(FULL, memo_top, 0);
+    int fr_top = -1;
+    if (memo) fr_top = __ldg(T.bu + min(max(e_top, 0), T.bu_len - 1)).x;
     bool staged = __all_sync(FULL, mbar_wait0(bar_a, 1 << 24));
-    // the tables are in: each lane turns its byte into a lexer byte class
-    if (staged && active && parse && lane < len) tokc[warp][lane] = sm[T.o_bc + tbyte];
-    __syncwarp();
     if (!staged) {
         // the copy did not land: give the rows a LIMIT status, wait (bounded) for the copy, return
         if (threadIdx.x == 0) {
@@ -1261,66 +1285,64 @@ __global__ void __launch_bounds__(ADV_WARPS * 32, 1)   // the staged tables leav
     if (parse) {
         const AdvTabs A(smem_addr(sm), T);
         int nq = q, nd = depth;
-        const uint32_t ca = smem_addr(&tokc[warp][0]);
         const uint32_t la = smem_addr(&lexcls[warp][0]);
-        int ncls = -1;   // classes in lexcls; -1: the token is lexed by lane 0 (longer than 32 bytes)
-        if (len <= 32) {
+        const int len = __shfl_sync(FULL, tbyte, 31);
+        int ncls = -1;   // classes in lexcls; -1: the token is lexed by lane 0 (longer than 31 bytes)
+        if (len <= 31) {
             // Lexing in parallel (the lexer does not depend on the parser): lane j runs the
-            // lexer DFA over the lexeme that starts afresh at byte j, lane 0 over the
-            // continuation of the row's pending lexeme; each records where its lexeme
-            // ends (the byte it cannot take, or the end of the token) and the DFA state
-            // there.  Then the lexemes are followed from one end to the next.
-            int ls = lane == 0 ? q : A.q0;
-            int le = lane;
-            int pre = -2;   // class of the pending lexeme when the token's first byte ends it
-            auto run = [&]() {
-                while (le < len) {
-                    int nx = lds_s16(A.trans + ls * A.trans_row + 2u * lds_u8(ca + le));
-                    if (nx < 0) break;
-                    ls = nx;
-                    le++;
+            // lexer DFA over the lexeme that starts afresh at byte j (ls, ending at le), every
+            // lane over the row's pending lexeme from the first byte on (ps, ending at pe); an
+            // end is the byte that a lexeme cannot take, or the token's.  The lanes go in
+            // step, the bytes' classes coming by shuffles, so a byte costs one dependent
+            // shared-memory read (a lane that has stopped, or a position past the token,
+            // reads on without effect).
+            const int cls_of = lds_u8(A.bc + tbyte);   // lane i: the class of byte i
+            int ls = A.q0, le = lane, ps = q, pe = 0;
+            bool run = lane < len, prun = len > 0;
+            for (int k = 0; k < len; k += 4) {
+                int c[4], pc[4];
+#pragma unroll
+                for (int i = 0; i < 4; i++) {
+                    c[i] = __shfl_down_sync(FULL, cls_of, k + i);
+                    pc[i] = __shfl_sync(FULL, cls_of, k + i);
                 }
+#pragma unroll
+                for (int i = 0; i < 4; i++) {
+                    int nx = lds_s16(A.trans + ls * A.trans_row + 2u * c[i]);
+                    int px = lds_s16(A.trans + ps * A.trans_row + 2u * pc[i]);
+                    run = run && nx >= 0 && lane + k + i < len;
+                    prun = prun && px >= 0 && k + i < len;
+                    ls = run ? nx : ls;
+                    le += run ? 1 : 0;
+                    ps = prun ? px : ps;
+                    pe += prun ? 1 : 0;
+                }
+            }
+            // each lane's lexeme: its end, whether it is ignored, ends the token, or is none
+            // (no byte taken, or incomplete), and its class; then the lexemes are followed
+            // from one end to the next, the pending one first
+            constexpr uint32_t IGN = 64u, LAST = 128u, NONE = 256u;
+            auto lexeme_of = [&](int state, int end, bool some) -> uint32_t {
+                int a = lds_s16(A.acc + 2u * state);
+                return (uint32_t)end | (end == len ? LAST : a < 0 || !some ? NONE : 0u) | (a & 1 ? IGN : 0u) |
+                       (uint32_t)(a >> 1) << 16;
             };
-            if (lane < len) {
-                run();
-                if (lane == 0 && le == 0 && q != A.q0) {
-                    pre = lds_s16(A.acc + 2u * q);
-                    ls = A.q0;
-                    run();
-                }
-            }
-            pre = __shfl_sync(FULL, pre, 0);
-            ncls = 0;
-            if (pre != -2) {
-                if (pre < 0) {
-                    status = ROW_REJECTED;
-                } else if (!lds_u8(A.ign + pre)) {
-                    if (lane == 0) sts_u16(la, pre);
-                    ncls = 1;
-                }
-            }
+            const uint32_t fresh = lexeme_of(ls, le, le > lane);
+            uint32_t lx = q == A.q0 ? __shfl_sync(FULL, fresh, 0) : lexeme_of(ps, pe, true);
             int pos = 0;
-            while (status == ROW_OK) {   // warp-uniform: pos and the lexeme ends come by shuffles
-                int ep = __shfl_sync(FULL, le, pos), sp = __shfl_sync(FULL, ls, pos);
-                if (ep == len) {   // the last lexeme stays pending
-                    nq = sp;
-                    break;
-                }
-                if (ep == pos) {   // the byte at pos starts no lexeme
-                    status = ROW_REJECTED;
-                    break;
-                }
-                int cls = sp == A.q0 ? -1 : lds_s16(A.acc + 2u * sp);
-                if (cls < 0) {
-                    status = ROW_REJECTED;
-                    break;
-                }
-                if (!lds_u8(A.ign + cls)) {
-                    if (lane == 0) sts_u16(la + 2u * ncls, cls);
+            bool pending = q != A.q0;
+            ncls = 0;
+            while (!(lx & (LAST | NONE))) {   // warp-uniform
+                if (!(lx & IGN)) {
+                    if (lane == 0) sts_u16(la + 2u * ncls, (int)(lx >> 16));
                     ncls++;
                 }
-                pos = ep;
+                pos = (int)(lx & 63u);
+                pending = false;
+                lx = __shfl_sync(FULL, fresh, pos);
             }
+            if (lx & LAST) nq = pending ? ps : __shfl_sync(FULL, ls, pos & 31);   // the last lexeme stays pending
+            else status = ROW_REJECTED;
         }
         __syncwarp();
         if (lane == 0) {
@@ -1338,17 +1360,17 @@ __global__ void __launch_bounds__(ADV_WARPS * 32, 1)   // the staged tables leav
                         nq = nx;
                         return;
                     }
-                    int cls = nq == A.q0 ? -1 : lds_s16(A.acc + 2u * nq);
-                    if (cls < 0) {
+                    int a = lds_s16(A.acc + 2u * nq);
+                    if (a < 0) {
                         status = ROW_REJECTED;
                         return;
                     }
-                    if (!lds_u8(A.ign + cls)) status = feed_class<PACKED, COMB>(A, sv, nd, top, below, S.cap, cls);
+                    if (!(a & 1)) status = feed_class<PACKED, COMB>(A, sv, nd, top, below, S.cap, a >> 1);
                     nq = lds_s16(A.trans + A.q0 * A.trans_row + 2u * c);
                     if (nq < 0) status = ROW_REJECTED;
                 };
-                for (int i = 0; i < 32 && status == ROW_OK; i++) lex(lds_u8(ca + i));
-                for (int i = 32; i < len && status == ROW_OK; i++) lex(lds_u8(A.bc + T.vocab[vlo + i]));
+                for (int64_t i = T.vocab_off[tok]; i < T.vocab_off[tok + 1] && status == ROW_OK; i++)
+                    lex(lds_u8(A.bc + T.vocab[i]));
             }
             if (!((mword >> (tok & 31)) & 1)) status = ROW_REJECTED;
             if (status == ROW_OK) {
@@ -1361,14 +1383,20 @@ __global__ void __launch_bounds__(ADV_WARPS * 32, 1)   // the staged tables leav
         depth = __shfl_sync(FULL, nd, 0);
         sv.lo = __shfl_sync(FULL, sv.lo, 0);
         __syncwarp();
-        if (status == ROW_OK) {
-            // window entries from the lowest one written up to the new depth (lo stays
-            // INT_MAX when nothing was written: clamp before adding the lane)
-            int hi = depth < sv.base + ADV_WIN ? depth : sv.base + ADV_WIN;
-            int from = sv.lo > sv.base ? sv.lo : sv.base;
-            from = from < hi ? from : hi;
-            for (int i = from + lane; i < hi; i += 32) sv.st[i] = sv.win[i - sv.base];
-        }
+    }
+    if (eos) status = ((mword >> (tok & 31)) & 1) ? ROW_DONE : ROW_REJECTED;   // here, not before: it waits for mword
+    // the lowest stack entry written (depth: none), and the edge slots of the entries from
+    // there on, in flight while the stack is written back
+    const int from = parse && sv.lo < depth ? sv.lo : depth;
+    const bool ok = status == ROW_OK && depth >= 1 && depth <= S.cap;
+    const int slot = memo && ok ? edge_slot(T, sv, (from > 1 ? from : 1) + lane, depth) : -1;
+    if (parse && status == ROW_OK) {
+        // window entries from the lowest one written up to the new depth (lo stays
+        // INT_MAX when nothing was written: clamp before adding the lane)
+        int hi = depth < sv.base + ADV_WIN ? depth : sv.base + ADV_WIN;
+        int w0 = sv.lo > sv.base ? sv.lo : sv.base;
+        w0 = w0 < hi ? w0 : hi;
+        for (int i = w0 + lane; i < hi; i += 32) sv.st[i] = sv.win[i - sv.base];
     }
     if (lane == 0) {
         if (tok >= 0) S.status[b] = status;
@@ -1381,20 +1409,20 @@ __global__ void __launch_bounds__(ADV_WARPS * 32, 1)   // the staged tables leav
         mid = 1;
     } else if (status != ROW_OK) {
         mid = 0;
-    } else if (depth < 1 || depth > S.cap || q < 0 || q >= T.nq) {
+    } else if (!ok || q < 0 || q >= T.nq) {
         mid = 0;
     } else {
         mid = -1;
         if (memo) {
             // bottom-up classifier: re-read the entries from the lowest one written
             // (none written: the stack is as kept) and look the lexer state up
-            int from = parse && sv.lo < depth ? sv.lo : depth;
             int below = from - 1;                    // block of stack [0, below] as kept
             int d = depth0 - 1 - below;              // its lane in the prefetched top
             int e_below = -1;
             if (below >= 0) e_below = d >= 0 && d < 32 ? __shfl_sync(FULL, memo_top, d) : memo[below];
-            int e = warp_memo_extend(T, sv, memo, from, depth, e_below, lane);
-            mid = memo_mask(T, e, q);
+            int fr = from < depth || d != 0 ? -1 : fr_top;
+            int e = warp_memo_extend(T, sv, memo, from, depth, e_below, slot, lane, fr);
+            mid = memo_mask(T, e, fr, q);
         }
         if (mid < 0) mid = warp_walk(T, sv, q, depth, lane);
     }
@@ -1813,7 +1841,8 @@ std::vector<uint8_t> build_advance_blob(const psc::Tables& t, DevTables& d, int 
     d.adv_bytes = 0;
     d.adv_comb = 0;
     int n_rules = (int)t.rule_len.size();
-    if (t.n_lr >= 8192 || n_rules >= 8192 || t.nq >= 32768 || t.n_terms >= 32768) return blob;
+    if (t.n_lr >= 8192 || n_rules >= 8192 || t.nq >= 32768 || t.n_terms >= 32768 || t.n_classes >= 16384)
+        return blob;
     for (int L : t.rule_len)
         if (L > 255) return blob;
     // byte classes of the lexer DFA
@@ -1840,7 +1869,6 @@ std::vector<uint8_t> build_advance_blob(const psc::Tables& t, DevTables& d, int 
     d.o_bc = take(256);
     d.o_trans = take((size_t)t.nq * nbc * 2);
     d.o_accept = take((size_t)t.nq * 2);
-    d.o_ign = take((size_t)std::max(ncls, 1));
     d.o_resolve = take((size_t)std::max(ncls, 1) * t.n_lr * 2);
     d.o_action = take((size_t)t.n_lr * t.n_terms * 2);
     d.o_go = take((size_t)t.n_lr * t.n_nts * 2);
@@ -1850,6 +1878,11 @@ std::vector<uint8_t> build_advance_blob(const psc::Tables& t, DevTables& d, int 
         fprintf(stderr, "psc: advance tables %zu B (lexer %d x %d classes, resolve %d x %d, action %d x %d, goto %d x %d)%s\n",
                 off, t.nq, nbc, ncls, t.n_lr, t.n_lr, t.n_terms, t.n_lr, t.n_nts,
                 off > ADV_TABLE_MAX ? ": too large for shared memory" : "");
+    // class << 1 | ignored of a complete lexeme; -1 where none is complete, and in the start state
+    auto enc_accept = [&](int q) {
+        int c = t.lex_accept[q];
+        return (int16_t)(c < 0 || q == t.q0 ? -1 : c << 1 | (t.cls_ignored[c] ? 1 : 0));
+    };
     int max_len = 0;
     for (int L : t.rule_len) max_len = std::max(max_len, L);
     d.adv_packed = (max_len < 16 && t.n_nts <= 1024) ? 1 : 0;
@@ -1978,10 +2011,9 @@ std::vector<uint8_t> build_advance_blob(const psc::Tables& t, DevTables& d, int 
             for (int b = 0; b < 256; b++)
                 reinterpret_cast<int16_t*>(blob.data() + d.o_trans)[(size_t)q * nbc + bc[b]] =
                     (int16_t)t.lex_trans[(size_t)q * 256 + b];
-            reinterpret_cast<int16_t*>(blob.data() + d.o_accept)[q] = (int16_t)t.lex_accept[q];
+            reinterpret_cast<int16_t*>(blob.data() + d.o_accept)[q] = enc_accept(q);
         }
         for (int c = 0; c < ncls; c++) {
-            blob[d.o_ign + c] = t.cls_ignored[c];
             for (int k = 0; k < kc; k++)
                 reinterpret_cast<int16_t*>(blob.data() + d.o_cand)[(size_t)c * kc + k] =
                     (int16_t)(k < (int)cands[c].size() ? cands[c][k] : -1);
@@ -2005,10 +2037,9 @@ std::vector<uint8_t> build_advance_blob(const psc::Tables& t, DevTables& d, int 
     for (int b = 0; b < 256; b++) blob[d.o_bc + b] = (uint8_t)bc[b];
     for (int q = 0; q < t.nq; q++) {
         for (int b = 0; b < 256; b++) put16(d.o_trans, (size_t)q * nbc + bc[b], t.lex_trans[(size_t)q * 256 + b]);
-        put16(d.o_accept, q, t.lex_accept[q]);
+        put16(d.o_accept, q, enc_accept(q));
     }
     for (int c = 0; c < ncls; c++) {
-        blob[d.o_ign + c] = t.cls_ignored[c];
         for (int s = 0; s < t.n_lr; s++) put16(d.o_resolve, (size_t)c * t.n_lr + s, t.resolve[(size_t)c * t.n_lr + s]);
     }
     // a reduce entry carries its rule's length and left-hand side when they fit in 14 bits
@@ -2050,13 +2081,30 @@ psc_status noalloc_scratch(int device, int32_t** out) {
 }  // namespace
 
 namespace {
-// The first 32 bytes of every token, zero-padded to 32 ([V][32]): the advance loads a
-// token's bytes with its length, instead of after its offset.
-std::vector<uint8_t> token_prefixes(const psc::Tables& t) {
+// One 32-byte record per token ([V][32]): its bytes and, in the last byte, its length (255:
+// longer than 31 bytes), so that the advance has both in one load.
+std::vector<uint8_t> token_records(const psc::Tables& t) {
     std::vector<uint8_t> out((size_t)t.V * 32, 0);
     for (int v = 0; v < t.V; v++) {
-        int64_t lo = t.vocab_off[v], n = std::min<int64_t>(32, t.vocab_off[v + 1] - lo);
-        if (n > 0) std::memcpy(out.data() + (size_t)v * 32, t.vocab_bytes.data() + lo, (size_t)n);
+        int64_t lo = t.vocab_off[v], n = t.vocab_off[v + 1] - lo;
+        if (n > 0) std::memcpy(out.data() + (size_t)v * 32, t.vocab_bytes.data() + lo, (size_t)std::min<int64_t>(n, 31));
+        out[(size_t)v * 32 + 31] = n > 31 ? 255 : (uint8_t)n;
+    }
+    return out;
+}
+
+// The bottom-up classifier's blocks with every successor's final row beside it (the mask
+// lookup after the last stack entry read then needs one load less).
+std::vector<int2> bottom_up_blocks(const psc::Tables& t) {
+    std::vector<int> deg(t.n_lr, 0);
+    for (int a = 0; a < t.n_lr; a++)
+        for (int u = 0; u < t.n_lr; u++) deg[a] += t.bu_slot[(size_t)a * t.n_lr + u] >= 0;
+    std::vector<int2> out(t.bu.size());
+    size_t e = 0;
+    for (int r = 0; r < t.n_bu; r++) {
+        out[e] = make_int2(t.bu[e], 0);
+        for (int k = 1; k <= deg[t.bu_t[r]]; k++) out[e + k] = make_int2(t.bu[e + k], t.bu[(size_t)t.bu[e + k]]);
+        e += 1 + (size_t)deg[t.bu_t[r]];
     }
     return out;
 }
@@ -2105,7 +2153,7 @@ psc_status upload_tables(std::unique_ptr<psc_handle>& h, int tables) {
         (s = upload(h.get(), dfa_mask, &d.dfa_mask)) || (s = upload(h.get(), t.mask_chunks, &d.mchunks)) ||
         (s = upload(h.get(), t.mask_rows, &d.mrows)) ||
         (s = upload(h.get(), t.vocab_bytes, &d.vocab, 16)) || (s = upload(h.get(), t.vocab_off, &d.vocab_off)) ||
-        (s = upload(h.get(), token_prefixes(t), &d.tok32))) {
+        (s = upload(h.get(), token_records(t), &d.tok32))) {
         for (int i = 0; i < h->n_blocks; i++) cudaFree(h->blocks[i]);
         return s;
     }
@@ -2114,7 +2162,7 @@ psc_status upload_tables(std::unique_ptr<psc_handle>& h, int tables) {
     d.bu_F = nullptr;
     d.bu_len = d.n_frow = 0;
     if (t.n_bu > 0) {
-        if ((s = upload(h.get(), t.bu, &d.bu)) || (s = upload(h.get(), t.bu_slot, &d.bu_slot)) ||
+        if ((s = upload(h.get(), bottom_up_blocks(t), &d.bu)) || (s = upload(h.get(), t.bu_slot, &d.bu_slot)) ||
             (s = upload(h.get(), t.bu_F, &d.bu_F))) {
             for (int i = 0; i < h->n_blocks; i++) cudaFree(h->blocks[i]);
             return s;
@@ -2245,7 +2293,7 @@ psc_status psc_info(const psc_handle* h, psc_info_t* out) {
         out->advance_tables_packed = h->d.adv_bytes > 0 && h->d.adv_comb;
     }
     out->bottom_up_states = t.n_bu;
-    out->bottom_up_bytes = (int64_t)(t.bu.size() + t.bu_F.size()) * 4 + (int64_t)t.bu_slot.size() * 2;
+    out->bottom_up_bytes = (int64_t)(2 * t.bu.size() + t.bu_F.size()) * 4 + (int64_t)t.bu_slot.size() * 2;
     out->device_timeouts = 0;
     if (!h->host_only) {
         int v = 0;
@@ -2267,28 +2315,34 @@ psc_status psc_state_init(const psc_handle* h, int32_t B, int32_t cap, void* str
     DevStates& d = st->d;
     d.B = B;
     d.cap = cap;
-    // the fault word, then the bottom-up classifier's kept blocks only when the handle has
-    // that classifier
-    const int n_arr = h->d.bu ? 8 : 7;
-    void* p[8] = {};
-    size_t sz[8] = {sizeof(int32_t) * B, sizeof(int32_t) * B, sizeof(int32_t) * B, sizeof(uint16_t) * (size_t)B * cap,
-                    sizeof(int32_t) * B, sizeof(unsigned long long) * B, sizeof(int32_t),
-                    sizeof(int32_t) * (size_t)B * cap};
-    for (int i = 0; i < n_arr; i++) {
-        s = cuda_check(cudaMalloc(&p[i], sz[i]), "cudaMalloc(states)");
-        if (s != PSC_OK) {
-            for (int j = 0; j < i; j++) cudaFree(p[j]);
-            return s;
-        }
-    }
-    d.q = (int32_t*)p[0];
-    d.depth = (int32_t*)p[1];
-    d.status = (int32_t*)p[2];
-    d.stack = (uint16_t*)p[3];
-    d.mid = (int32_t*)p[4];
-    d.best = (unsigned long long*)p[5];
-    d.fault = (int32_t*)p[6];
-    d.rmemo = (int32_t*)p[7];
+    // one allocation for all the arrays (the advance reads most of them in its first two
+    // round trips: fewer pages to translate), the kept blocks only when the handle has the
+    // bottom-up classifier, the fault word last
+    size_t off = 0;
+    auto take = [&](size_t bytes) {
+        size_t o = off;
+        off = (off + bytes + 255) & ~(size_t)255;
+        return o;
+    };
+    const size_t o_q = take(sizeof(int32_t) * (size_t)B), o_depth = take(sizeof(int32_t) * (size_t)B),
+                 o_status = take(sizeof(int32_t) * (size_t)B), o_mid = take(sizeof(int32_t) * (size_t)B),
+                 o_best = take(sizeof(unsigned long long) * (size_t)B),
+                 o_stack = take(sizeof(uint16_t) * (size_t)B * cap),
+                 o_memo = take(h->d.bu ? sizeof(int32_t) * (size_t)B * cap : 0);
+    st->copy_bytes = off;
+    const size_t o_fault = take(sizeof(int32_t));
+    uint8_t* base = nullptr;
+    s = cuda_check(cudaMalloc(&base, off), "cudaMalloc(states)");
+    if (s != PSC_OK) return s;
+    st->base = base;
+    d.q = (int32_t*)(base + o_q);
+    d.depth = (int32_t*)(base + o_depth);
+    d.status = (int32_t*)(base + o_status);
+    d.mid = (int32_t*)(base + o_mid);
+    d.best = (unsigned long long*)(base + o_best);
+    d.stack = (uint16_t*)(base + o_stack);
+    d.rmemo = h->d.bu ? (int32_t*)(base + o_memo) : nullptr;
+    d.fault = (int32_t*)(base + o_fault);
     cudaStream_t cs = (cudaStream_t)stream;
     s = cuda_check(cudaMemsetAsync(d.fault, 0, sizeof(int32_t), cs), "cudaMemsetAsync(fault)");
     if (s == PSC_OK) {
@@ -2297,7 +2351,7 @@ psc_status psc_state_init(const psc_handle* h, int32_t B, int32_t cap, void* str
         st->mid_gen = st->gen;
     }
     if (s != PSC_OK) {
-        for (int j = 0; j < n_arr; j++) cudaFree(p[j]);
+        cudaFree(base);
         return s;
     }
     *out = st.release();
@@ -2312,26 +2366,10 @@ psc_status psc_state_copy(psc_states* dst, const psc_states* src, void* stream) 
     cudaGetDevice(&dev);
     if (dev != dst->device) return fail_with(PSC_ERR_ARG, "psc_state_copy: current device differs from the states'");
     cudaStream_t cs = (cudaStream_t)stream;
-    const DevStates& a = src->d;
-    DevStates& b = dst->d;
-    size_t B = (size_t)a.B;
-    // one kernel for all the arrays (a copy per array costs a stream round trip each)
-    CopySegs c{};
-    auto add = [&](const void* src, void* dst, size_t bytes) {
-        c.src[c.n] = static_cast<const uint8_t*>(src);
-        c.dst[c.n] = static_cast<uint8_t*>(dst);
-        c.bytes[c.n++] = bytes;
-    };
-    add(a.q, b.q, B * 4);
-    add(a.depth, b.depth, B * 4);
-    add(a.status, b.status, B * 4);
-    add(a.stack, b.stack, B * (size_t)a.cap * 2);
-    add(a.mid, b.mid, B * 4);
-    if (a.best && b.best) add(a.best, b.best, B * 8);
-    if (a.rmemo && b.rmemo) add(a.rmemo, b.rmemo, B * (size_t)a.cap * 4);
-    size_t v16 = (B * (size_t)a.cap * 6 + B * 24) / 16;
-    int grid = (int)std::max<size_t>(1, std::min<size_t>((v16 + 255) / 256, (size_t)sm_count(dev) * 4));
-    psc_status s = launch_pdl(k_state_copy, dim3(grid), dim3(256), 0, cs, "k_state_copy", c);
+    const size_t n16 = src->copy_bytes / 16;
+    int grid = (int)std::max<size_t>(1, std::min<size_t>((n16 + 255) / 256, (size_t)sm_count(dev) * 4));
+    psc_status s = launch_pdl(k_state_copy, dim3(grid), dim3(256), 0, cs, "k_state_copy", (const uint4*)src->base,
+                              (uint4*)dst->base, n16);
     if (s != PSC_OK) return s;
     dst->gen++;
     dst->mid_gen = src->mid_gen == src->gen ? dst->gen : 0;   // the mask ids are as current as src's
@@ -2357,14 +2395,7 @@ psc_status psc_state_reset(psc_states* st, const int32_t* d_rows, int32_t n, voi
 
 void psc_state_destroy(psc_states* st) {
     if (!st) return;
-    cudaFree(st->d.q);
-    cudaFree(st->d.depth);
-    cudaFree(st->d.status);
-    cudaFree(st->d.stack);
-    cudaFree(st->d.mid);
-    cudaFree(st->d.best);
-    cudaFree(st->d.fault);
-    cudaFree(st->d.rmemo);
+    cudaFree(st->base);
     delete st;
 }
 

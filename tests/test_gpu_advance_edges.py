@@ -1,0 +1,72 @@
+"""GPU: the advance at the edges of its token records, stack window and row layout (tokens of
+29-70 bytes and as many lexemes, stacks past the shared-memory window, capacities that are
+not whole 16-byte pieces), against the library's host step and host classification, which
+the CPU tests hold to the oracle."""
+from __future__ import annotations
+
+import numpy as np
+import pytest
+
+from workloads import grammars
+
+torch = pytest.importorskip("torch")
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module")
+def psc():
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    from paper_2608_03065_gb300 import build, psc as mod
+    build.build()
+    mod.load()
+    return mod
+
+
+@pytest.mark.parametrize("cap", [400, 397, 64])
+@pytest.mark.parametrize("bottom_up", [True, False])
+@pytest.mark.parametrize("tables", ["dense", "packed"])
+def test_long_tokens_and_deep_stacks(psc, tables, bottom_up, cap):
+    lengths = (1, 29, 30, 31, 32, 33, 40, 70)
+    toks = [bytes([c]) for c in b'[]{}:,"0123456789truefalsn -.e\\ab']
+    for n in lengths:
+        toks += [b"[" * n, b"]" * n, b"a" * n, b"1" * n, b" " * n, b'"' + b"b" * (n - 1), b'b"' + b"," + b"1" * n,
+                 b"1," * n, b"[1]," * (n // 2 + 1), b'["' + b"a" * n + b'"']
+    toks = list(dict.fromkeys(toks)) + [b""]
+    V = len(toks)
+    h = psc.psc_compile(grammars.json_grammar().text(), toks, V - 1, packed_tables=tables == "packed", bottom_up=bottom_up)
+    rng = np.random.default_rng([cap, len(tables), bottom_up])
+    B = 24
+    st = psc.psc_state_init(h, B, cap)
+    rows = [h.host_initial() for _ in range(B)]
+    deep = [toks.index(b"[" * n) for n in (70, 40, 33, 32, 31)]
+    for step in range(26):
+        t = np.full(B, -1, dtype=np.int32)
+        for b, r in enumerate(rows):
+            if r["status"] != 0:
+                continue
+            mask = h.host_mask_row(h.host_classify(r["q"], r["stack"], r["status"]))
+            ok = np.nonzero(np.unpackbits(mask.view(np.uint8), bitorder="little")[:V])[0]
+            long_ok = [v for v in ok if len(toks[v]) > 20]
+            if step < 6 and b % 3:
+                t[b] = deep[int(rng.integers(0, len(deep)))]       # down past the window
+            elif len(long_ok) and rng.random() < 0.8:
+                t[b] = int(rng.choice(long_ok))
+            elif len(ok) and rng.random() < 0.95:
+                t[b] = int(rng.choice(ok))
+            else:
+                t[b] = int(rng.integers(0, V))                     # most likely rejected
+        psc.psc_advance(h, st, torch.from_numpy(t).cuda())
+        rows = [h.host_advance(r, int(t[b]), cap) if t[b] >= 0 else r for b, r in enumerate(rows)]
+        got = psc.psc_states_download(st)
+        bm = torch.zeros(B, h.W, dtype=torch.int32, device="cuda")
+        psc.psc_fill_mask(h, st, bm)
+        bm = bm.cpu().numpy().view(np.uint32)
+        for b, r in enumerate(rows):
+            assert got["status"][b] == r["status"], (step, b, toks[t[b]])
+            if r["status"] == 0:
+                assert got["q"][b] == r["q"] and got["depth"][b] == len(r["stack"]), (step, b, toks[t[b]])
+                assert got["stack"][b, :len(r["stack"])].tolist() == r["stack"], (step, b, toks[t[b]])
+            want = h.host_mask_row(h.host_classify(r["q"], r["stack"], r["status"]))
+            assert np.array_equal(bm[b], want), (step, b, toks[t[b]])
+    assert max(len(r["stack"]) for r in rows) > (192 if cap > 64 else 20)
