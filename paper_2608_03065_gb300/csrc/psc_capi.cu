@@ -115,6 +115,10 @@ struct psc_handle {
     int n_blocks = 0;
     int tables = 0;             // psc_options.global_tables the handle was made with
     int mid0 = 0;               // mask id of the empty prefix
+    int sms = 1;                // the device's SMs
+    int row_cta_smem = 0;       // shared memory of a k_decode_row CTA, with what the hardware reserves
+    int row_cluster = 1;        // CTAs of a k_decode_row cluster at most
+    int row_sm_smem = 0;        // shared memory of an SM (0: k_decode_row cannot stage the tables)
 };
 
 struct psc_states {
@@ -125,6 +129,7 @@ struct psc_states {
     size_t copy_bytes = 0;   // what psc_state_copy copies of it (all but the fault word)
     uint64_t gen = 1;        // bumped by every call that changes the rows
     uint64_t mid_gen = 0;    // generation the mask ids in d.mid were computed for
+    bool keys = false;       // psc_decode_step_mask left greedy choices that nothing consumed yet
     bool after_mask = false; // the last work enqueued on these states is the masking pass with the
                              // mask ids as they were (the advance may read the rows early)
 };
@@ -811,8 +816,10 @@ constexpr int ADV_WIN = 256;     // stack entries held per row
 constexpr int ADV_KEEP = 192;    // entries copied in (the rest is room for pushes)
 constexpr size_t ADV_TABLE_MAX = 200 * 1024;   // staged tables at most (one CTA of 8 rows per SM)
 
-// Dynamic shared memory of k_advance_warp: the staged tables, then the stack windows.
+// Dynamic shared memory of k_advance_warp (k_decode_row): the staged tables, then the stack
+// windows (window).
 int adv_smem(const DevTables& d) { return d.adv_bytes + ADV_WARPS * ADV_WIN * 2; }
+int row_smem(const DevTables& d) { return d.adv_bytes + ADV_WIN * 2; }
 
 __device__ __forceinline__ uint32_t smem_addr(const void* p) {
     return static_cast<uint32_t>(__cvta_generic_to_shared(p));
@@ -838,6 +845,21 @@ __device__ __forceinline__ bool mbar_wait0(uint32_t bar, int limit) {
         uint32_t ok;
         asm volatile(
             "{\n .reg .pred p;\n mbarrier.try_wait.parity.shared::cta.b64 p, [%1], 0;\n selp.u32 %0, 1, 0, p;\n}"
+            : "=r"(ok)
+            : "r"(bar)
+            : "memory");
+        if (ok) return true;
+    }
+    return false;
+}
+
+// The same, with what the cluster's threads released at their arrivals made visible.
+__device__ __forceinline__ bool mbar_wait0_cluster(uint32_t bar, int limit) {
+    for (int it = 0; it < limit; it++) {
+        uint32_t ok;
+        asm volatile(
+            "{\n .reg .pred p;\n mbarrier.try_wait.parity.acquire.cluster.shared::cta.b64 p, [%1], 0;\n"
+            " selp.u32 %0, 1, 0, p;\n}"
             : "=r"(ok)
             : "r"(bar)
             : "memory");
@@ -1152,142 +1174,133 @@ __device__ __forceinline__ int warp_memo_extend(const DevTables& T, const StackV
 // now), parsing (up to 5,000), edge slots and blocks of the entries written (loads in
 // flight during the write-back), the mask id (two loads before, one now: a block's final
 // row comes with the block).
-// early: the row's state (lexer state, depth, status, mask id, stack window, kept
-// bottom-up blocks) is read before waiting for the previous kernel.  Only the greedy
-// keys come from that kernel (the masking pass), and the masking pass lets this
-// kernel start only after its own wait for the advance before it, which wrote the
-// rows; the host sets `early` only when the masking pass is the last work on
-// these states and took the mask ids as they were.
 template <bool PACKED, bool COMB>
-__global__ void __launch_bounds__(ADV_WARPS * 32, 1)   // the staged tables leave room for one CTA per SM: no spills
-    k_advance_warp(DevTables T, DevStates S, const int32_t* tokens,
-                                                                 int B, int32_t* status_out,
-                                                                 int from_keys, int32_t* tokens_out, int early) {
-    extern __shared__ uint4 smem4[];
-    __shared__ __align__(8) uint64_t bar;
-    __shared__ uint16_t lexcls[ADV_WARPS][32];  // the lexeme classes the token emits (tokens up to 32 bytes)
-    uint8_t* sm = reinterpret_cast<uint8_t*>(smem4);
-    // one TMA bulk copy stages the compact tables (16-byte aligned, multiple of 16 bytes)
-    uint32_t bar_a = smem_addr(&bar);
-    if (threadIdx.x == 0) {
-        asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(bar_a) : "memory");
-        asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
-        asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(bar_a), "r"(T.adv_bytes) : "memory");
-        asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];"
-                     ::"r"(smem_addr(sm)), "l"(gmem_addr(T.adv)), "r"(T.adv_bytes), "r"(bar_a)
-                     : "memory");
-    }
-    grid_dep_launch();
-    __syncthreads();   // the mbarrier; before the wait, so that no row waits for another row's loads
-    int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    int b = blockIdx.x * ADV_WARPS + warp;
-    bool active = b < B;   // warp-uniform
-    StackView sv{reinterpret_cast<uint16_t*>(sm + T.adv_bytes) + warp * ADV_WIN,
-                 S.stack + (size_t)(active ? b : 0) * S.cap, 0x40000000, 0x7FFFFFFF, 0u};
-    sv.wa = smem_addr(sv.win);
-    int tok = -1, status = ROW_OK, q = 0, depth = 0;
-    bool parse = false;
-    int32_t* memo = active && S.rmemo && T.bu ? S.rmemo + (size_t)b * S.cap : nullptr;
-    int memo_top = -1, depth0 = 0;
-    uint32_t mchunk = 0;   // the mask chunk that holds the token's bit
-    bool eos = false;
-    int tbyte = 0;   // lane i: byte i of the token (lane 31: its length)
-    int cur_mid = 0;   // the mask the row's token is checked against
-    bool live = false;
-    // the row's state, then the window of its stack top (for the parse and for the
-    // classifier walk after it) and the kept bottom-up blocks of the top 32 prefixes; read
-    // from L2 (an SM's L1 may still hold these lines from an earlier kernel)
-    auto load_row = [&]() {
+struct RowAdvance {
+    const DevTables& T;
+    const DevStates& S;
+    const int b, lane;
+    StackView sv;
+    int32_t* const memo;     // the row's kept bottom-up blocks (null: none)
+    const uint32_t la;       // shared-window address of 32 uint16: the lexeme classes the token emits
+    const bool vec;          // stacks of whole 16-byte pieces (their allocation is aligned)
+    int tok = -1, status = ROW_OK, q = 0, depth = 0, depth0 = 0;
+    int mid = 0;             // the row's mask id
+    int memo_top = -1;       // lane l: the kept block of the stack without its top l entries
+    int tbyte = 0;           // lane i: byte i of the token (lane 31: its length)
+    uint32_t mchunk = 0;     // the mask chunk that holds the token's bit
+    uint4 wv = make_uint4(0u, 0u, 0u, 0u);
+    bool live = false, parse = false, eos = false;
+
+    __device__ __forceinline__ RowAdvance(const DevTables& T, const DevStates& S, int b, int lane, uint16_t* win, uint32_t la)
+        : T(T), S(S), b(b), lane(lane), sv{win, S.stack + (size_t)b * S.cap, 0x40000000, 0x7FFFFFFF, smem_addr(win)},
+          memo(S.rmemo && T.bu ? S.rmemo + (size_t)b * S.cap : nullptr), la(la), vec(S.cap % 8 == 0) {}
+
+    // The row's state, then the window of its stack top (for the parse and for the
+    // classifier walk after it) and the kept blocks of the top 32 prefixes; read from L2
+    // (an SM's L1 may still hold these lines from an earlier kernel).  load_window issues
+    // its loads, place_window waits for them.
+    __device__ __forceinline__ void load_row() {
         q = __ldcg(S.q + b);
         depth = __ldcg(S.depth + b);
         status = __ldcg(S.status + b);
-        cur_mid = __ldcg(S.mid + b);
-    };
-    const bool vec = S.cap % 8 == 0;   // rows of whole 16-byte pieces (their allocation is aligned)
-    uint4 wv = make_uint4(0u, 0u, 0u, 0u);
-    auto load_window = [&]() {   // issues the loads; place_window waits for them
+        mid = __ldcg(S.mid + b);
+    }
+    __device__ __forceinline__ void load_window() {
         depth0 = depth;
         live = status == ROW_OK && depth >= 1 && depth <= S.cap;
         if (!live) return;
         sv.base = depth > ADV_KEEP ? (depth - ADV_KEEP + 7) & ~7 : 0;
         if (vec && lane * 8 < depth - sv.base) wv = __ldcg(reinterpret_cast<const uint4*>(sv.st + sv.base) + lane);
-        if (memo && depth - 1 - lane >= 0) memo_top = __ldcg(memo + depth - 1 - lane);   // lane l: stack [0, depth-1-l]
-    };
-    auto place_window = [&]() {
+        if (memo && depth - 1 - lane >= 0) memo_top = __ldcg(memo + depth - 1 - lane);
+    }
+    __device__ __forceinline__ void place_window() {
         if (!live) return;
         if (vec) {
             if (lane * 8 < depth - sv.base) *(reinterpret_cast<uint4*>(sv.win) + lane) = wv;
         } else {
             for (int i = lane; i < depth - sv.base; i += 32) sv.win[i] = __ldcg(sv.st + sv.base + i);
         }
-    };
-    if (active && early) {
-        load_row();
-        load_window();
-        place_window();
     }
-    grid_dep_wait();   // the greedy keys (and, unless early, the rows) come from the previous kernel
-    if (active) {
-        // one round trip for the token and the row's state, the next for the token's bytes,
-        // the mask's chunk id and the window
-        unsigned long long key = 0ull;
-        if (from_keys) key = __ldcg(S.best + b);   // the greedy choice of the masking pass
-        else tok = tokens[b];
-        if (!early) load_row();
-        if (from_keys) tok = key ? (int32_t)(~(uint32_t)(key & 0xFFFFFFFFu)) : -1;
-        const bool known = tok >= 0 && tok < T.V;
-        if (known) tbyte = T.tok32[(size_t)tok * 32 + lane];   // lane i holds byte i, lane 31 the length
-        if (!early) load_window();
-        if (known && status == ROW_OK) mchunk = __ldg(T.mrows + (size_t)cur_mid * T.nch + (tok >> 10));
-        if (!early) place_window();
-        __syncwarp();   // every lane has read the key
-        if (from_keys && lane == 0) {
-            S.best[b] = 0ull;
-            tokens_out[b] = tok;
-        }
-        if (tok >= 0) {
-            if (status == ROW_DONE) {
-                status = tok == T.eos_id ? ROW_DONE : ROW_REJECTED;
-            } else if (status == ROW_OK) {
-                if (!known) status = ROW_REJECTED;
-                else if (tok == T.eos_id) eos = true;
-                else if (!live) status = ROW_REJECTED;
-                else parse = true;
-            }
+    // The loads that need only the token (tok set), and with the row's status known the
+    // chunk of its mask that holds the token's bit (unless the token is known to be allowed).
+    __device__ __forceinline__ void load_token() {
+        if (tok >= 0 && tok < T.V) tbyte = T.tok32[(size_t)tok * 32 + lane];
+    }
+    __device__ __forceinline__ void load_mask_chunk() {
+        if (tok >= 0 && tok < T.V && status == ROW_OK) mchunk = __ldg(T.mrows + (size_t)mid * T.nch + (tok >> 10));
+    }
+    // What the token does to the row, the parse apart.
+    __device__ __forceinline__ void judge() {
+        if (tok < 0) return;
+        if (status == ROW_DONE) {
+            status = tok == T.eos_id ? ROW_DONE : ROW_REJECTED;
+        } else if (status == ROW_OK) {
+            if (tok >= T.V) status = ROW_REJECTED;
+            else if (tok == T.eos_id) eos = true;
+            else if (!live) status = ROW_REJECTED;
+            else parse = true;
         }
     }
-    // the token's mask word (in flight while the token is parsed); the row is only
-    // committed (q, depth) when the token's bit is set
-    // (chunk 0 when there is no such token: loads without a condition, so that nothing waits
-    // for them here)
-    const uint32_t mword = __ldg(T.mchunks + (size_t)mchunk * 32 + ((tok >> 5) & 31));
-    // the final row of the stack as it is (used when the token writes no stack entry)
-    const int e_top = __shfl_sync(FULL, memo_top, 0);
-    int fr_top = -1;
-    if (memo) fr_top = __ldg(T.bu + min(max(e_top, 0), T.bu_len - 1)).x;
-    bool staged = __all_sync(FULL, mbar_wait0(bar_a, 1 << 24));
-    if (!staged) {
-        // the copy did not land: give the rows a LIMIT status, wait (bounded) for the copy, return
-        if (threadIdx.x == 0) {
-            atomicAdd(&g_pipeline_timeouts, 1);
-            if (S.fault) atomicAdd(S.fault, 1);
+    // The rows that could not be advanced (a wait gave up).
+    __device__ __forceinline__ void give_up(int32_t* status_out) {
+        if (lane != 0) return;
+        if (status == ROW_OK) status = ROW_LIMIT;
+        S.status[b] = status;
+        if (status_out) status_out[b] = status;
+        S.mid[b] = 0;
+    }
+    // Lexing, parsing, write-back and classification, with the staged tables at tables.
+    // The row is only committed (q, depth, stack) when allowed.  fr_top: the final row of
+    // the block memo_top of the whole stack.
+    __device__ __forceinline__ void finish(uint32_t tables, uint32_t mword, int fr_top, int32_t* status_out) {
+        if (parse) lex_and_parse(AdvTabs(tables, T), mword);
+        if (eos) status = ((mword >> (tok & 31)) & 1) ? ROW_DONE : ROW_REJECTED;   // here, not before: it waits for mword
+        // the lowest stack entry written (depth: none), and the edge slots of the entries from
+        // there on, in flight while the stack is written back
+        const int from = parse && sv.lo < depth ? sv.lo : depth;
+        const bool ok = status == ROW_OK && depth >= 1 && depth <= S.cap;
+        const int slot = memo && ok ? edge_slot(T, sv, (from > 1 ? from : 1) + lane, depth) : -1;
+        if (parse && status == ROW_OK) {
+            // window entries from the lowest one written up to the new depth (lo stays
+            // INT_MAX when nothing was written: clamp before adding the lane)
+            int hi = depth < sv.base + ADV_WIN ? depth : sv.base + ADV_WIN;
+            int w0 = sv.lo > sv.base ? sv.lo : sv.base;
+            w0 = w0 < hi ? w0 : hi;
+            for (int i = w0 + lane; i < hi; i += 32) sv.st[i] = sv.win[i - sv.base];
         }
-        if (active && lane == 0) {
-            if (status == ROW_OK) status = ROW_LIMIT;
-            S.status[b] = status;
+        if (lane == 0) {
+            if (tok >= 0) S.status[b] = status;
             if (status_out) status_out[b] = status;
-            S.mid[b] = 0;
         }
-        mbar_wait0(bar_a, 1 << 24);
-        return;
+        // the next masking pass's mask id (the window holds the stack top of every live
+        // row; for the others sv.base still points past any stack index)
+        if (status == ROW_DONE) {
+            mid = 1;
+        } else if (status != ROW_OK) {
+            mid = 0;
+        } else if (!ok || q < 0 || q >= T.nq) {
+            mid = 0;
+        } else {
+            mid = -1;
+            if (memo) {
+                // bottom-up classifier: re-read the entries from the lowest one written
+                // (none written: the stack is as kept) and look the lexer state up
+                int below = from - 1;                    // block of stack [0, below] as kept
+                int d = depth0 - 1 - below;              // its lane in the prefetched top
+                int e_below = -1;
+                if (below >= 0) e_below = d >= 0 && d < 32 ? __shfl_sync(FULL, memo_top, d) : memo[below];
+                int fr = from < depth || d != 0 ? -1 : fr_top;
+                int e = warp_memo_extend(T, sv, memo, from, depth, e_below, slot, lane, fr);
+                mid = memo_mask(T, e, fr, q);
+            }
+            if (mid < 0) mid = warp_walk(T, sv, q, depth, lane);
+        }
+        if (lane == 0) S.mid[b] = mid;
     }
-    if (!active) return;
-    if (parse) {
-        const AdvTabs A(smem_addr(sm), T);
+    __device__ __forceinline__ void lex_and_parse(const AdvTabs A, uint32_t mword) {
         int nq = q, nd = depth;
-        const uint32_t la = smem_addr(&lexcls[warp][0]);
         const int len = __shfl_sync(FULL, tbyte, 31);
-        int ncls = -1;   // classes in lexcls; -1: the token is lexed by lane 0 (longer than 31 bytes)
+        int ncls = -1;   // classes at la; -1: the token is lexed by lane 0 (longer than 31 bytes)
         if (len <= 31) {
             // Lexing in parallel (the lexer does not depend on the parser): lane j runs the
             // lexer DFA over the lexeme that starts afresh at byte j (ls, ending at le), every
@@ -1384,49 +1397,86 @@ __global__ void __launch_bounds__(ADV_WARPS * 32, 1)   // the staged tables leav
         sv.lo = __shfl_sync(FULL, sv.lo, 0);
         __syncwarp();
     }
-    if (eos) status = ((mword >> (tok & 31)) & 1) ? ROW_DONE : ROW_REJECTED;   // here, not before: it waits for mword
-    // the lowest stack entry written (depth: none), and the edge slots of the entries from
-    // there on, in flight while the stack is written back
-    const int from = parse && sv.lo < depth ? sv.lo : depth;
-    const bool ok = status == ROW_OK && depth >= 1 && depth <= S.cap;
-    const int slot = memo && ok ? edge_slot(T, sv, (from > 1 ? from : 1) + lane, depth) : -1;
-    if (parse && status == ROW_OK) {
-        // window entries from the lowest one written up to the new depth (lo stays
-        // INT_MAX when nothing was written: clamp before adding the lane)
-        int hi = depth < sv.base + ADV_WIN ? depth : sv.base + ADV_WIN;
-        int w0 = sv.lo > sv.base ? sv.lo : sv.base;
-        w0 = w0 < hi ? w0 : hi;
-        for (int i = w0 + lane; i < hi; i += 32) sv.st[i] = sv.win[i - sv.base];
+};
+
+// One TMA bulk copy stages the compact tables (16-byte aligned, multiple of 16 bytes),
+// completing phase 0 of the mbarrier at bar.
+__device__ __forceinline__ void stage_tables(const DevTables& T, uint32_t dst, uint32_t bar) {
+    asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(bar) : "memory");
+    asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+    asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(bar), "r"(T.adv_bytes) : "memory");
+    asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];"
+                 ::"r"(dst), "l"(gmem_addr(T.adv)), "r"(T.adv_bytes), "r"(bar)
+                 : "memory");
+}
+
+// early: the row's state (lexer state, depth, status, mask id, stack window, kept
+// bottom-up blocks) is read before waiting for the previous kernel.  Only the greedy
+// keys come from that kernel (the masking pass), and the masking pass lets this
+// kernel start only after its own wait for the advance before it, which wrote the
+// rows; the host sets `early` only when the masking pass is the last work on
+// these states and took the mask ids as they were.
+template <bool PACKED, bool COMB>
+__global__ void __launch_bounds__(ADV_WARPS * 32, 1)   // the staged tables leave room for one CTA per SM: no spills
+    k_advance_warp(DevTables T, DevStates S, const int32_t* tokens, int B, int32_t* status_out, int from_keys,
+                   int32_t* tokens_out, int early) {
+    extern __shared__ uint4 smem4[];
+    __shared__ __align__(8) uint64_t bar;
+    __shared__ uint16_t lexcls[ADV_WARPS][32];
+    uint8_t* sm = reinterpret_cast<uint8_t*>(smem4);
+    const uint32_t bar_a = smem_addr(&bar);
+    if (threadIdx.x == 0) stage_tables(T, smem_addr(sm), bar_a);
+    grid_dep_launch();
+    __syncthreads();   // the mbarrier; before the wait, so that no row waits for another row's loads
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int b = blockIdx.x * ADV_WARPS + warp;
+    const bool active = b < B;   // warp-uniform
+    RowAdvance<PACKED, COMB> r(T, S, active ? b : 0, lane, reinterpret_cast<uint16_t*>(sm + T.adv_bytes) + warp * ADV_WIN,
+                               smem_addr(&lexcls[warp][0]));
+    if (active && early) {
+        r.load_row();
+        r.load_window();
+        r.place_window();
     }
-    if (lane == 0) {
-        if (tok >= 0) S.status[b] = status;
-        if (status_out) status_out[b] = status;
-    }
-    // the next masking pass's mask id (the window holds the stack top of every live
-    // row; for the others sv.base still points past any stack index)
-    int mid;
-    if (status == ROW_DONE) {
-        mid = 1;
-    } else if (status != ROW_OK) {
-        mid = 0;
-    } else if (!ok || q < 0 || q >= T.nq) {
-        mid = 0;
-    } else {
-        mid = -1;
-        if (memo) {
-            // bottom-up classifier: re-read the entries from the lowest one written
-            // (none written: the stack is as kept) and look the lexer state up
-            int below = from - 1;                    // block of stack [0, below] as kept
-            int d = depth0 - 1 - below;              // its lane in the prefetched top
-            int e_below = -1;
-            if (below >= 0) e_below = d >= 0 && d < 32 ? __shfl_sync(FULL, memo_top, d) : memo[below];
-            int fr = from < depth || d != 0 ? -1 : fr_top;
-            int e = warp_memo_extend(T, sv, memo, from, depth, e_below, slot, lane, fr);
-            mid = memo_mask(T, e, fr, q);
+    grid_dep_wait();   // the greedy keys (and, unless early, the rows) come from the previous kernel
+    if (active) {
+        // one round trip for the token and the row's state, the next for the token's bytes,
+        // the mask's chunk id and the window
+        unsigned long long key = 0ull;
+        if (from_keys) key = __ldcg(S.best + b);   // the greedy choice of the masking pass
+        else r.tok = tokens[b];
+        if (!early) r.load_row();
+        if (from_keys) r.tok = key ? (int32_t)(~(uint32_t)(key & 0xFFFFFFFFu)) : -1;
+        r.load_token();
+        if (!early) r.load_window();
+        r.load_mask_chunk();
+        if (!early) r.place_window();
+        __syncwarp();   // every lane has read the key
+        if (from_keys && lane == 0) {
+            S.best[b] = 0ull;
+            tokens_out[b] = r.tok;
         }
-        if (mid < 0) mid = warp_walk(T, sv, q, depth, lane);
+        r.judge();
     }
-    if (lane == 0) S.mid[b] = mid;
+    // the token's mask word and the final row of the stack as it is, in flight while the
+    // token is parsed (chunk 0 when there is no such token: loads without a condition, so
+    // that nothing waits for them here)
+    const uint32_t mword = __ldg(T.mchunks + (size_t)r.mchunk * 32 + ((r.tok >> 5) & 31));
+    const int e_top = __shfl_sync(FULL, r.memo_top, 0);
+    int fr_top = -1;
+    if (r.memo) fr_top = __ldg(T.bu + min(max(e_top, 0), T.bu_len - 1)).x;
+    const bool staged = __all_sync(FULL, mbar_wait0(bar_a, 1 << 24));
+    if (!staged) {
+        // the copy did not land: give the rows a LIMIT status, wait (bounded) for the copy, return
+        if (threadIdx.x == 0) {
+            atomicAdd(&g_pipeline_timeouts, 1);
+            if (S.fault) atomicAdd(S.fault, 1);
+        }
+        if (active) r.give_up(status_out);
+        mbar_wait0(bar_a, 1 << 24);
+        return;
+    }
+    if (active) r.finish(smem_addr(sm), mword, fr_top, status_out);
 }
 
 // ------------------------------------------------------------ decode masking pass
@@ -1508,6 +1558,96 @@ __global__ void __launch_bounds__(256) k_mask_rows_ahead(T* logits, int64_t stri
         const unsigned long long key = warp_max_key(best_key_of(best));
         if (lane == 0 && key) atomicMax(best_key + b, key);
     }
+}
+
+// A whole decode step (masking, greedy choice, advance, classification) of small bf16
+// batches in one kernel: a cluster of csize CTAs per row, a warp per chunk.  Every warp masks
+// its chunk as in k_mask_rows_ahead and sends its greedy key to the first CTA's
+// shared memory (distributed shared memory, an mbarrier counting the keys); that CTA's
+// first warp then advances the row as in k_advance_warp, its state loaded during the
+// masking.  Bound by the same chain of dependent steps as the two kernels, without the
+// kernel boundary, the trip to the key in global memory, and the mask check (a greedy
+// choice is allowed), and with one launch for the host.
+constexpr int ROW_WARPS = 16;       // warps per CTA at most
+constexpr int ROW_CLUSTER = 16;     // CTAs per row at most (past 8: a non-portable cluster size)
+template <bool PACKED, bool COMB, bool ANY>
+__global__ void __launch_bounds__(ROW_WARPS * 32, 2)   // at most 64 registers
+    k_decode_row(uint16_t* logits, int64_t stride, MaskSrc M, DevTables T, DevStates S, int V, int csize,
+                 int32_t* tokens_out, int32_t* status_out) {
+    extern __shared__ uint4 smem4[];
+    __shared__ uint4 s_lut[256];
+    __shared__ unsigned long long s_key[ROW_CLUSTER * ROW_WARPS];
+    __shared__ __align__(8) uint64_t s_bar[2];   // the staged tables, the keys
+    __shared__ uint16_t lexcls[32];
+    uint8_t* sm = reinterpret_cast<uint8_t*>(smem4);
+    const int b = blockIdx.x / csize, rank = blockIdx.x - b * csize;
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, warps = blockDim.x >> 5;
+    const uint32_t bar_tables = smem_addr(&s_bar[0]), bar_keys = smem_addr(&s_bar[1]);
+    if (rank == 0 && threadIdx.x == 0) {
+        asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(bar_keys) : "memory");
+        asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+        asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(bar_keys), "r"(csize * warps * 8)
+                     : "memory");
+        stage_tables(T, smem_addr(sm), bar_tables);
+    }
+    build_allow_lut<uint16_t>(s_lut);
+    __syncthreads();
+    // the first CTA has started and its mbarriers are set up once every CTA has passed here
+    asm volatile("barrier.cluster.arrive.release.aligned;\nbarrier.cluster.wait.acquire.aligned;" ::: "memory");
+    grid_dep_wait();   // logits and rows come from earlier kernels
+    grid_dep_launch();
+    const bool advances = rank == 0 && warp == 0;
+    RowAdvance<PACKED, COMB> r(T, S, b, lane, reinterpret_cast<uint16_t*>(sm + T.adv_bytes), smem_addr(lexcls));
+    if (advances) r.load_row();
+    const RowView<uint16_t, ANY> R(logits + (size_t)b * stride, V);
+    const int n = R.chunks();
+    Best best;
+    for (int j = rank * warps + warp; j < n; j += csize * warps) {
+        const ChunkAhead<uint16_t> ahead(R, j, lane);
+        const uint32_t cur = M.template word<true>(b, j, lane, M.template locate<true>(b, j, 0));
+        const uint32_t before = ANY ? M.template word_before<true>(b, j) : 0u;
+        if (M.copy_out && j * 32 + lane < M.W) M.copy_out[(size_t)b * M.W + j * 32 + lane] = cur;
+        mask_chunk<uint16_t, true>(R, j, view_word(cur, before, R.a, lane), lane, s_lut, &ahead, best);
+    }
+    if (advances) r.load_window();
+    const unsigned long long key = warp_max_key(best_key_of(best));
+    if (lane == 0) {
+        uint32_t slot, bar;
+        asm volatile("mapa.shared::cluster.u32 %0, %1, 0;" : "=r"(slot) : "r"(smem_addr(&s_key[rank * warps + warp])));
+        asm volatile("mapa.shared::cluster.u32 %0, %1, 0;" : "=r"(bar) : "r"(bar_keys));
+        // an asynchronous store that counts its bytes on the mbarrier: a releasing arrival
+        // would first wait for this warp's stores to the logits (1,200 cycles)
+        asm volatile("st.async.shared::cluster.mbarrier::complete_tx::bytes.u64 [%0], %1, [%2];" ::"r"(slot), "l"(key), "r"(bar)
+                     : "memory");
+    }
+    if (!advances) return;
+    r.place_window();
+    const int e_top = __shfl_sync(FULL, r.memo_top, 0);
+    int fr_top = -1;
+    if (r.memo) fr_top = __ldg(T.bu + min(max(e_top, 0), T.bu_len - 1)).x;
+    bool ok = __all_sync(FULL, mbar_wait0_cluster(bar_keys, 1 << 24));
+    if (ok) {
+        unsigned long long k = 0ull;
+        for (int i = lane; i < csize * warps; i += 32) k = s_key[i] > k ? s_key[i] : k;
+        k = warp_max_key(k);
+        r.tok = k ? (int32_t)(~(uint32_t)k) : -1;
+        r.load_token();
+        if (lane == 0) tokens_out[b] = r.tok;
+        r.judge();
+    }
+    ok = __all_sync(FULL, mbar_wait0(bar_tables, 1 << 24)) && ok;
+    if (!ok) {
+        // a key or the tables did not arrive: LIMIT status; wait (bounded) for what is in flight
+        if (lane == 0) {
+            atomicAdd(&g_pipeline_timeouts, 1);
+            if (S.fault) atomicAdd(S.fault, 1);
+        }
+        r.give_up(status_out);
+        mbar_wait0(bar_tables, 1 << 24);
+        mbar_wait0_cluster(bar_keys, 1 << 24);
+        return;
+    }
+    r.finish(smem_addr(sm), FULL, fr_top, status_out);
 }
 
 // out[b][:] = masks[mid[b]][:]: a warp takes FILL_SPAN neighbouring 32-word chunks of a
@@ -1659,7 +1799,7 @@ psc_status launch_choose(const T* logits, int64_t stride, const psc_handle* h, c
                          int32_t* d_tokens, cudaStream_t cs) {
     int chunks = (V + 32 + 1023) / 1024;
     int csize = 1;
-    while (csize < CHOOSE_CLUSTER && (long)B * csize < 4L * sm_count(h->device) && csize * 8 < chunks) csize *= 2;
+    while (csize < CHOOSE_CLUSTER && (long)B * csize < 4L * h->sms && csize * 8 < chunks) csize *= 2;
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3((unsigned)(B * csize));
     cfg.blockDim = dim3(256);
@@ -1681,12 +1821,20 @@ AdvanceKernel advance_kernel(const DevTables& d) {
     return d.adv_packed ? k_advance_warp<true, false> : k_advance_warp<false, false>;
 }
 
+using RowKernel = void (*)(uint16_t*, int64_t, MaskSrc, DevTables, DevStates, int, int, int32_t*, int32_t*);
+template <bool ANY>
+RowKernel row_kernel(const DevTables& d) {
+    if (d.adv_comb) return d.adv_packed ? k_decode_row<true, true, ANY> : k_decode_row<false, true, ANY>;
+    return d.adv_packed ? k_decode_row<true, false, ANY> : k_decode_row<false, false, ANY>;
+}
+
 psc_status launch_advance(const psc_handle* h, psc_states* st, const int32_t* d_tokens, int32_t* d_row_status,
                           int32_t* d_tokens_out, cudaStream_t cs) {
     int B = st->d.B;
     int from_keys = d_tokens_out ? 1 : 0;
     int early = from_keys && st->after_mask ? 1 : 0;
     st->after_mask = false;
+    if (from_keys) st->keys = false;
     psc_status s;
     if (h->d.adv_bytes > 0) {
         s = launch_pdl(advance_kernel(h->d),
@@ -1750,6 +1898,56 @@ psc_status launch_fused(const psc_handle* h, const psc_states* st, void* d_logit
     MaskSrc M{nullptr, h->d.mchunks, h->d.mrows, st->d.mid, h->d.W, h->d.nch, d_bitmask_out};
     s = launch_mask<true, true>(d_logits, dtype, row_stride, M, B, V, st->d.best, cs);
     const_cast<psc_states*>(st)->after_mask = s == PSC_OK;
+    return s;
+}
+
+// A decode step in one kernel, for bf16 batches small enough that this step's CTAs and the
+// next one's (which set up and stage their tables meanwhile) are resident together, at no
+// more than ROW_WARPS warps per CTA; *done = false: not such a batch.  As many CTAs per row
+// as that allows with four warps each: one SM moves the logits of 32 chunks in 3,000 cycles
+// more than those of 16.  Decode steps replayed from a CUDA graph, two kernels / this one (us): one row x 32,000
+// 5.2 / 4.5, x 128,256 5.1 / 4.5, x 262,144 5.4 / 5.1; 4 x 262,144 6.6 / 6.2; 16 x 32,000 6.8
+// / 6.2; 64 x 32,000 9.4 / 9.3; called one by one from Python, one row x 32,000 8.1 / 6.2.  Past the rule: 8 x 262,144 (16 CTAs a row, no room for the
+// next step) 7.8 / 9.1, 16 x 262,144 (8 CTAs of 32 warps a row) 9.7 / 11.0, 16 x 50,257 with
+// the Java-sized tables (8 CTAs a row) 8.2 / 9.4.
+psc_status launch_decode_row(const psc_handle* h, psc_states* st, void* d_logits, psc_dtype dtype, int64_t row_stride,
+                             int V, uint32_t* d_bitmask_out, int32_t* d_tokens, int32_t* d_row_status, cudaStream_t cs,
+                             bool* done) {
+    *done = false;
+    if (dtype != PSC_BF16 || !h->row_sm_smem || st->keys) return PSC_OK;
+    const int B = st->d.B, lead = row_lead(d_logits, dtype, row_stride, B);
+    const long cpv = ((long)lead + V + 1023) / 1024;
+    int csize = 2 * h->row_cluster;
+    long warps, fit;
+    do {
+        csize /= 2;
+        warps = (cpv + csize - 1) / csize;
+        // resident CTAs: shared memory, and 64 registers per thread
+        fit = std::min<long>(std::min<long>(h->row_sm_smem / h->row_cta_smem, 1024 / (32 * warps)), 32) * h->sms;
+    } while (csize > 1 && (4L * csize > cpv || 2L * B * csize > fit));
+    if (warps > ROW_WARPS || 2L * B * csize > fit) return PSC_OK;
+    psc_status s = ensure_mid(h, st, cs);
+    if (s != PSC_OK) return s;
+    MaskSrc M{nullptr, h->d.mchunks, h->d.mrows, st->d.mid, h->d.W, h->d.nch, d_bitmask_out};
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3((unsigned)(B * csize));
+    cfg.blockDim = dim3((unsigned)(warps * 32));
+    cfg.dynamicSmemBytes = row_smem(h->d);
+    cfg.stream = cs;
+    cudaLaunchAttribute attr[2];
+    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[0].val.programmaticStreamSerializationAllowed = 1;
+    attr[1].id = cudaLaunchAttributeClusterDimension;
+    attr[1].val.clusterDim = {(unsigned)csize, 1u, 1u};
+    cfg.attrs = attr;
+    cfg.numAttrs = 2;
+    s = cuda_check(cudaLaunchKernelEx(&cfg, lead != 0 || V % 1024 != 0 ? row_kernel<true>(h->d) : row_kernel<false>(h->d),
+                                      (uint16_t*)d_logits, row_stride, M, h->d, st->d, V, csize, d_tokens, d_row_status),
+                   "k_decode_row");
+    st->gen++;
+    if (s == PSC_OK) st->mid_gen = st->gen;
+    st->after_mask = false;
+    *done = true;
     return s;
 }
 
@@ -2193,7 +2391,46 @@ psc_status upload_tables(std::unique_ptr<psc_handle>& h, int tables) {
             for (int i = 0; i < h->n_blocks; i++) cudaFree(h->blocks[i]);
             return s;
         }
+        if (d.adv_bytes > 0) {   // the same for the one-kernel step
+            int per_sm = 0, reserved = 0;
+            cudaDeviceGetAttribute(&per_sm, cudaDevAttrMaxSharedMemoryPerMultiprocessor, h->device);
+            cudaDeviceGetAttribute(&reserved, cudaDevAttrReservedSharedMemoryPerBlock, h->device);
+            for (auto k : {row_kernel<false>(d), row_kernel<true>(d)}) {
+                cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, h->device);
+                cudaFuncGetAttributes(&fa, k);
+                optin -= (int)fa.sharedSizeBytes;
+                if (optin < row_smem(d)) {
+                    per_sm = 0;
+                    break;
+                }
+                if ((s = cuda_check(cudaFuncSetAttribute(k, cudaFuncAttributeNonPortableClusterSizeAllowed, 1),
+                                    "cudaFuncSetAttribute(k_decode_row)")) != PSC_OK ||
+                    (s = cuda_check(cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, optin),
+                                    "cudaFuncSetAttribute(k_decode_row)")) != PSC_OK) {
+                    for (int i = 0; i < h->n_blocks; i++) cudaFree(h->blocks[i]);
+                    return s;
+                }
+                h->row_cta_smem = std::max(h->row_cta_smem, row_smem(d) + (int)fa.sharedSizeBytes + reserved);
+            }
+            h->row_sm_smem = per_sm;
+            // the largest cluster that this device runs with these tables
+            for (h->row_cluster = ROW_CLUSTER; per_sm && h->row_cluster > 1; h->row_cluster /= 2) {
+                cudaLaunchConfig_t cfg = {};
+                cfg.gridDim = dim3((unsigned)h->row_cluster);
+                cfg.blockDim = dim3(ROW_WARPS * 32);
+                cfg.dynamicSmemBytes = row_smem(d);
+                cudaLaunchAttribute attr[1];
+                attr[0].id = cudaLaunchAttributeClusterDimension;
+                attr[0].val.clusterDim = {(unsigned)h->row_cluster, 1u, 1u};
+                cfg.attrs = attr;
+                cfg.numAttrs = 1;
+                int n = 0;
+                if (cudaOccupancyMaxActiveClusters(&n, row_kernel<true>(d), &cfg) == cudaSuccess && n > 0) break;
+                cudaGetLastError();   // not an error of the caller's
+            }
+        }
     }
+    h->sms = sm_count(h->device);
     d.q0 = t.q0;
     d.nq = t.nq;
     d.n_lr = t.n_lr;
@@ -2367,13 +2604,14 @@ psc_status psc_state_copy(psc_states* dst, const psc_states* src, void* stream) 
     if (dev != dst->device) return fail_with(PSC_ERR_ARG, "psc_state_copy: current device differs from the states'");
     cudaStream_t cs = (cudaStream_t)stream;
     const size_t n16 = src->copy_bytes / 16;
-    int grid = (int)std::max<size_t>(1, std::min<size_t>((n16 + 255) / 256, (size_t)sm_count(dev) * 4));
+    int grid = (int)std::max<size_t>(1, std::min<size_t>((n16 + 255) / 256, (size_t)dst->h->sms * 4));
     psc_status s = launch_pdl(k_state_copy, dim3(grid), dim3(256), 0, cs, "k_state_copy", (const uint4*)src->base,
                               (uint4*)dst->base, n16);
     if (s != PSC_OK) return s;
     dst->gen++;
     dst->mid_gen = src->mid_gen == src->gen ? dst->gen : 0;   // the mask ids are as current as src's
     dst->after_mask = false;
+    dst->keys = src->keys;
     return PSC_OK;
 }
 
@@ -2383,6 +2621,7 @@ psc_status psc_state_reset(psc_states* st, const int32_t* d_rows, int32_t n, voi
     if (cnt < 0) return fail_with(PSC_ERR_ARG, "psc_state_reset: negative count");
     // the reset rows get the empty prefix's mask id: the mask ids stay current when they were
     const bool current = st->mid_gen == st->gen || !d_rows;
+    if (!d_rows) st->keys = false;
     st->gen++;
     st->after_mask = false;
     psc_status s = PSC_OK;
@@ -2467,6 +2706,7 @@ psc_status psc_fill_apply_argmax(const psc_handle* h, const psc_states* st, int3
     cudaStream_t cs = (cudaStream_t)stream;
     if ((s = launch_fused(h, st, d_logits, dtype, row_stride, V, d_bitmask_out, cs)) != PSC_OK) return s;
     const_cast<psc_states*>(st)->after_mask = false;
+    const_cast<psc_states*>(st)->keys = false;
     k_finalize_tokens<<<(B + 255) / 256, 256, 0, cs>>>(st->d.best, B, d_tokens);
     return launch_check("k_finalize_tokens");
 }
@@ -2480,6 +2720,9 @@ psc_status psc_decode_step(const psc_handle* h, psc_states* st, int32_t B, void*
         (dtype != PSC_F32 && dtype != PSC_BF16))
         return fail_with(PSC_ERR_ARG, "psc_decode_step: bad arguments");
     cudaStream_t cs = (cudaStream_t)stream;
+    bool done = false;
+    s = launch_decode_row(h, st, d_logits, dtype, row_stride, V, d_bitmask_out, d_tokens, d_row_status, cs, &done);
+    if (s != PSC_OK || done) return s;
     if ((s = launch_fused(h, st, d_logits, dtype, row_stride, V, d_bitmask_out, cs)) != PSC_OK) return s;
     return launch_advance(h, st, nullptr, d_row_status, d_tokens, cs);
 }
@@ -2491,7 +2734,9 @@ psc_status psc_decode_step_mask(const psc_handle* h, psc_states* st, int32_t B, 
     if (!st || st->h != h || B != st->d.B || !d_logits || V != h->d.V || row_stride < V ||
         (dtype != PSC_F32 && dtype != PSC_BF16))
         return fail_with(PSC_ERR_ARG, "psc_decode_step_mask: bad arguments");
-    return launch_fused(h, st, d_logits, dtype, row_stride, V, d_bitmask_out, (cudaStream_t)stream);
+    s = launch_fused(h, st, d_logits, dtype, row_stride, V, d_bitmask_out, (cudaStream_t)stream);
+    if (s == PSC_OK) st->keys = true;
+    return s;
 }
 
 psc_status psc_decode_step_advance(const psc_handle* h, psc_states* st, int32_t B, int32_t* d_tokens,

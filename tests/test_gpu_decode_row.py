@@ -1,0 +1,93 @@
+"""GPU: psc_decode_step on small batches (one kernel, a cluster of CTAs per row) against its two
+halves, psc_decode_step_mask and psc_decode_step_advance, on a copy of the batch: logits,
+masks, tokens, statuses and states over several steps, at row lengths around the cluster
+sizes and where a row does not start on a 16-byte boundary."""
+from __future__ import annotations
+
+import numpy as np
+import pytest
+
+from workloads import grammars, sample
+
+torch = pytest.importorskip("torch")
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module")
+def psc():
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    from paper_2608_03065_gb300 import build, psc as mod
+    build.build()
+    mod.load()
+    return mod
+
+
+def _vocabulary(g, V):
+    rng = np.random.default_rng(V)
+    text = b" ".join(sample.SentenceSampler(g, max_depth=30).text(rng, 2048)[0] for _ in range(8))
+    toks = dict.fromkeys(list(sample.PRINTABLE) + [m.group(0) for m in sample.PRETOKEN.finditer(text)])
+    while len(toks) < V:
+        toks[bytes(rng.integers(97, 123, int(rng.integers(2, 9))).astype(np.uint8))] = None
+    return list(toks)[:V - 1] + [b""]
+
+
+@pytest.mark.parametrize("grammar,options", [("json_grammar", {}), ("json_grammar", {"packed_tables": True}),
+                                             ("c_like", {}), ("c_like", {"packed_tables": True, "bottom_up": False})])
+@pytest.mark.parametrize("V,batches", [(300, (1, 70)), (1024, (3,)), (1030, (2, 33)), (9001, (1, 5)), (32768, (1, 16)),
+                                       (50257, (2,)), (200000, (1, 4)), (262144, (1,))])
+def test_one_kernel_step_equals_two(psc, grammar, options, V, batches):
+    g = getattr(grammars, grammar)()
+    h = psc.psc_compile(g.text(), _vocabulary(g, V), V - 1, **options)
+    for B in batches:
+        for off, ld in ((0, V), (0, -(-V // 64) * 64), (3, V + 5)):
+            gen = torch.Generator(device="cuda").manual_seed(V + off + B)
+            one, two = psc.psc_state_init(h, B, 256), psc.psc_state_init(h, B, 256)
+            for step in range(5):
+                x = torch.randn(off + B * ld + 64, generator=gen, device="cuda").bfloat16()
+                if step == 3:
+                    x[off + (B - 1) * ld:off + (B - 1) * ld + V] = float("nan")    # the last row chooses nothing
+                y = x.clone()
+                outs = []
+                for st, buf in ((one, x), (two, y)):
+                    lg = buf.as_strided((B, V), (ld, 1), off)
+                    bm = torch.full((B, h.W), -1, dtype=torch.int32, device="cuda")
+                    tok = torch.full((B,), -7, dtype=torch.int32, device="cuda")
+                    status = torch.full((B,), -7, dtype=torch.int32, device="cuda")
+                    if st is one:
+                        psc.psc_decode_step(h, st, lg, tok, bm, status)
+                    else:
+                        psc.psc_decode_step_mask(h, st, lg, bm)
+                        psc.psc_decode_step_advance(h, st, tok, status)
+                    outs.append((tok, bm, status))
+                assert torch.equal(x.view(torch.int16), y.view(torch.int16)), (B, off, step)
+                for a, b in zip(*outs):
+                    assert torch.equal(a, b), (B, off, step)
+                assert (outs[0][0][-1].item() == -1) == (step == 3)
+                a, b = psc.psc_states_download(one), psc.psc_states_download(two)
+                for k in ("q", "depth", "status"):
+                    np.testing.assert_array_equal(a[k], b[k])
+                for r in range(B):
+                    np.testing.assert_array_equal(a["stack"][r, :a["depth"][r]], b["stack"][r, :b["depth"][r]])
+            assert psc.psc_state_faults(one) == 0
+
+
+def test_step_after_an_unconsumed_mask_pass(psc):
+    """Choices that psc_decode_step_mask left are merged with the step's, as its two halves do."""
+    g = grammars.json_grammar()
+    V = 2000
+    h = psc.psc_compile(g.text(), _vocabulary(g, V), V - 1)
+    gen = torch.Generator(device="cuda").manual_seed(1)
+    x = [torch.randn(2, V, generator=gen, device="cuda").bfloat16() for _ in range(2)]
+    tokens = []
+    for halves in (False, True):
+        st = psc.psc_state_init(h, 2, 64)
+        tok = torch.zeros(2, dtype=torch.int32, device="cuda")
+        psc.psc_decode_step_mask(h, st, x[0].clone())
+        if halves:
+            psc.psc_decode_step_mask(h, st, x[1].clone())
+            psc.psc_decode_step_advance(h, st, tok)
+        else:
+            psc.psc_decode_step(h, st, x[1].clone(), tok)
+        tokens.append(tok)
+    assert torch.equal(*tokens)
