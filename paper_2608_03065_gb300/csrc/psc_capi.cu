@@ -73,6 +73,8 @@ struct DevTables {
     const int64_t* vocab_off;
     const uint8_t* tok32;      // [V][32] tokens of up to 31 bytes: the bytes, zeros, the length in the last one;
                                // longer ones: their first 31 bytes, then 255
+    const uint16_t* tok_lex;   // [V][16] the lexemes of every token from its first byte on, none pending:
+                               // what they are (TokLex), the pending lexer state after it, the classes
     int q0, nq, n_lr, n_terms, n_nts, end_term;
     int V, W, nch, eos_id, n_masks;
     // compact lexer/parser tables for k_advance_warp (adv_bytes = 0: not built)
@@ -91,6 +93,10 @@ struct DevTables {
     const int32_t* bu_F;      // [n_frow][nq] mask ids
     int bu_len, n_frow;
 };
+
+// tok_lex[v][0]: how many classes the token emits (at most TOK_LEX_CLASSES), or why there are none
+constexpr int TOK_LEX_CLASSES = 14;
+enum TokLex { TOK_LEX_REJECTED = 254, TOK_LEX_LONG = 255 };   // a byte fits no lexeme; not held
 
 struct DevStates {
     int32_t* q;
@@ -1178,8 +1184,9 @@ __device__ __forceinline__ int warp_memo_extend(const DevTables& T, const StackV
 // masking pass 8,500 / 7,500): the row's state and token in one round trip, the token's
 // record (bytes and length), mask chunk and stack window in the next (2,100-3,900 before,
 // when the window took a trip per 32 entries and the mask word was waited for; 1,600-2,600
-// now), lexing (two dependent shared reads and a divergent branch per byte before, one read
-// now), parsing (up to 5,000), edge slots and blocks of the entries written (loads in
+// now), lexing (two dependent shared reads and a divergent branch per byte and a walk over the
+// lexemes before, 1,000-1,900; now one read per byte of the pending lexeme and, when that ends
+// at the token's start, the token's own lexemes from its record, 600-950), parsing (up to 5,000), edge slots and blocks of the entries written (loads in
 // flight during the write-back), the mask id (two loads before, one now: a block's final
 // row comes with the block).
 template <bool PACKED, bool COMB>
@@ -1195,6 +1202,7 @@ struct RowAdvance {
     int mid = 0;             // the row's mask id
     int memo_top = -1;       // lane l: the kept block of the stack without its top l entries
     int tbyte = 0;           // lane i: byte i of the token (lane 31: its length)
+    int tlex = 0;            // lane i: word i % 16 of the token's lexemes
     uint32_t mchunk = 0;     // the mask chunk that holds the token's bit
     uint4 wv = make_uint4(0u, 0u, 0u, 0u);
     bool live = false, parse = false, eos = false;
@@ -1232,7 +1240,10 @@ struct RowAdvance {
     // The loads that need only the token (tok set), and with the row's status known the
     // chunk of its mask that holds the token's bit (unless the token is known to be allowed).
     __device__ __forceinline__ void load_token() {
-        if (tok >= 0 && tok < T.V) tbyte = T.tok32[(size_t)tok * 32 + lane];
+        if (tok >= 0 && tok < T.V) {
+            tbyte = T.tok32[(size_t)tok * 32 + lane];
+            tlex = T.tok_lex[(size_t)tok * 16 + (lane & 15)];
+        }
     }
     __device__ __forceinline__ void load_mask_chunk() {
         if (tok >= 0 && tok < T.V && status == ROW_OK) mchunk = __ldg(T.mrows + (size_t)mid * T.nch + (tok >> 10));
@@ -1310,60 +1321,84 @@ struct RowAdvance {
         const int len = __shfl_sync(FULL, tbyte, 31);
         int ncls = -1;   // classes at la; -1: the token is lexed by lane 0 (longer than 31 bytes)
         if (len <= 31) {
-            // Lexing in parallel (the lexer does not depend on the parser): lane j runs the
-            // lexer DFA over the lexeme that starts afresh at byte j (ls, ending at le), every
-            // lane over the row's pending lexeme from the first byte on (ps, ending at pe); an
-            // end is the byte that a lexeme cannot take, or the token's.  The lanes go in
-            // step, the bytes' classes coming by shuffles, so a byte costs one dependent
-            // shared-memory read (a lane that has stopped, or a position past the token,
-            // reads on without effect).
+            // The lexer does not depend on the parser.  The row's pending lexeme first: every
+            // lane runs it over the token's bytes (ps, up to byte pe), the bytes' classes
+            // coming by shuffles, so that a byte costs one dependent shared-memory read.
             const int cls_of = lds_u8(A.bc + tbyte);   // lane i: the class of byte i
-            int ls = A.q0, le = lane, ps = q, pe = 0;
-            bool run = lane < len, prun = len > 0;
-            for (int k = 0; k < len; k += 4) {
-                int c[4], pc[4];
-#pragma unroll
-                for (int i = 0; i < 4; i++) {
-                    c[i] = __shfl_down_sync(FULL, cls_of, k + i);
-                    pc[i] = __shfl_sync(FULL, cls_of, k + i);
-                }
-#pragma unroll
-                for (int i = 0; i < 4; i++) {
-                    int nx = lds_s16(A.trans + ls * A.trans_row + 2u * c[i]);
-                    int px = lds_s16(A.trans + ps * A.trans_row + 2u * pc[i]);
-                    run = run && nx >= 0 && lane + k + i < len;
-                    prun = prun && px >= 0 && k + i < len;
-                    ls = run ? nx : ls;
-                    le += run ? 1 : 0;
-                    ps = prun ? px : ps;
-                    pe += prun ? 1 : 0;
-                }
-            }
-            // each lane's lexeme: its end, whether it is ignored, ends the token, or is none
-            // (no byte taken, or incomplete), and its class; then the lexemes are followed
-            // from one end to the next, the pending one first
-            constexpr uint32_t IGN = 64u, LAST = 128u, NONE = 256u;
-            auto lexeme_of = [&](int state, int end, bool some) -> uint32_t {
-                int a = lds_s16(A.acc + 2u * state);
-                return (uint32_t)end | (end == len ? LAST : a < 0 || !some ? NONE : 0u) | (a & 1 ? IGN : 0u) |
-                       (uint32_t)(a >> 1) << 16;
-            };
-            const uint32_t fresh = lexeme_of(ls, le, le > lane);
-            uint32_t lx = q == A.q0 ? __shfl_sync(FULL, fresh, 0) : lexeme_of(ps, pe, true);
-            int pos = 0;
-            bool pending = q != A.q0;
+            int ps = q, pe = 0;
             ncls = 0;
-            while (!(lx & (LAST | NONE))) {   // warp-uniform
-                if (!(lx & IGN)) {
-                    if (lane == 0) sts_u16(la + 2u * ncls, (int)(lx >> 16));
-                    ncls++;
+            bool fresh_from = q == A.q0;   // the rest of the token starts a lexeme of its own
+            if (!fresh_from) {
+                int c = __shfl_sync(FULL, cls_of, 0);
+                while (pe < len) {
+                    const int cn = __shfl_sync(FULL, cls_of, pe + 1);
+                    const int px = lds_s16(A.trans + ps * A.trans_row + 2u * c);
+                    if (px < 0) break;
+                    ps = px;
+                    c = cn;
+                    pe++;
                 }
-                pos = (int)(lx & 63u);
-                pending = false;
-                lx = __shfl_sync(FULL, fresh, pos);
+                if (pe == len) {
+                    nq = ps;   // it stays pending
+                } else {
+                    const int a = lds_s16(A.acc + 2u * ps);
+                    if (a < 0) status = ROW_REJECTED;
+                    else fresh_from = true;
+                    if (a >= 0 && !(a & 1)) {
+                        if (lane == 0) sts_u16(la, a >> 1);
+                        ncls = 1;
+                    }
+                }
             }
-            if (lx & LAST) nq = pending ? ps : __shfl_sync(FULL, ls, pos & 31);   // the last lexeme stays pending
-            else status = ROW_REJECTED;
+            const int held = __shfl_sync(FULL, tlex, 0);
+            if (fresh_from && pe == 0 && held != TOK_LEX_LONG) {
+                // the whole token lexed afresh: the same for every row, so it is in the token's record
+                nq = __shfl_sync(FULL, tlex, 1);
+                if (held == TOK_LEX_REJECTED) {
+                    status = ROW_REJECTED;
+                } else {
+                    if (lane >= 2 && lane < 2 + held) sts_u16(la + 2u * (ncls + lane - 2), tlex);
+                    ncls += held;
+                }
+            } else if (fresh_from) {
+                // lexing in parallel: lane j runs the lexer DFA over the lexeme that starts at
+                // byte j (ls, ending at le: the byte that it cannot take, or the token's end);
+                // the lanes go in step (one that has stopped, or a position past the token,
+                // reads on without effect)
+                int ls = A.q0, le = lane;
+                bool run = lane < len;
+                for (int k = 0; k < len - pe; k += 4) {
+                    int c[4];
+#pragma unroll
+                    for (int i = 0; i < 4; i++) c[i] = __shfl_down_sync(FULL, cls_of, k + i);
+#pragma unroll
+                    for (int i = 0; i < 4; i++) {
+                        int nx = lds_s16(A.trans + ls * A.trans_row + 2u * c[i]);
+                        run = run && nx >= 0 && lane + k + i < len;
+                        ls = run ? nx : ls;
+                        le += run ? 1 : 0;
+                    }
+                }
+                // each lane's lexeme: its end, whether it is ignored, ends the token, or is
+                // none (no byte taken, or incomplete), and its class; then the lexemes are
+                // followed from one end to the next
+                constexpr uint32_t IGN = 64u, LAST = 128u, NONE = 256u;
+                const int a = lds_s16(A.acc + 2u * ls);
+                const uint32_t lexeme = (uint32_t)le | (le == len ? LAST : a < 0 || le == lane ? NONE : 0u) |
+                                        (a & 1 ? IGN : 0u) | (uint32_t)(a >> 1) << 16;
+                int pos = pe;
+                uint32_t lx = __shfl_sync(FULL, lexeme, pos);
+                while (!(lx & (LAST | NONE))) {   // warp-uniform
+                    if (!(lx & IGN)) {
+                        if (lane == 0) sts_u16(la + 2u * ncls, (int)(lx >> 16));
+                        ncls++;
+                    }
+                    pos = (int)(lx & 63u);
+                    lx = __shfl_sync(FULL, lexeme, pos);
+                }
+                if (lx & LAST) nq = __shfl_sync(FULL, ls, pos);   // the last lexeme stays pending
+                else status = ROW_REJECTED;
+            }
         }
         __syncwarp();
         if (lane == 0) {
@@ -2301,6 +2336,35 @@ std::vector<uint8_t> token_records(const psc::Tables& t) {
     return out;
 }
 
+// Every token's lexemes from its first byte on with none pending ([V][16], see DevTables:
+// tok_lex): the row-independent part of lexing, done once.
+std::vector<uint16_t> token_lexemes(const psc::Tables& t) {
+    std::vector<uint16_t> out((size_t)t.V * 16, 0);
+    for (int v = 0; v < t.V; v++) {
+        uint16_t* w = out.data() + (size_t)v * 16;
+        const int64_t lo = t.vocab_off[v], hi = t.vocab_off[v + 1];
+        int q = t.q0, n = 0;
+        w[0] = hi - lo > 31 ? TOK_LEX_LONG : 0;
+        for (int64_t i = lo; i < hi && w[0] == 0; i++) {
+            const int c = t.vocab_bytes[i];
+            int nx = t.lex_trans[(size_t)q * 256 + c];
+            if (nx < 0) {   // the lexeme ends before this byte, which starts the next one
+                const int cls = q == t.q0 ? -1 : t.lex_accept[q];
+                nx = cls < 0 ? -1 : t.lex_trans[(size_t)t.q0 * 256 + c];
+                if (nx < 0) w[0] = TOK_LEX_REJECTED;
+                else if (!t.cls_ignored[cls]) {
+                    if (n == TOK_LEX_CLASSES) w[0] = TOK_LEX_LONG;
+                    else w[2 + n++] = (uint16_t)cls;
+                }
+            }
+            q = nx;
+        }
+        if (w[0] == 0) w[0] = (uint16_t)n;
+        w[1] = (uint16_t)std::max(q, 0);
+    }
+    return out;
+}
+
 // The bottom-up classifier's blocks with every successor's final row beside it (the mask
 // lookup after the last stack entry read then needs one load less).
 std::vector<int2> bottom_up_blocks(const psc::Tables& t) {
@@ -2361,7 +2425,8 @@ psc_status upload_tables(std::unique_ptr<psc_handle>& h, int tables) {
         (s = upload(h.get(), dfa_mask, &d.dfa_mask)) || (s = upload(h.get(), t.mask_chunks, &d.mchunks)) ||
         (s = upload(h.get(), t.mask_rows, &d.mrows)) ||
         (s = upload(h.get(), t.vocab_bytes, &d.vocab, 16)) || (s = upload(h.get(), t.vocab_off, &d.vocab_off)) ||
-        (s = upload(h.get(), token_records(t), &d.tok32))) {
+        (s = upload(h.get(), token_records(t), &d.tok32)) ||
+        (s = upload(h.get(), token_lexemes(t), &d.tok_lex))) {
         for (int i = 0; i < h->n_blocks; i++) cudaFree(h->blocks[i]);
         return s;
     }

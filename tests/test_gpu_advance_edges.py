@@ -32,6 +32,7 @@ def test_long_tokens_and_deep_stacks(psc, tables, bottom_up, cap):
     for n in lengths:
         toks += [b"[" * n, b"]" * n, b"a" * n, b"1" * n, b" " * n, b'"' + b"b" * (n - 1), b'b"' + b"," + b"1" * n,
                  b"1," * n, b"[1]," * (n // 2 + 1), b'["' + b"a" * n + b'"']
+    toks += [b"[" * n for n in (13, 14, 15, 16)] + [b" [" * 14, b"[ " * 15, b"x1", b"1x", b"[x", b"1,x"]
     toks = list(dict.fromkeys(toks)) + [b""]
     V = len(toks)
     h = psc.psc_compile(grammars.json_grammar().text(), toks, V - 1, packed_tables=tables == "packed", bottom_up=bottom_up)
