@@ -951,7 +951,8 @@ struct AdvTabs {
 // of one-symbol reductions takes a short loop (one action and one goto lookup
 // each, the goto row of `below` fixed for the run) and the new top is written
 // to the stack once, when the run ends (not at all when a longer reduction then
-// pops it).
+// pops it).  A missing GOTO is the state n_lr, whose ACTION row is all errors: the
+// loops need not test for it.
 template <bool PACKED>
 __device__ __forceinline__ int feed_class_win(const AdvTabs& A, StackView& sv, int& depth, int& top, int& below,
                                               int cap, int cls) {
@@ -959,22 +960,21 @@ __device__ __forceinline__ int feed_class_win(const AdvTabs& A, StackView& sv, i
     if (t < 0) return ROW_REJECTED;
     const uint32_t col = A.act + 2u * t;   // ACTION[.][t]
     bool dirty = false;                     // top changed by one-symbol reductions, not yet on the stack
-    for (int guard = 0; guard < 4 * cap + 64; guard++) {
-        int a = lds_s16(col + top * A.act_row);
-        if (PACKED) {
-            // packed unit reduction: kind REDUCE, rule length 1 (bits 12-15), lhs in bits 2-11
+    int left = 4 * cap + 64;                // reductions left
+    int a = lds_s16(col + top * A.act_row);
+    for (;;) {
+        if (PACKED && (a & 0xF003) == 0x1002 && depth >= 2) {
+            // packed unit reductions: kind REDUCE, rule length 1 (bits 12-15), lhs in bits 2-11
             const uint32_t go_below = A.go + below * A.go_row;
-            while ((a & 0xF003) == 0x1002 && depth >= 2) {
-                int g = lds_s16(go_below + ((a >> 1) & 0x7FE));   // GOTO[below][lhs], 2 * lhs = (a >> 1) & 0x7FE
-                if (g < 0) return ROW_REJECTED;
-                if (++guard >= 4 * cap + 64) return ROW_LIMIT;
-                top = g;
-                dirty = true;
+            do {
+                top = lds_s16(go_below + ((a >> 1) & 0x7FE));   // GOTO[below][lhs], 2 * lhs = (a >> 1) & 0x7FE
                 a = lds_s16(col + top * A.act_row);
-            }
+            } while (--left > 0 && (a & 0xF003) == 0x1002);
+            dirty = true;
         }
-        int kind = a & 3, val = (a >> 2) & 0x3FFF;
-        if (kind == psc::ACT_SHIFT) {
+        const int kind = a & 3, val = (a >> 2) & 0x3FFF;
+        if (kind != psc::ACT_REDUCE) {
+            if (kind != psc::ACT_SHIFT) return ROW_REJECTED;
             if (depth >= cap) return ROW_OVERFLOW;
             if (dirty) sv.set(depth - 1, top);
             sv.set(depth++, val);
@@ -982,7 +982,7 @@ __device__ __forceinline__ int feed_class_win(const AdvTabs& A, StackView& sv, i
             top = val;
             return ROW_OK;
         }
-        if (kind != psc::ACT_REDUCE) return ROW_REJECTED;
+        if (--left < 0) return ROW_LIMIT;
         int k, lhs;
         if (PACKED) {
             k = val >> 10;
@@ -995,20 +995,17 @@ __device__ __forceinline__ int feed_class_win(const AdvTabs& A, StackView& sv, i
         if (k == 0 && dirty) sv.set(depth - 1, top);   // an empty rule pushes above the current top
         dirty = false;
         depth -= k;
+        if (depth >= cap) return ROW_OVERFLOW;
         // the entry the reduction uncovers: the one below the top (k = 1), the top
         // itself (k = 0), else read from the stack
         int under;
-        if (k == 1) under = below;
-        else if (k == 0) under = top;
-        else under = sv.get(depth - 1);
-        int g = lds_s16(A.go + under * A.go_row + 2u * lhs);
-        if (g < 0) return ROW_REJECTED;
-        if (depth >= cap) return ROW_OVERFLOW;
-        sv.set(depth++, g);
+        if (k >= 2) under = sv.get(depth - 1);
+        else under = k == 1 ? below : top;
+        top = lds_s16(A.go + under * A.go_row + 2u * lhs);
         below = under;
-        top = g;
+        a = lds_s16(col + top * A.act_row);
+        sv.set(depth++, top);
     }
-    return ROW_LIMIT;
 }
 
 // Entry x of a packed table's row (w = the state's word, row id << 17 | base): the
@@ -1039,22 +1036,22 @@ __device__ __forceinline__ int feed_class_comb(const AdvTabs& A, StackView& sv, 
     }
     if (t < 0) return ROW_REJECTED;
     bool dirty = false;
-    for (int guard = 0; guard < 4 * cap + 64; guard++) {
-        if (guard > 0) a = comb_get(A.acmb, tw, t, 0);
+    int left = 4 * cap + 64;
+    for (;;) {
         if (PACKED && (a & 0xF003) == 0x1002 && depth >= 2) {
             const uint32_t bw = lds_u32(A.gbase + 4u * below);
             do {   // one-symbol reductions: GOTO[below][lhs], lhs in bits 2-11
                 int g = comb_get(A.gcmb, bw, (a >> 2) & 1023, -1);
                 if (g < 0) return ROW_REJECTED;
-                if (++guard >= 4 * cap + 64) return ROW_LIMIT;
                 top = g;
-                dirty = true;
                 tw = lds_u32(A.abase + 4u * top);
                 a = comb_get(A.acmb, tw, t, 0);
-            } while ((a & 0xF003) == 0x1002);
+            } while (--left > 0 && (a & 0xF003) == 0x1002);
+            dirty = true;
         }
-        int kind = a & 3, val = (a >> 2) & 0x3FFF;
-        if (kind == psc::ACT_SHIFT) {
+        const int kind = a & 3, val = (a >> 2) & 0x3FFF;
+        if (kind != psc::ACT_REDUCE) {
+            if (kind != psc::ACT_SHIFT) return ROW_REJECTED;
             if (depth >= cap) return ROW_OVERFLOW;
             if (dirty) sv.set(depth - 1, top);
             sv.set(depth++, val);
@@ -1062,7 +1059,7 @@ __device__ __forceinline__ int feed_class_comb(const AdvTabs& A, StackView& sv, 
             top = val;
             return ROW_OK;
         }
-        if (kind != psc::ACT_REDUCE) return ROW_REJECTED;
+        if (--left < 0) return ROW_LIMIT;
         int k, lhs;
         if (PACKED) {
             k = val >> 10;
@@ -1075,19 +1072,18 @@ __device__ __forceinline__ int feed_class_comb(const AdvTabs& A, StackView& sv, 
         if (k == 0 && dirty) sv.set(depth - 1, top);
         dirty = false;
         depth -= k;
+        if (depth >= cap) return ROW_OVERFLOW;
         int under;
-        if (k == 1) under = below;
-        else if (k == 0) under = top;
-        else under = sv.get(depth - 1);
+        if (k >= 2) under = sv.get(depth - 1);
+        else under = k == 1 ? below : top;
         int g = comb_get(A.gcmb, lds_u32(A.gbase + 4u * under), lhs, -1);
         if (g < 0) return ROW_REJECTED;
-        if (depth >= cap) return ROW_OVERFLOW;
-        sv.set(depth++, g);
         below = under;
         top = g;
         tw = lds_u32(A.abase + 4u * top);
+        a = comb_get(A.acmb, tw, t, 0);
+        sv.set(depth++, g);
     }
-    return ROW_LIMIT;
 }
 
 template <bool PACKED, bool COMB>
@@ -2113,7 +2109,7 @@ std::vector<uint8_t> build_advance_blob(const psc::Tables& t, DevTables& d, int 
     d.o_trans = take((size_t)t.nq * nbc * 2);
     d.o_accept = take((size_t)t.nq * 2);
     d.o_resolve = take((size_t)std::max(ncls, 1) * t.n_lr * 2);
-    d.o_action = take((size_t)t.n_lr * t.n_terms * 2);
+    d.o_action = take((size_t)(t.n_lr + 1) * t.n_terms * 2);   // the last row: no actions (a missing GOTO leads there)
     d.o_go = take((size_t)t.n_lr * t.n_nts * 2);
     d.o_rlen = take((size_t)n_rules);
     d.o_rlhs = take((size_t)n_rules * 2);
@@ -2288,7 +2284,7 @@ std::vector<uint8_t> build_advance_blob(const psc::Tables& t, DevTables& d, int 
     // a reduce entry carries its rule's length and left-hand side when they fit in 14 bits
     // (one dependent shared-memory read less per reduction)
     for (size_t i = 0; i < t.action.size(); i++) put16(d.o_action, i, enc_action(t.action[i]));
-    for (size_t i = 0; i < t.go.size(); i++) put16(d.o_go, i, t.go[i]);
+    for (size_t i = 0; i < t.go.size(); i++) put16(d.o_go, i, t.go[i] >= 0 ? t.go[i] : t.n_lr);
     for (int r = 0; r < n_rules; r++) {
         blob[d.o_rlen + r] = (uint8_t)t.rule_len[r];
         put16(d.o_rlhs, r, t.rule_lhs[r]);
