@@ -71,10 +71,10 @@ struct DevTables {
     const uint32_t* mrows;     // mask rows as chunk ids [n_masks][nch]
     const uint8_t* vocab;
     const int64_t* vocab_off;
-    const uint8_t* tok32;      // [V][32] tokens of up to 31 bytes: the bytes, zeros, the length in the last one;
-                               // longer ones: their first 31 bytes, then 255
-    const uint16_t* tok_lex;   // [V][16] the lexemes of every token from its first byte on, none pending:
-                               // what they are (TokLex), the pending lexer state after it, the classes
+    const uint8_t* tok_rec;    // [V][64] a record per token.  Bytes 0-31: tokens of up to 31 bytes: the bytes,
+                               // zeros, the length in the last one; longer ones: their first 31 bytes, then
+                               // 255.  Then 16 uint16: the lexemes of the token from its first byte on, none
+                               // pending: what they are (TokLex), the pending lexer state after it, the classes
     int q0, nq, n_lr, n_terms, n_nts, end_term;
     int V, W, nch, eos_id, n_masks;
     // compact lexer/parser tables for k_advance_warp (adv_bytes = 0: not built)
@@ -94,7 +94,7 @@ struct DevTables {
     int bu_len, n_frow;
 };
 
-// tok_lex[v][0]: how many classes the token emits (at most TOK_LEX_CLASSES), or why there are none
+// the first word of a record's lexemes: how many classes the token emits (at most TOK_LEX_CLASSES), or why there are none
 constexpr int TOK_LEX_CLASSES = 14;
 enum TokLex { TOK_LEX_REJECTED = 254, TOK_LEX_LONG = 255 };   // a byte fits no lexeme; not held
 
@@ -1197,8 +1197,7 @@ struct RowAdvance {
     int tok = -1, status = ROW_OK, q = 0, depth = 0, depth0 = 0;
     int mid = 0;             // the row's mask id
     int memo_top = -1;       // lane l: the kept block of the stack without its top l entries
-    int tbyte = 0;           // lane i: byte i of the token (lane 31: its length)
-    int tlex = 0;            // lane i: word i % 16 of the token's lexemes
+    int rec = 0;             // the token's record, two bytes per lane
     uint32_t mchunk = 0;     // the mask chunk that holds the token's bit
     uint4 wv = make_uint4(0u, 0u, 0u, 0u);
     bool live = false, parse = false, eos = false;
@@ -1236,10 +1235,7 @@ struct RowAdvance {
     // The loads that need only the token (tok set), and with the row's status known the
     // chunk of its mask that holds the token's bit (unless the token is known to be allowed).
     __device__ __forceinline__ void load_token() {
-        if (tok >= 0 && tok < T.V) {
-            tbyte = T.tok32[(size_t)tok * 32 + lane];
-            tlex = T.tok_lex[(size_t)tok * 16 + (lane & 15)];
-        }
+        if (tok >= 0 && tok < T.V) rec = __ldg(reinterpret_cast<const uint16_t*>(T.tok_rec + (size_t)tok * 64) + lane);
     }
     __device__ __forceinline__ void load_mask_chunk() {
         if (tok >= 0 && tok < T.V && status == ROW_OK) mchunk = __ldg(T.mrows + (size_t)mid * T.nch + (tok >> 10));
@@ -1314,7 +1310,8 @@ struct RowAdvance {
     }
     __device__ __forceinline__ void lex_and_parse(const AdvTabs A, uint32_t mword) {
         int nq = q, nd = depth;
-        const int len = __shfl_sync(FULL, tbyte, 31);
+        const int tbyte = (__shfl_sync(FULL, rec, lane >> 1) >> ((lane & 1) * 8)) & 0xFF;   // lane i: byte i of the token
+        const int len = __shfl_sync(FULL, rec, 15) >> 8;
         int ncls = -1;   // classes at la; -1: the token is lexed by lane 0 (longer than 31 bytes)
         if (len <= 31) {
             // The lexer does not depend on the parser.  The row's pending lexeme first: every
@@ -1346,14 +1343,14 @@ struct RowAdvance {
                     }
                 }
             }
-            const int held = __shfl_sync(FULL, tlex, 0);
+            const int held = __shfl_sync(FULL, rec, 16);
             if (fresh_from && pe == 0 && held != TOK_LEX_LONG) {
                 // the whole token lexed afresh: the same for every row, so it is in the token's record
-                nq = __shfl_sync(FULL, tlex, 1);
+                nq = __shfl_sync(FULL, rec, 17);
                 if (held == TOK_LEX_REJECTED) {
                     status = ROW_REJECTED;
                 } else {
-                    if (lane >= 2 && lane < 2 + held) sts_u16(la + 2u * (ncls + lane - 2), tlex);
+                    if (lane >= 18 && lane < 18 + held) sts_u16(la + 2u * (ncls + lane - 18), rec);
                     ncls += held;
                 }
             } else if (fresh_from) {
@@ -2320,27 +2317,20 @@ psc_status noalloc_scratch(int device, int32_t** out) {
 }  // namespace
 
 namespace {
-// One 32-byte record per token ([V][32]): its bytes and, in the last byte, its length (255:
-// longer than 31 bytes), so that the advance has both in one load.
+// One 64-byte record per token (DevTables::tok_rec): its bytes with their length, so that the
+// advance has both in one load, and its lexemes from the first byte on with none pending,
+// the row-independent part of lexing, done once.  (One load of two bytes per lane: with the
+// lexemes in a table of their own, their load came 440 cycles behind the bytes'.)
 std::vector<uint8_t> token_records(const psc::Tables& t) {
-    std::vector<uint8_t> out((size_t)t.V * 32, 0);
+    std::vector<uint8_t> out((size_t)t.V * 64, 0);
     for (int v = 0; v < t.V; v++) {
-        int64_t lo = t.vocab_off[v], n = t.vocab_off[v + 1] - lo;
-        if (n > 0) std::memcpy(out.data() + (size_t)v * 32, t.vocab_bytes.data() + lo, (size_t)std::min<int64_t>(n, 31));
-        out[(size_t)v * 32 + 31] = n > 31 ? 255 : (uint8_t)n;
-    }
-    return out;
-}
-
-// Every token's lexemes from its first byte on with none pending ([V][16], see DevTables:
-// tok_lex): the row-independent part of lexing, done once.
-std::vector<uint16_t> token_lexemes(const psc::Tables& t) {
-    std::vector<uint16_t> out((size_t)t.V * 16, 0);
-    for (int v = 0; v < t.V; v++) {
-        uint16_t* w = out.data() + (size_t)v * 16;
-        const int64_t lo = t.vocab_off[v], hi = t.vocab_off[v + 1];
+        uint8_t* rec = out.data() + (size_t)v * 64;
+        const int64_t lo = t.vocab_off[v], hi = t.vocab_off[v + 1], len = hi - lo;
+        if (len > 0) std::memcpy(rec, t.vocab_bytes.data() + lo, (size_t)std::min<int64_t>(len, 31));
+        rec[31] = len > 31 ? 255 : (uint8_t)len;
+        uint16_t w[16] = {};
         int q = t.q0, n = 0;
-        w[0] = hi - lo > 31 ? TOK_LEX_LONG : 0;
+        w[0] = len > 31 ? TOK_LEX_LONG : 0;
         for (int64_t i = lo; i < hi && w[0] == 0; i++) {
             const int c = t.vocab_bytes[i];
             int nx = t.lex_trans[(size_t)q * 256 + c];
@@ -2357,6 +2347,7 @@ std::vector<uint16_t> token_lexemes(const psc::Tables& t) {
         }
         if (w[0] == 0) w[0] = (uint16_t)n;
         w[1] = (uint16_t)std::max(q, 0);
+        std::memcpy(rec + 32, w, sizeof w);
     }
     return out;
 }
@@ -2421,8 +2412,7 @@ psc_status upload_tables(std::unique_ptr<psc_handle>& h, int tables) {
         (s = upload(h.get(), dfa_mask, &d.dfa_mask)) || (s = upload(h.get(), t.mask_chunks, &d.mchunks)) ||
         (s = upload(h.get(), t.mask_rows, &d.mrows)) ||
         (s = upload(h.get(), t.vocab_bytes, &d.vocab, 16)) || (s = upload(h.get(), t.vocab_off, &d.vocab_off)) ||
-        (s = upload(h.get(), token_records(t), &d.tok32)) ||
-        (s = upload(h.get(), token_lexemes(t), &d.tok_lex))) {
+        (s = upload(h.get(), token_records(t), &d.tok_rec))) {
         for (int i = 0; i < h->n_blocks; i++) cudaFree(h->blocks[i]);
         return s;
     }
