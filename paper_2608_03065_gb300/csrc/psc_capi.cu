@@ -108,6 +108,7 @@ struct DevStates {
     unsigned long long* best;   // per-row greedy-choice key (nullable)
     int32_t* rmemo;             // [B][cap] bottom-up classifier block after each stack prefix (nullable)
     int32_t* fault;             // bounded in-kernel waits on these states that gave up (nullable)
+    int32_t* done;              // [B] warps of the row through k_mask_rows_ahead (zero between calls)
 };
 
 }  // namespace
@@ -1569,10 +1570,14 @@ __global__ void __launch_bounds__(256, ANY ? 4 : 5) k_mask_rows(T* logits, int64
 // The same for small batches, a warp per chunk: there the chain of loads (mask id, chunk
 // id, mask word, logits) is what takes the time, so all the chunk's pieces are read while
 // the mask word arrives, whatever the mask (one row of 151,936 f32 tokens: 8.9 us per
-// decode step instead of 10.3; one of 262,144 bf16 tokens 7.3 instead of 7.7).
+// decode step instead of 10.3; one of 262,144 bf16 tokens 7.3 instead of 7.7).  With tokens,
+// the last warp of a row (done: warps of the row that are through, zero between calls)
+// writes the row's choice instead of a kernel after this one: psc_fill_apply_argmax of 8 x
+// 512 f32 called from Python 7.1 -> 5.5 us.  Not at large batches: every warp would wait for its
+// own stores before it counts.
 template <typename T, bool GREEDY, bool TABLE, bool ANY>
 __global__ void __launch_bounds__(256) k_mask_rows_ahead(T* logits, int64_t stride, MaskSrc M, int B, int V, int cpv,
-                                                         unsigned long long* __restrict__ best_key) {
+                                                         unsigned long long* best_key, int32_t* tokens, int32_t* done) {
     __shared__ uint4 s_lut[sizeof(T) == 2 ? 256 : 1];
     if (sizeof(T) == 2) build_allow_lut<T>(s_lut);
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
@@ -1591,8 +1596,23 @@ __global__ void __launch_bounds__(256) k_mask_rows_ahead(T* logits, int64_t stri
     Best best;
     mask_chunk<T, GREEDY>(R, j, view_word(cur, before, R.a, lane), lane, s_lut, &ahead, best);
     if (GREEDY) {
-        const unsigned long long key = warp_max_key(best_key_of(best));
-        if (lane == 0 && key) atomicMax(best_key + b, key);
+        unsigned long long key = warp_max_key(best_key_of(best));
+        if (lane != 0) return;
+        const int n = R.chunks();
+        if (!tokens || n > 1) {
+            if (key) atomicMax(best_key + b, key);
+            if (!tokens) return;
+            __threadfence();   // the key before the count
+            if (atomicAdd(done + b, 1) != n - 1) return;
+            __threadfence();
+            key = atomicExch(best_key + b, 0ull);
+            done[b] = 0;
+        } else {   // the row's only warp
+            const unsigned long long kept = __ldcg(best_key + b);   // of a masking pass nothing consumed
+            key = kept > key ? kept : key;
+            if (kept) best_key[b] = 0ull;
+        }
+        tokens[b] = key ? (int32_t)(~(uint32_t)key) : -1;
     }
 }
 
@@ -1905,36 +1925,41 @@ constexpr long AHEAD_CHUNKS_BF16 = 4096, AHEAD_CHUNKS_F32 = 8192, SPAN4_CHUNKS =
 
 template <bool GREEDY, bool TABLE, typename T>
 psc_status launch_rows(T* logits, int64_t stride, const MaskSrc& M, int B, int V, int lead, unsigned long long* best,
-                       cudaStream_t cs) {
+                       int32_t** tokens, int32_t* done, cudaStream_t cs) {
     const int cpv = (lead + V + 1023) / 1024;
     const long chunks = (long)B * cpv;
     const bool any = lead != 0 || V % 1024 != 0;
-    if (chunks <= (sizeof(T) == 2 ? AHEAD_CHUNKS_BF16 : AHEAD_CHUNKS_F32))
+    if (chunks <= (sizeof(T) == 2 ? AHEAD_CHUNKS_BF16 : AHEAD_CHUNKS_F32)) {
+        int32_t* out = tokens ? *tokens : nullptr;
+        if (tokens) *tokens = nullptr;
         return launch_pdl(any ? k_mask_rows_ahead<T, GREEDY, TABLE, true> : k_mask_rows_ahead<T, GREEDY, TABLE, false>,
                           dim3((unsigned)((chunks + 7) / 8)), dim3(256), 0, cs, "k_mask_rows_ahead", logits, stride, M, B,
-                          V, cpv, best);
+                          V, cpv, best, out, done);
+    }
     const int span = std::min(sizeof(T) == 2 && any && chunks > SPAN4_CHUNKS ? 4 : 2, cpv);
     dim3 grid((unsigned)(((long)B * ((cpv + span - 1) / span) + 7) / 8));
     return launch_pdl(any ? k_mask_rows<T, GREEDY, TABLE, true> : k_mask_rows<T, GREEDY, TABLE, false>, grid, dim3(256), 0,
                       cs, "k_mask_rows", logits, stride, M, B, V, cpv, span, best);
 }
 
+// tokens: where the greedy choices go, set to null when the launched kernel writes them
+// itself (else they stay as keys in best).
 template <bool GREEDY, bool TABLE>
 psc_status launch_mask(void* d_logits, psc_dtype dtype, int64_t stride, const MaskSrc& M, int B, int V,
-                       unsigned long long* best, cudaStream_t cs) {
+                       unsigned long long* best, int32_t** tokens, int32_t* done, cudaStream_t cs) {
     const int lead = row_lead(d_logits, dtype, stride, B);
-    if (dtype == PSC_F32) return launch_rows<GREEDY, TABLE>((uint32_t*)d_logits, stride, M, B, V, lead, best, cs);
-    return launch_rows<GREEDY, TABLE>((uint16_t*)d_logits, stride, M, B, V, lead, best, cs);
+    if (dtype == PSC_F32) return launch_rows<GREEDY, TABLE>((uint32_t*)d_logits, stride, M, B, V, lead, best, tokens, done, cs);
+    return launch_rows<GREEDY, TABLE>((uint16_t*)d_logits, stride, M, B, V, lead, best, tokens, done, cs);
 }
 
-// Masking + greedy choice; leaves each row's key in st->d.best.
+// Masking + greedy choice; leaves each row's key in st->d.best (tokens: see launch_mask).
 psc_status launch_fused(const psc_handle* h, const psc_states* st, void* d_logits, psc_dtype dtype, int64_t row_stride,
-                        int V, uint32_t* d_bitmask_out, cudaStream_t cs) {
+                        int V, uint32_t* d_bitmask_out, cudaStream_t cs, int32_t** tokens = nullptr) {
     int B = st->d.B;
     psc_status s = ensure_mid(h, st, cs);
     if (s != PSC_OK) return s;
     MaskSrc M{nullptr, h->d.mchunks, h->d.mrows, st->d.mid, h->d.W, h->d.nch, d_bitmask_out};
-    s = launch_mask<true, true>(d_logits, dtype, row_stride, M, B, V, st->d.best, cs);
+    s = launch_mask<true, true>(d_logits, dtype, row_stride, M, B, V, st->d.best, tokens, st->d.done, cs);
     const_cast<psc_states*>(st)->after_mask = s == PSC_OK;
     return s;
 }
@@ -2628,7 +2653,7 @@ psc_status psc_state_init(const psc_handle* h, int32_t B, int32_t cap, void* str
                  o_stack = take(sizeof(uint16_t) * (size_t)B * cap),
                  o_memo = take(h->d.bu ? sizeof(int32_t) * (size_t)B * cap : 0);
     st->copy_bytes = off;
-    const size_t o_fault = take(sizeof(int32_t));
+    const size_t o_fault = take(sizeof(int32_t)), o_done = take(sizeof(int32_t) * (size_t)B);
     uint8_t* base = nullptr;
     s = cuda_check(cudaMalloc(&base, off), "cudaMalloc(states)");
     if (s != PSC_OK) return s;
@@ -2641,8 +2666,9 @@ psc_status psc_state_init(const psc_handle* h, int32_t B, int32_t cap, void* str
     d.stack = (uint16_t*)(base + o_stack);
     d.rmemo = h->d.bu ? (int32_t*)(base + o_memo) : nullptr;
     d.fault = (int32_t*)(base + o_fault);
+    d.done = (int32_t*)(base + o_done);
     cudaStream_t cs = (cudaStream_t)stream;
-    s = cuda_check(cudaMemsetAsync(d.fault, 0, sizeof(int32_t), cs), "cudaMemsetAsync(fault)");
+    s = cuda_check(cudaMemsetAsync(d.fault, 0, off - o_fault, cs), "cudaMemsetAsync(fault)");
     if (s == PSC_OK) {
         s = launch_pdl(k_state_init, dim3((B + 255) / 256), dim3(256), 0, cs, "k_state_init", d, h->d.q0, h->mid0,
                        (const int32_t*)nullptr, B);
@@ -2726,7 +2752,7 @@ psc_status psc_apply_mask(void* d_logits, psc_dtype dtype, int64_t row_stride, c
         return fail_with(PSC_ERR_ARG, "psc_apply_mask: bad arguments");
     if (B == 0) return PSC_OK;
     MaskSrc M{d_bitmask, nullptr, nullptr, nullptr, (V + 31) / 32, 0, nullptr};
-    return launch_mask<false, false>(d_logits, dtype, row_stride, M, B, V, nullptr, (cudaStream_t)stream);
+    return launch_mask<false, false>(d_logits, dtype, row_stride, M, B, V, nullptr, nullptr, nullptr, (cudaStream_t)stream);
 }
 
 psc_status psc_fill_apply(const psc_handle* h, const psc_states* st, int32_t B, void* d_logits, psc_dtype dtype,
@@ -2739,7 +2765,7 @@ psc_status psc_fill_apply(const psc_handle* h, const psc_states* st, int32_t B, 
     cudaStream_t cs = (cudaStream_t)stream;
     if ((s = ensure_mid(h, st, cs)) != PSC_OK) return s;
     MaskSrc M{nullptr, h->d.mchunks, h->d.mrows, st->d.mid, h->d.W, h->d.nch, d_bitmask_out};
-    return launch_mask<false, true>(d_logits, dtype, row_stride, M, B, V, nullptr, cs);
+    return launch_mask<false, true>(d_logits, dtype, row_stride, M, B, V, nullptr, nullptr, nullptr, cs);
 }
 
 psc_status psc_argmax_masked(const psc_handle* h, const psc_states* st, int32_t B, const void* d_logits,
@@ -2765,9 +2791,11 @@ psc_status psc_fill_apply_argmax(const psc_handle* h, const psc_states* st, int3
         (dtype != PSC_F32 && dtype != PSC_BF16))
         return fail_with(PSC_ERR_ARG, "psc_fill_apply_argmax: bad arguments");
     cudaStream_t cs = (cudaStream_t)stream;
-    if ((s = launch_fused(h, st, d_logits, dtype, row_stride, V, d_bitmask_out, cs)) != PSC_OK) return s;
+    int32_t* tokens = d_tokens;
+    if ((s = launch_fused(h, st, d_logits, dtype, row_stride, V, d_bitmask_out, cs, &tokens)) != PSC_OK) return s;
     const_cast<psc_states*>(st)->after_mask = false;
     const_cast<psc_states*>(st)->keys = false;
+    if (!tokens) return PSC_OK;
     return launch_pdl(k_finalize_tokens, dim3((unsigned)((B + 255) / 256)), dim3(256), 0, cs, "k_finalize_tokens",
                       st->d.best, B, d_tokens);
 }
@@ -2950,7 +2978,7 @@ psc_status psc_fill_apply_noalloc(const psc_handle* h, const int32_t* d_q, const
     cudaStream_t cs = (cudaStream_t)stream;
     if ((s = launch_classify(h->d, S, cs)) != PSC_OK) return s;
     MaskSrc M{nullptr, h->d.mchunks, h->d.mrows, mid, h->d.W, h->d.nch, d_bitmask_out};
-    return launch_mask<false, true>(d_logits, dtype, row_stride, M, B, V, nullptr, cs);
+    return launch_mask<false, true>(d_logits, dtype, row_stride, M, B, V, nullptr, nullptr, nullptr, cs);
 }
 
 psc_status psc_save(const psc_handle* h, const char* path) {
