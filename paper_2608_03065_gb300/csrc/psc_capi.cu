@@ -472,22 +472,24 @@ __device__ __forceinline__ unsigned long long best_key_of(const Best& b) {
     return b.col >= 0 ? make_key(f32_order(__float_as_uint(b.val)), b.col) : 0ull;
 }
 
-// Allowed-position masks of one 16-byte piece, indexed by its mask bits:
-// bf16 (8 bits -> 0xFFFF per allowed half of the 4 words), f32 (4 bits ->
-// 0xFFFFFFFF per allowed word).  Built in shared memory by every CTA.
-template <typename T>
+// Allowed-position masks of a 16-byte piece of bf16, indexed by its 8 mask bits: 0xFFFF per
+// allowed half of the 4 words.
 __device__ __forceinline__ void build_allow_lut(uint4* lut) {
-    constexpr int N = sizeof(T) == 2 ? 256 : 16;
-    for (int i = threadIdx.x; i < N; i += blockDim.x) {
+    for (int i = threadIdx.x; i < 256; i += blockDim.x) {
         uint32_t w[4];
-        for (int k = 0; k < 4; k++) {
-            if (sizeof(T) == 2)
-                w[k] = (((i >> (2 * k)) & 1) ? 0x0000FFFFu : 0u) | (((i >> (2 * k + 1)) & 1) ? 0xFFFF0000u : 0u);
-            else
-                w[k] = ((i >> k) & 1) ? 0xFFFFFFFFu : 0u;
-        }
+        for (int k = 0; k < 4; k++)
+            w[k] = (((i >> (2 * k)) & 1) ? 0x0000FFFFu : 0u) | (((i >> (2 * k + 1)) & 1) ? 0xFFFF0000u : 0u);
         lut[i] = make_uint4(w[0], w[1], w[2], w[3]);
     }
+}
+
+// Byte permutation of x (PTX prmt): nibble k of sel picks byte k; a nibble with its top bit
+// set replicates that byte's sign bit instead.
+template <uint32_t SEL>
+__device__ __forceinline__ uint32_t prmt(uint32_t x) {
+    uint32_t d;
+    asm("prmt.b32 %0, %1, %1, %2;" : "=r"(d) : "r"(x), "n"(SEL));
+    return d;
 }
 
 __device__ __forceinline__ uint32_t sel_ninf(uint32_t w, uint32_t allow, uint32_t ninf) {
@@ -506,7 +508,6 @@ template <typename T, bool ANY = true>
 struct RowView {
     static constexpr int E = 16 / sizeof(T);         // elements per piece
     static constexpr int PIECES = 1024 / E / 32;     // pieces of a chunk per lane
-    static constexpr uint32_t FULLBITS = (1u << E) - 1u;
     T* org;
     int a, lo, hi, end;
     __device__ __forceinline__ RowView() {}
@@ -540,11 +541,23 @@ __device__ __forceinline__ uint32_t view_word(uint32_t cur, uint32_t before, int
     return __funnelshift_l(lane == 0 ? before : p, cur, a);
 }
 
-// Mask bits of piece k of this lane, from the chunk's view words.
+// The view word that holds the mask bits of piece k of this lane (and of its neighbour in the
+// same 32-byte sector), and those bits.
 template <typename T>
-__device__ __forceinline__ uint32_t piece_bits(uint32_t word, int k, int lane) {
-    constexpr int E = RowView<T>::E, PPW = 32 / E;   // pieces per mask word
-    return (__shfl_sync(FULL, word, k * (32 / PPW) + lane / PPW) >> ((lane % PPW) * E)) & RowView<T>::FULLBITS;
+__device__ __forceinline__ uint32_t piece_word(uint32_t word, int k, int lane) {
+    constexpr int PPW = 32 / RowView<T>::E;   // pieces per mask word
+    return __shfl_sync(FULL, word, k * (32 / PPW) + lane / PPW);
+}
+template <typename T>
+__device__ __forceinline__ uint32_t piece_bits(uint32_t pw, int lane) {
+    constexpr int E = RowView<T>::E, PPW = 32 / E;
+    return (pw >> ((lane % PPW) * E)) & ((1u << E) - 1u);
+}
+template <typename T>
+__device__ __forceinline__ bool sector_full(uint32_t pw, int lane) {
+    constexpr int E = RowView<T>::E, PPW = 32 / E;
+    constexpr uint32_t S = (1u << (2 * E)) - 1u;
+    return (~pw & (S << ((lane % PPW & ~1) * E))) == 0u;
 }
 
 template <typename T>
@@ -615,13 +628,24 @@ __device__ __forceinline__ void fold_quad(Best& best, const uint32_t (&bits)[4],
     }
 }
 
-// Allowed-position masks of a 16-byte piece: the shared-memory table of bf16 pieces, or
-// (f32) one comparison per element.
+// A piece with -inf where its mask bits are 0.  bf16: from the table of the 256 patterns in
+// shared memory when there is one, else four bits at a time are spread to the bytes' sign
+// bits by one multiplication and replicated over the halves.  (The masking pass with the
+// greedy choice takes the table: the masks' registers otherwise keep loads from being in
+// flight, 1024 rows x 262,144 153 us per step instead of 142, x 262,145 189 instead of 152;
+// without the choice the arithmetic is faster, its pass needs no table built: 64 x 128,256
+// 5.2 us instead of 5.5.)
 template <typename T>
 __device__ __forceinline__ uint4 mask_piece(const uint4& v, uint32_t bits, const uint4* lut) {
     constexpr uint32_t N = NegInf<T>::pair;
     if (sizeof(T) == 2) {
-        uint4 am = lut[bits];
+        uint4 am;
+        if (lut) {
+            am = lut[bits];
+        } else {
+            const uint32_t lo = (bits & 15u) * 0x10204080u, hi = (bits >> 4) * 0x10204080u;   // bit i -> bit 8 i + 7
+            am = make_uint4(prmt<0x9988u>(lo), prmt<0xBBAAu>(lo), prmt<0x9988u>(hi), prmt<0xBBAAu>(hi));
+        }
         return make_uint4(sel_ninf(v.x, am.x, N), sel_ninf(v.y, am.y, N), sel_ninf(v.z, am.z, N), sel_ninf(v.w, am.w, N));
     }
     return make_uint4(bits & 1u ? v.x : N, bits & 2u ? v.y : N, bits & 4u ? v.z : N, bits & 8u ? v.w : N);
@@ -647,10 +671,7 @@ constexpr int CHOOSE_CLUSTER = 8;
 template <typename T>
 __global__ void __launch_bounds__(256) k_choose(const T* logits, int64_t stride, DevTables D, const int32_t* mid, int V,
                                                 int csize, int32_t* tokens) {
-    __shared__ uint4 s_lut[sizeof(T) == 2 ? 256 : 1];
     __shared__ unsigned long long s_key[CHOOSE_CLUSTER * 8];
-    if (sizeof(T) == 2) build_allow_lut<T>(s_lut);
-    __syncthreads();
     const int b = blockIdx.x / csize, rank = blockIdx.x - b * csize;
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     // every CTA of the cluster has started before its shared memory is written to
@@ -676,7 +697,7 @@ __global__ void __launch_bounds__(256) k_choose(const T* logits, int64_t stride,
         if (__ballot_sync(FULL, w != 0u) == 0u) continue;
         uint32_t bits[RowView<T>::PIECES];
 #pragma unroll
-        for (int k = 0; k < RowView<T>::PIECES; k++) bits[k] = piece_bits<T>(w, k, lane);
+        for (int k = 0; k < RowView<T>::PIECES; k++) bits[k] = piece_bits<T>(piece_word<T>(w, k, lane), lane);
         const int x0 = (j << 10) + lane * RowView<T>::E;
         const bool edged = R.edge(j);
         if (edged) {
@@ -694,7 +715,7 @@ __global__ void __launch_bounds__(256) k_choose(const T* logits, int64_t stride,
                 v[k] = qb[k] ? *reinterpret_cast<const uint4*>(R.org + x0 + (h + k) * 32 * RowView<T>::E) : make_uint4(0u, 0u, 0u, 0u);
             }
 #pragma unroll
-            for (int k = 0; k < 4; k++) v[k] = mask_piece<T>(v[k], qb[k], s_lut);
+            for (int k = 0; k < 4; k++) v[k] = mask_piece<T>(v[k], qb[k], nullptr);
             fold_quad<T>(best, qb, v, x0 + h * 32 * RowView<T>::E - R.a);
         }
         if (edged) {
@@ -753,18 +774,28 @@ template <typename T, bool GREEDY, bool EDGED, bool ANY>
 __device__ __forceinline__ void mask_quad(const RowView<T, ANY>& R, int j, int h, uint32_t w, int lane, const uint4* lut,
                                           const ChunkAhead<T>* ahead, Best& best) {
     constexpr int E = RowView<T, ANY>::E;
-    constexpr uint32_t F = RowView<T, ANY>::FULLBITS, N = NegInf<T>::pair;
+    constexpr uint32_t N = NegInf<T>::pair;
     const int x0 = (j << 10) + (h * 32 + lane) * E;
     uint32_t bits[4];
     uint4 v[4];
     bool store[4];
 #pragma unroll
     for (int k = 0; k < 4; k++) {
-        bits[k] = piece_bits<T>(w, h + k, lane);
-        const bool in = !EDGED || R.whole(x0 + k * 32 * E);
-        if (!in) bits[k] = F;   // not this row's, or handled element by element: left as it is
-        store[k] = (bits[k] & __shfl_xor_sync(FULL, bits[k], 1)) != F && in;
-        if (!in) bits[k] = 0u;
+        const uint32_t pw = piece_word<T>(w, h + k, lane);
+        bits[k] = piece_bits<T>(pw, lane);
+        if (!EDGED && !(GREEDY && ANY)) {
+            store[k] = !sector_full<T>(pw, lane);
+        } else {
+            // a piece that is not this row's, or handled element by element, is left as it is
+            // (with the greedy choice the instance with row ends asks the neighbouring lane
+            // everywhere: with the other test its whole chunks took 196 us instead of 152 on
+            // 1024 rows x 262,145)
+            constexpr uint32_t F = (1u << E) - 1u;
+            const bool in = !EDGED || R.whole(x0 + k * 32 * E);
+            if (!in) bits[k] = F;
+            store[k] = (bits[k] & __shfl_xor_sync(FULL, bits[k], 1)) != F && in;
+            if (!in) bits[k] = 0u;
+        }
     }
 #pragma unroll
     for (int k = 0; k < 4; k++) {
@@ -1535,15 +1566,16 @@ __global__ void __launch_bounds__(ADV_WARPS * 32, 1)   // the staged tables leav
 template <typename T, bool GREEDY, bool TABLE, bool ANY>
 __global__ void __launch_bounds__(256, ANY ? 4 : 5) k_mask_rows(T* logits, int64_t stride, MaskSrc M, int B, int V, int cpv,
                                                    int span, unsigned long long* __restrict__ best_key) {
-    __shared__ uint4 s_lut[sizeof(T) == 2 ? 256 : 1];
-    if (sizeof(T) == 2) build_allow_lut<T>(s_lut);
+    constexpr bool TABLE_OF_MASKS = GREEDY && sizeof(T) == 2;
+    __shared__ uint4 s_lut[TABLE_OF_MASKS ? 256 : 1];
+    if (TABLE_OF_MASKS) build_allow_lut(s_lut);
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const unsigned c = blockIdx.x * 8u + warp;   // fewer than 2^32: a chunk takes 2 KiB of logits or a whole row
     const unsigned spr = (unsigned)(cpv + span - 1) / (unsigned)span;
     const int b = (int)(c / spr), j0 = (int)(c - (unsigned)b * spr) * span;
     grid_dep_wait();   // logits, mask ids and greedy keys come from earlier kernels
     grid_dep_launch();
-    __syncthreads();   // the allow-mask table
+    if (TABLE_OF_MASKS) __syncthreads();
     if (b >= B) return;
     const RowView<T, ANY> R(logits + (size_t)b * stride, V);
     const int j1 = min(j0 + span, R.chunks());
@@ -1557,7 +1589,8 @@ __global__ void __launch_bounds__(256, ANY ? 4 : 5) k_mask_rows(T* logits, int64
         uint32_t next = 0u;
         if (j + 1 < j1) next = M.template word<TABLE>(b, j + 1, lane, __shfl_sync(FULL, id, j + 1 - j0));
         if (M.copy_out && j * 32 + lane < M.W) M.copy_out[(size_t)b * M.W + j * 32 + lane] = cur;
-        mask_chunk<T, GREEDY>(R, j, view_word(cur, before, R.a, lane), lane, s_lut, (const ChunkAhead<T>*)nullptr, best);
+        mask_chunk<T, GREEDY>(R, j, view_word(cur, before, R.a, lane), lane, TABLE_OF_MASKS ? s_lut : nullptr,
+                              (const ChunkAhead<T>*)nullptr, best);
         if (ANY) before = __shfl_sync(FULL, cur, 31);
         cur = next;
     }
@@ -1578,14 +1611,15 @@ __global__ void __launch_bounds__(256, ANY ? 4 : 5) k_mask_rows(T* logits, int64
 template <typename T, bool GREEDY, bool TABLE, bool ANY>
 __global__ void __launch_bounds__(256) k_mask_rows_ahead(T* logits, int64_t stride, MaskSrc M, int B, int V, int cpv,
                                                          unsigned long long* best_key, int32_t* tokens, int32_t* done) {
-    __shared__ uint4 s_lut[sizeof(T) == 2 ? 256 : 1];
-    if (sizeof(T) == 2) build_allow_lut<T>(s_lut);
+    constexpr bool TABLE_OF_MASKS = GREEDY && sizeof(T) == 2;
+    __shared__ uint4 s_lut[TABLE_OF_MASKS ? 256 : 1];
+    if (TABLE_OF_MASKS) build_allow_lut(s_lut);
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const unsigned c = blockIdx.x * 8u + warp;
     const int b = (int)(c / (unsigned)cpv), j = (int)(c - (unsigned)b * (unsigned)cpv);
     grid_dep_wait();
     grid_dep_launch();
-    __syncthreads();   // the allow-mask table
+    if (TABLE_OF_MASKS) __syncthreads();
     if (b >= B) return;
     const RowView<T, ANY> R(logits + (size_t)b * stride, V);
     if (j >= R.chunks()) return;
@@ -1594,7 +1628,8 @@ __global__ void __launch_bounds__(256) k_mask_rows_ahead(T* logits, int64_t stri
     const uint32_t before = ANY ? M.template word_before<TABLE>(b, j) : 0u;
     if (M.copy_out && j * 32 + lane < M.W) M.copy_out[(size_t)b * M.W + j * 32 + lane] = cur;
     Best best;
-    mask_chunk<T, GREEDY>(R, j, view_word(cur, before, R.a, lane), lane, s_lut, &ahead, best);
+    mask_chunk<T, GREEDY>(R, j, view_word(cur, before, R.a, lane), lane, TABLE_OF_MASKS ? s_lut : nullptr,
+                          &ahead, best);
     if (GREEDY) {
         unsigned long long key = warp_max_key(best_key_of(best));
         if (lane != 0) return;
@@ -1631,7 +1666,6 @@ __global__ void __launch_bounds__(ROW_WARPS * 32, 2)   // at most 64 registers
     k_decode_row(uint16_t* logits, int64_t stride, MaskSrc M, DevTables T, DevStates S, int V, int csize,
                  int32_t* tokens_out, int32_t* status_out) {
     extern __shared__ uint4 smem4[];
-    __shared__ uint4 s_lut[256];
     __shared__ unsigned long long s_key[ROW_CLUSTER * ROW_WARPS];
     __shared__ __align__(8) uint64_t s_bar[2];   // the staged tables, the keys
     __shared__ uint16_t lexcls[32];
@@ -1646,7 +1680,6 @@ __global__ void __launch_bounds__(ROW_WARPS * 32, 2)   // at most 64 registers
                      : "memory");
         stage_tables(T, smem_addr(sm), bar_tables);
     }
-    build_allow_lut<uint16_t>(s_lut);
     __syncthreads();
     // the first CTA has started and its mbarriers are set up once every CTA has passed here
     asm volatile("barrier.cluster.arrive.release.aligned;\nbarrier.cluster.wait.acquire.aligned;" ::: "memory");
@@ -1663,7 +1696,7 @@ __global__ void __launch_bounds__(ROW_WARPS * 32, 2)   // at most 64 registers
         const uint32_t cur = M.template word<true>(b, j, lane, M.template locate<true>(b, j, 0));
         const uint32_t before = ANY ? M.template word_before<true>(b, j) : 0u;
         if (M.copy_out && j * 32 + lane < M.W) M.copy_out[(size_t)b * M.W + j * 32 + lane] = cur;
-        mask_chunk<uint16_t, true>(R, j, view_word(cur, before, R.a, lane), lane, s_lut, &ahead, best);
+        mask_chunk<uint16_t, true>(R, j, view_word(cur, before, R.a, lane), lane, nullptr, &ahead, best);
     }
     if (advances) r.load_window();
     const unsigned long long key = warp_max_key(best_key_of(best));
