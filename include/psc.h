@@ -333,26 +333,14 @@ psc_status psc_host_advance(const psc_handle* h, int32_t* q, uint16_t* h_stack, 
  *
  * It does exactly what psc_fill_apply does, but the parser configurations
  * come from caller-owned device arrays instead of a psc_states object, and the
- * per-row mask ids it needs between the classifier walk and the masking pass
- * live in one library-owned scratch array of PSC_NOALLOC_MAX_ROWS int32 that
- * is part of the loaded module (a file-scope __device__ array, 64 KiB, held by
- * every GPU that loads the library until the process exits).  Nothing is
- * allocated or freed by the call.
+ * rows are classified in the masking pass itself: nothing is kept between the
+ * two, and nothing is allocated or freed by the call.
  *   d_q, d_depth, d_status : device int32 [B] (lexer state, stack depth, row status)
  *   d_stack                : device uint16 [B][cap], bottom first (the layout psc_states_download returns);
  *                            a row whose lexer state, depth or stack symbols are out of range gets
  *                            the empty mask (its logits all -inf)
  *   other arguments        : as for psc_fill_apply
- * Errors: PSC_ERR_LIMIT when B > PSC_NOALLOC_MAX_ROWS; PSC_ERR_ARG for bad arguments.
- * The first call on a device looks up the scratch array's device address
- * (cudaGetSymbolAddress) with that device current; make that first call
- * before any stream capture.  The address is kept for the life of the
- * process: it does not survive cudaDeviceReset (which unloads the module), so
- * do not call this entry point after resetting the device.  Every call shares the same scratch array, which
- * keeps the last call's contents (each call writes every entry it reads, so
- * nothing needs clearing); calls that overlap on the GPU (different streams,
- * or host threads racing on one device) race on it and must be serialised by
- * the caller. */
+ * Errors: PSC_ERR_LIMIT when B > PSC_NOALLOC_MAX_ROWS; PSC_ERR_ARG for bad arguments. */
 #define PSC_NOALLOC_MAX_ROWS 16384
 psc_status psc_fill_apply_noalloc(const psc_handle* h, const int32_t* d_q, const int32_t* d_depth,
                                   const int32_t* d_status, const uint16_t* d_stack, int32_t cap, int32_t B,

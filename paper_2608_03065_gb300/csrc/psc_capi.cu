@@ -31,7 +31,6 @@
 #include <cstring>
 #include <map>
 #include <memory>
-#include <mutex>
 #include <new>
 #include <string>
 
@@ -305,7 +304,11 @@ struct MaskSrc {
     // lane l: what locates chunk j + l of row b (its id in the device mask table)
     template <bool TABLE>
     __device__ __forceinline__ uint32_t locate(int b, int j, int lane) const {
-        return TABLE ? __ldg(rows + (size_t)__ldcg(mid + b) * nch + min(j + lane, nch - 1)) : 0u;
+        return TABLE ? locate_in(__ldcg(mid + b), j, lane) : 0u;
+    }
+    // the same for the row's mask id m
+    __device__ __forceinline__ uint32_t locate_in(int m, int j, int lane) const {
+        return __ldg(rows + (size_t)m * nch + min(j + lane, nch - 1));
     }
     // word `lane` of chunk j of row b, id: what locates that chunk (0 past W)
     template <bool TABLE>
@@ -1600,6 +1603,45 @@ __global__ void __launch_bounds__(256, ANY ? 4 : 5) k_mask_rows(T* logits, int64
     }
 }
 
+// Masking of rows whose mask ids nobody has (psc_fill_apply_noalloc): a CTA takes 8 x span
+// neighbouring chunks of one row, its first warp classifies the row (every CTA of the row
+// does: the walk's few loads hit L2), and the masking is that of k_mask_rows without the
+// choice.  Classifying all rows in a kernel before the masking made every row wait for the
+// deepest stack: one row x 262,144 5.5 us, here 4.8; 256 rows 39.7, here 36.6; 64 rows x
+// 128,256 of the Java-sized grammar 11.7, here 9.6.
+template <typename T, bool ANY>
+__global__ void __launch_bounds__(256, ANY ? 4 : 5) k_walk_mask_rows(T* logits, int64_t stride, MaskSrc M, DevTables D,
+                                                                     DevStates S, int V, int groups, int span) {
+    __shared__ int s_mid;
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int b = blockIdx.x / groups, j0 = ((blockIdx.x - b * groups) * 8 + warp) * span;
+    grid_dep_wait();   // logits and rows come from earlier kernels
+    grid_dep_launch();
+    if (warp == 0) {
+        const int m = warp_classify(D, S, b, lane);
+        if (lane == 0) s_mid = m;
+    }
+    __syncthreads();
+    const int m = s_mid;
+    const RowView<T, ANY> R(logits + (size_t)b * stride, V);
+    const int j1 = min(j0 + span, R.chunks());
+    if (j0 >= j1) return;
+    const uint32_t id = M.locate_in(m, j0, lane);
+    uint32_t cur = M.template word<true>(b, j0, lane, __shfl_sync(FULL, id, 0));
+    uint32_t before = 0u;
+    if (ANY && j0 > 0) before = M.template word<true>(b, j0 - 1, 31, M.locate_in(m, j0 - 1, 0));
+    Best best;
+#pragma unroll 1
+    for (int j = j0; j < j1; j++) {
+        uint32_t next = 0u;
+        if (j + 1 < j1) next = M.template word<true>(b, j + 1, lane, __shfl_sync(FULL, id, j + 1 - j0));
+        if (M.copy_out && j * 32 + lane < M.W) M.copy_out[(size_t)b * M.W + j * 32 + lane] = cur;
+        mask_chunk<T, false>(R, j, view_word(cur, before, R.a, lane), lane, nullptr, (const ChunkAhead<T>*)nullptr, best);
+        if (ANY) before = __shfl_sync(FULL, cur, 31);
+        cur = next;
+    }
+}
+
 // The same for small batches, a warp per chunk: there the chain of loads (mask id, chunk
 // id, mask word, logits) is what takes the time, so all the chunk's pieces are read while
 // the mask word arrives, whatever the mask (one row of 151,936 f32 tokens: 8.9 us per
@@ -1985,6 +2027,19 @@ psc_status launch_mask(void* d_logits, psc_dtype dtype, int64_t stride, const Ma
     return launch_rows<GREEDY, TABLE>((uint16_t*)d_logits, stride, M, B, V, lead, best, tokens, done, cs);
 }
 
+// One chunk per warp at small batches (more warps for the latency), up to four at large ones
+// (fewer CTAs that walk a row's stack): 64 rows x 262,144 14.7 us with two chunks, 15.4 with
+// one; 1024 rows 126 with four, 132 with two, 152 with one; 1024 x 128,256 60 / 69 / 92.
+template <typename T>
+psc_status launch_walk_rows(T* logits, psc_dtype dtype, int64_t stride, const MaskSrc& M, const DevTables& D,
+                            const DevStates& S, int V, cudaStream_t cs) {
+    const int lead = row_lead(logits, dtype, stride, S.B), cpv = (lead + V + 1023) / 1024;
+    const int span = (long)S.B * cpv <= AHEAD_CHUNKS_BF16 ? 1 : (long)S.B * cpv <= 16384 ? 2 : 4, groups = (cpv + 8 * span - 1) / (8 * span);
+    return launch_pdl(lead != 0 || V % 1024 != 0 ? k_walk_mask_rows<T, true> : k_walk_mask_rows<T, false>,
+                      dim3((unsigned)((long)S.B * groups)), dim3(256), 0, cs, "k_walk_mask_rows", logits, stride, M, D, S,
+                      V, groups, span);
+}
+
 // Masking + greedy choice; leaves each row's key in st->d.best (tokens: see launch_mask).
 psc_status launch_fused(const psc_handle* h, const psc_states* st, void* d_logits, psc_dtype dtype, int64_t row_stride,
                         int V, uint32_t* d_bitmask_out, cudaStream_t cs, int32_t** tokens = nullptr) {
@@ -2349,29 +2404,6 @@ std::vector<uint8_t> build_advance_blob(const psc::Tables& t, DevTables& d, int 
     return blob;
 }
 
-}  // namespace
-
-// Scratch of psc_fill_apply_noalloc: per-row mask ids between the classifier
-// walk and the masking pass, in the module itself so the call allocates nothing.
-static __device__ __align__(256) int32_t g_noalloc_mid[PSC_NOALLOC_MAX_ROWS];
-
-namespace {
-std::mutex g_noalloc_mu;
-int32_t* g_noalloc_ptr[256] = {};
-
-// Device address of g_noalloc_mid on the current device (looked up once per device).
-psc_status noalloc_scratch(int device, int32_t** out) {
-    if (device < 0 || device >= 256) return fail_with(PSC_ERR_ARG, "psc_fill_apply_noalloc: bad device id");
-    std::lock_guard<std::mutex> lk(g_noalloc_mu);
-    if (!g_noalloc_ptr[device]) {
-        void* p = nullptr;
-        psc_status s = cuda_check(cudaGetSymbolAddress(&p, g_noalloc_mid), "cudaGetSymbolAddress(scratch)");
-        if (s != PSC_OK) return s;
-        g_noalloc_ptr[device] = static_cast<int32_t*>(p);
-    }
-    *out = g_noalloc_ptr[device];
-    return PSC_OK;
-}
 }  // namespace
 
 namespace {
@@ -3004,14 +3036,12 @@ psc_status psc_fill_apply_noalloc(const psc_handle* h, const int32_t* d_q, const
     if (B <= 0 || !d_q || !d_depth || !d_status || !d_stack || cap < 2 || !d_logits || V != h->d.V ||
         row_stride < V || (dtype != PSC_F32 && dtype != PSC_BF16))
         return fail_with(PSC_ERR_ARG, "psc_fill_apply_noalloc: bad arguments");
-    int32_t* mid = nullptr;
-    if ((s = noalloc_scratch(h->device, &mid)) != PSC_OK) return s;
     DevStates S{const_cast<int32_t*>(d_q), const_cast<int32_t*>(d_depth), const_cast<int32_t*>(d_status),
-                const_cast<uint16_t*>(d_stack), mid, B, cap};
+                const_cast<uint16_t*>(d_stack), nullptr, B, cap};
+    MaskSrc M{nullptr, h->d.mchunks, h->d.mrows, nullptr, h->d.W, h->d.nch, d_bitmask_out};
     cudaStream_t cs = (cudaStream_t)stream;
-    if ((s = launch_classify(h->d, S, cs)) != PSC_OK) return s;
-    MaskSrc M{nullptr, h->d.mchunks, h->d.mrows, mid, h->d.W, h->d.nch, d_bitmask_out};
-    return launch_mask<false, true>(d_logits, dtype, row_stride, M, B, V, nullptr, nullptr, nullptr, cs);
+    if (dtype == PSC_F32) return launch_walk_rows((uint32_t*)d_logits, dtype, row_stride, M, h->d, S, V, cs);
+    return launch_walk_rows((uint16_t*)d_logits, dtype, row_stride, M, h->d, S, V, cs);
 }
 
 psc_status psc_save(const psc_handle* h, const char* path) {

@@ -67,6 +67,12 @@ def batches(psc):
     return out
 
 
+def _arrays(psc, st):
+    """The batch's parser states as caller-held device arrays."""
+    d = psc.psc_states_download(st)
+    return [torch.from_numpy(a).cuda() for a in (d["q"], d["depth"], d["status"], d["stack"].view(np.int16))]
+
+
 def _raw(t):
     t = t.cpu()
     return t.view(torch.int16 if t.dtype == torch.bfloat16 else torch.int32).numpy()
@@ -115,7 +121,7 @@ def test_rows_of_any_layout(psc, batches, V, dtype):
         psc.psc_fill_mask(h, st, bm)
         forked = psc.psc_state_init(h, B, 16)
         psc.psc_state_copy(forked, st)
-        for call in ("fill_apply", "apply_mask", "fill_apply_argmax", "decode_step"):
+        for call in ("fill_apply", "apply_mask", "fill_apply_argmax", "decode_step", "noalloc"):
             dev = base.cuda()
             lg = dev.as_strided((B, V), (ld, 1), off)
             tok = torch.full((B,), -7, dtype=torch.int32, device="cuda")
@@ -127,6 +133,9 @@ def test_rows_of_any_layout(psc, batches, V, dtype):
                 psc.psc_argmax_masked(h, st, lg, tok)
             elif call == "apply_mask":
                 psc.psc_apply_mask(lg, bm, B, V)
+            elif call == "noalloc":
+                psc.psc_fill_apply_noalloc(h, *_arrays(psc, st), lg, out)
+                psc.psc_argmax_masked(h, st, lg, tok)
             elif call == "fill_apply_argmax":
                 psc.psc_fill_apply_argmax(h, st, lg, tok, out)
             else:
@@ -167,7 +176,9 @@ def test_large_batches_of_odd_rows(psc, batches, V, rows, dtype):
         psc.psc_fill_mask(h, st, bm)
         word = bm[:, torch.arange(V, device="cuda") // 32] >> (torch.arange(V, device="cuda") % 32)
         assert torch.equal((word & 1).bool(), allowed)
-        for call in ("fill_apply", "apply_mask", "fill_apply_argmax"):
+        for call in ("fill_apply", "apply_mask", "fill_apply_argmax", "noalloc"):
+            if call == "noalloc" and rows > psc.NOALLOC_MAX_ROWS:
+                continue
             base = torch.full((off + rows * V + 64,), SENTINEL, dtype=dtype, device="cuda")
             lg = base[off:off + rows * V].view(rows, V)
             lg.copy_(x)
@@ -178,6 +189,9 @@ def test_large_batches_of_odd_rows(psc, batches, V, rows, dtype):
                 psc.psc_argmax_masked(h, st, lg, tok)
             elif call == "apply_mask":
                 psc.psc_apply_mask(lg, bm, rows, V)
+            elif call == "noalloc":
+                psc.psc_fill_apply_noalloc(h, *_arrays(psc, st), lg, out)
+                psc.psc_argmax_masked(h, st, lg, tok)
             else:
                 psc.psc_fill_apply_argmax(h, st, lg, tok, out)
             assert torch.equal(lg.view(bits), want.view(bits)), (call, off)

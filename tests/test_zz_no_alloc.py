@@ -3,8 +3,7 @@
 Callers that cannot allocate device memory at the point of the call (inside a
 CUDA graph capture, under a framework allocator that owns all memory, or in a
 loop where an allocation could synchronise the device) pass their own state
-arrays; the per-row scratch lives in a fixed array inside the library.  This
-file checks, through the C ABI, that two calls in a row give bit-for-bit the
+arrays; the masking pass classifies the rows itself.  This file checks, through the C ABI, that two calls in a row give bit-for-bit the
 masked logits and bitmask of psc_fill_apply on the same states.  It is named
 to be collected last.
 """
