@@ -4,10 +4,11 @@ One step = one pass of the whole per-step path over the batch, psc_decode_step
 (called as its two halves, psc_decode_step_mask + psc_decode_step_advance, so
 that the masking kernel can be timed on its own; the same steps replayed from a
 CUDA graph are reported beside the timed region):
-  k_step_tma       apply every row's precomputed mask to the bf16 logits in
+  k_mask_rows      apply every row's precomputed mask to the bf16 logits in
                    place, write the packed bitmask [B][V/32] and pick the greedy
-                   token among the allowed ones, in one TMA-pipelined pass
-                   (k_step_warp, a warp per 1024-column chunk, at small batches)
+                   token among the allowed ones, in one pass, a warp per two
+                   1024-column chunks (small batches: k_decode_row, the whole
+                   step in one kernel, or k_mask_rows_ahead)
   k_advance_warp   lex + parse the chosen tokens on the device-resident stacks
                    and classify the new configurations (bottom-up classifier:
                    only the stack entries the step changed are re-read)
@@ -40,7 +41,7 @@ WORKLOAD = 5
 SEQ = 32          # decode steps per sequence of the workload
 METRIC = "masked decode steps/s and µs/step at batch×vocab; HBM GB/s vs GB300 peak"
 UNIT = "steps/s"
-PROFILE_FILE = os.path.join(ROOT, "profiles", "k_step_tma_c5_traffic.txt")
+PROFILE_FILE = os.path.join(ROOT, "profiles", "k_mask_rows_c5_traffic.txt")
 
 
 def measured_peaks():
@@ -679,10 +680,10 @@ def run_paths(args):
     """A small case for profiler captures of the plain mask paths on config 5's
     tables and prefix states (one 512 MiB logits buffer), each in an NVTX range:
     "fill_apply" (psc_fill_apply: masks applied from the current mask ids,
-    k_apply_rows), "fill_mask" (psc_fill_mask, k_fill), "apply_mask"
-    (psc_apply_mask from that bitmask, k_apply_rows), "classify_walk"
+    k_mask_rows), "fill_mask" (psc_fill_mask, k_fill), "apply_mask"
+    (psc_apply_mask from that bitmask, k_mask_rows), "classify_walk"
     (psc_fill_apply_noalloc on the same rows as plain arrays: every stack walked
-    from the top by k_classify, then k_apply_rows), "classify_bottom_up" (a
+    from the top by k_classify, then k_mask_rows), "classify_bottom_up" (a
     psc_advance with no tokens: every row classified again through its kept
     bottom-up states)."""
     import numpy as np
@@ -966,14 +967,14 @@ def main():
         "graph": {"value": whole_job_rate(world, K, graph_ms), "unit": UNIT, "ms_per_step": graph_ms / K,
                   "note": "the same K steps captured once in a CUDA graph and replayed"},
         "decode_step_us": step_avg_ms * 1000.0,
-        "k_step_tma_us": mask_avg_ms * 1000.0,
+        "mask_pass_us": mask_avg_ms * 1000.0,
         "roofline": {"bound": "hbm", "achieved": achieved, "peak": peak, "unit": "GB/s",
                      "frac": achieved / peak, "traffic": traffic,
                      # the same duration over the DRAM bytes ncu measured for one launch (the
                      # kernel skips bytes the formula counts: frac can pass 1, this cannot)
                      "dram_achieved": traffic / (mask_avg_ms / 1000.0) / 1e9 if traffic else None,
                      "dram_frac": traffic / (mask_avg_ms / 1000.0) / 1e9 / peak if traffic else None,
-                     "kernel": "k_step_tma (masking pass + greedy choice, CUDA events around each launch)",
+                     "kernel": "k_mask_rows (masking pass + greedy choice, CUDA events around each launch)",
                      "algorithmic_bytes": alg_bytes, "peak_kind": peak_kind},
         "e2e": {"value": e2e_value, "unit": UNIT, "h2d_bytes_per_step": B * V * 2,
                 "d2h_bytes_per_step": B * 4},

@@ -250,13 +250,13 @@ psc_status psc_fill_apply_argmax(const psc_handle* h, const psc_states* st, int3
                                  int32_t* d_tokens, void* stream);
 
 /* One whole decoding step on the device (Algorithm 2 steps 1-4 plus masking and
- * greedy sampling), in two kernels: the masking pass applies every row's mask
- * (step 4) to the logits in place, writes the optional bitmask copy and picks
- * the greedy token per row; the advance kernel then feeds that token to the
- * row's lexer and parser (steps 1-2) and classifies the new configuration
- * (step 3), so the next step's masking pass reads the mask ids directly.  The
- * masking pass classifies rows itself when the mask ids are not current (after
- * psc_state_init or psc_state_reset).
+ * greedy sampling).  The masking pass applies every row's mask (step 4) to the
+ * logits in place, writes the optional bitmask copy and picks the greedy token
+ * per row; the advance then feeds that token to the row's lexer and parser
+ * (steps 1-2) and classifies the new configuration (step 3), so the next step's
+ * masking pass reads the mask ids directly (psc_state_init and psc_state_reset
+ * leave them current too).  Large batches run the two as two kernels, small ones
+ * as one.
  *   d_tokens      : device int32 [B]; receives the chosen tokens (-1 = nothing allowed)
  *   d_row_status  : optional device int32 [B] statuses after the step
  * Other arguments as for psc_fill_apply_argmax.  Equivalent to

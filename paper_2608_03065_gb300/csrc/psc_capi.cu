@@ -2029,7 +2029,9 @@ psc_status launch_mask(void* d_logits, psc_dtype dtype, int64_t stride, const Ma
 
 // One chunk per warp at small batches (more warps for the latency), up to four at large ones
 // (fewer CTAs that walk a row's stack): 64 rows x 262,144 14.7 us with two chunks, 15.4 with
-// one; 1024 rows 126 with four, 132 with two, 152 with one; 1024 x 128,256 60 / 69 / 92.
+// one; 1024 rows 126 with four, 132 with two, 152 with one; 1024 x 128,256 60 / 69 / 92.  With
+// 1024 deep stacks of the C-like grammar over 262,144 tokens a kernel that classifies first is
+// 4 % faster (169.5 us against 176.7; 512 rows are level, 92), not enough to hold scratch for it.
 template <typename T>
 psc_status launch_walk_rows(T* logits, psc_dtype dtype, int64_t stride, const MaskSrc& M, const DevTables& D,
                             const DevStates& S, int V, cudaStream_t cs) {
